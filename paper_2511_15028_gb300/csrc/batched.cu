@@ -38,8 +38,9 @@ __device__ __forceinline__ unsigned long long take_unit(unsigned long long *work
 
 __device__ __forceinline__ void start_lane(const TraceArgs &a, Lane &L, Stack &st, unsigned long long rid, bool own) {
   L.rid = rid;
-  setup_ray(ldg4f(a.rays + 2 * rid), ldg4f(a.rays + 2 * rid + 1), L.r);
-  L.b = Best{__int_as_float(0x7f800000), 0.f, 0.f, SCION_PRIM_MISS};
+  const float4 o = ldg4f(a.rays + 2 * rid), d = ldg4f(a.rays + 2 * rid + 1);
+  setup_ray(o, d, L.r);
+  L.b = Best{d.w, 0.f, 0.f, SCION_PRIM_MISS};
   L.steps = 0;
   L.err = 0;
   L.found = false;
@@ -52,6 +53,7 @@ __device__ __forceinline__ void finish_lane(const TraceArgs &a, Lane &L) {
     atomicCAS(a.status, 0u, L.err);
     L.b = Best{__int_as_float(0x7f800000), 0.f, 0.f, SCION_PRIM_ERROR};
   }
+  if (L.b.id == SCION_PRIM_MISS) L.b.t = __int_as_float(0x7f800000);
   static_cast<uint4 *>(a.out)[L.rid] =
       make_uint4(__float_as_uint(L.b.t), __float_as_uint(L.b.u), __float_as_uint(L.b.v), L.b.id);
 }
@@ -65,21 +67,19 @@ __device__ __forceinline__ void finish_lane(const TraceArgs &a, Lane &L) {
 // call lives in local memory, and so would the stack pointer on every step.
 template <bool OWN, int W, int PREC, int SOA>
 __device__ __noinline__ unsigned long long run_scene(const BatchScene &S, unsigned long long base,
-                                                     unsigned long long *work, uint2 *smem_col,
+                                                     unsigned long long *work, uint2 *smem_base,
                                                      uint32_t smem_stack) {
   Stack st;
   StackTail<false> tail;
   st.attach(tail);
-  st.sh = smem_col;
-  st.stride = blockDim.x;
-  st.cap_sh = (int)smem_stack;
+  st.columns(smem_base, smem_stack);
   st.reset();
   const TraceArgs &a = S.a;
   const unsigned long long s_lo = S.begin, s_hi = S.begin + ((a.n + 31ull) & ~31ull);
   const uint32_t lane = threadIdx.x & 31u;
   Counts cnt;
   Lane L;
-  if (a.refill_min == 0) {
+  if (a.refill_min == 32) {
     // warp batches: every lane traces its ray of the unit to completion
     while (base >= s_lo && base < s_hi) {
       const unsigned long long rid = base - s_lo + lane;
@@ -161,7 +161,6 @@ __global__ void __launch_bounds__(kMaxThreadsPerBlock, kMinBlocksPerSm)
   const uint32_t cached = n_scenes < (uint32_t)kMaxSharedScenes ? n_scenes : (uint32_t)kMaxSharedScenes;
   for (uint32_t i = threadIdx.x; i < cached; i += blockDim.x) starts[i] = scenes[i].begin;
   __syncthreads();
-  uint2 *const col = smem + threadIdx.x;  // this thread's shared-memory stack column
   unsigned long long base = take_unit(work);
   while (base < total) {
     // last scene whose start <= base (binary search, warp-uniform)
@@ -174,14 +173,14 @@ __global__ void __launch_bounds__(kMaxThreadsPerBlock, kMinBlocksPerSm)
     }
     const BatchScene &S = scenes[lo];
     switch (S.family) {
-      case kFamilyBin: base = run_scene<true, 2, PREC_F32, LAYOUT_AOS>(S, base, work, col, smem_stack); break;
-      case kFamilyBinQ16: base = run_scene<true, 2, PREC_Q16, LAYOUT_AOS>(S, base, work, col, smem_stack); break;
-      case kFamilyW4F32: base = run_scene<false, 4, PREC_F32, LAYOUT_SOA>(S, base, work, col, smem_stack); break;
-      case kFamilyW4F16: base = run_scene<false, 4, PREC_F16, LAYOUT_SOA>(S, base, work, col, smem_stack); break;
-      case kFamilyW4U8: base = run_scene<false, 4, PREC_U8, LAYOUT_SOA>(S, base, work, col, smem_stack); break;
-      case kFamilyW8F16: base = run_scene<false, 8, PREC_F16, LAYOUT_SOA>(S, base, work, col, smem_stack); break;
-      case kFamilyW8U8: base = run_scene<false, 8, PREC_U8, LAYOUT_AOS>(S, base, work, col, smem_stack); break;
-      case kFamilyW8U8S: base = run_scene<false, 8, PREC_U8, LAYOUT_SOA>(S, base, work, col, smem_stack); break;
+      case kFamilyBin: base = run_scene<true, 2, PREC_F32, LAYOUT_AOS>(S, base, work, smem, smem_stack); break;
+      case kFamilyBinQ16: base = run_scene<true, 2, PREC_Q16, LAYOUT_AOS>(S, base, work, smem, smem_stack); break;
+      case kFamilyW4F32: base = run_scene<false, 4, PREC_F32, LAYOUT_SOA>(S, base, work, smem, smem_stack); break;
+      case kFamilyW4F16: base = run_scene<false, 4, PREC_F16, LAYOUT_SOA>(S, base, work, smem, smem_stack); break;
+      case kFamilyW4U8: base = run_scene<false, 4, PREC_U8, LAYOUT_SOA>(S, base, work, smem, smem_stack); break;
+      case kFamilyW8F16: base = run_scene<false, 8, PREC_F16, LAYOUT_SOA>(S, base, work, smem, smem_stack); break;
+      case kFamilyW8U8: base = run_scene<false, 8, PREC_U8, LAYOUT_AOS>(S, base, work, smem, smem_stack); break;
+      case kFamilyW8U8S: base = run_scene<false, 8, PREC_U8, LAYOUT_SOA>(S, base, work, smem, smem_stack); break;
       default: base = take_unit(work); break;  // batch creation admits only the families above
     }
   }

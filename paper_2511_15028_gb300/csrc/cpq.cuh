@@ -357,9 +357,7 @@ __device__ __forceinline__ void cpq_kernel_body(const TraceArgs &a) {
   Stack st;
   StackTail<false> tail;
   st.attach(tail);
-  st.sh = smem_stack + threadIdx.x;
-  st.stride = blockDim.x;
-  st.cap_sh = (int)a.smem_stack;
+  st.columns(smem_stack, a.smem_stack);
   st.reset();
   Counts cnt;
   uint32_t n_pts = 0;

@@ -91,6 +91,21 @@ def test_config1_every_layout_bit_exact(sc_mod, config1, kw):
     assert sc_mod.scion_get_status(bvh) == 0
 
 
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 1000, 2431, 2433, 4865, 9729, 16383])
+def test_small_launches(sc_mod, config1, n):
+    """Launches below and around the sizes at which a warp takes fewer than 32
+    rays at a time: every ray is traced once, in every fetch mode and for tiles
+    cut short by the block size."""
+    sc, rays, exp, occ = config1
+    for kw in (dict(), dict(width=4, box_layout="soa"), dict(width=8, box_prec="u8")):
+        bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
+        for p in (None, dict(rays_per_fetch=4), dict(raster_width=37), dict(threads_per_block=32, ctas_per_sm=1)):
+            for _ in range(2):  # the counters are ready for the next launch
+                assert_same_hits(gpu_closest(sc_mod, bvh, rays[:n], params=p), exp[:n], f"{kw} {p}")
+            assert np.array_equal(gpu_any(sc_mod, bvh, rays[:n], params=p), occ[:n]), f"{kw} {p}"
+        assert sc_mod.scion_get_status(bvh) == 0
+
+
 def test_closed_form_scenes_on_gpu(sc_mod, oracle_mod):
     tri = np.array([[0, 0, 0], [1, 0, 0], [0, 1, 0]], np.float32)
     quad = np.array([[0, 0, 0], [1, 0, 0], [1, 1, 0], [0, 0, 0], [1, 1, 0], [0, 1, 0]], np.float32)
