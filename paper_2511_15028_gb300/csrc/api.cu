@@ -228,11 +228,10 @@ void small_launch(TraceArgs &a, uint64_t resident_warps) {
 
 // Shared-memory stack bytes per entry, as StackFor (trace.cuh) chooses them:
 // (ref, entry distance), plus the exit distance for the shared-slab layout,
-// whose traversal carries intervals; the reference alone for any hit and for
-// the other own-box nodes.
+// whose traversal carries intervals; the reference alone for any hit.
 size_t stack_entry_bytes(const scion_bvh b, int query) {
   if (query == kQueryPoint) return sizeof(uint2);
-  if (b->own_box) return b->desc.box_prec == PREC_SLAB ? sizeof(uint2) + sizeof(float) : sizeof(uint32_t);
+  if (b->own_box && b->desc.box_prec == PREC_SLAB) return sizeof(uint2) + sizeof(float);
   return query == kQueryAny ? sizeof(uint32_t) : sizeof(uint2);
 }
 

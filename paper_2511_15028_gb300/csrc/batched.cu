@@ -36,7 +36,8 @@ __device__ __forceinline__ unsigned long long take_unit(unsigned long long *work
   return __shfl_sync(0xFFFFFFFFu, b, 0);
 }
 
-__device__ __forceinline__ void start_lane(const TraceArgs &a, Lane &L, Stack &st, unsigned long long rid, bool own) {
+template <bool OWN, int PREC, int SOA>
+__device__ __forceinline__ void start_lane(const TraceArgs &a, Lane &L, Stack &st, unsigned long long rid) {
   L.rid = rid;
   const float4 o = ldg4f(a.rays + 2 * rid), d = ldg4f(a.rays + 2 * rid + 1);
   setup_ray(o, d, L.r);
@@ -45,7 +46,7 @@ __device__ __forceinline__ void start_lane(const TraceArgs &a, Lane &L, Stack &s
   L.err = 0;
   L.found = false;
   st.reset();
-  L.cur = own ? (a.n_nodes > 0 ? 0u : kEmptyRef) : a.root_ref;
+  start_ray<OWN, PREC, SOA>(a, L);
 }
 
 __device__ __forceinline__ void finish_lane(const TraceArgs &a, Lane &L) {
@@ -84,7 +85,7 @@ __device__ __noinline__ unsigned long long run_scene(const BatchScene &S, unsign
     while (base >= s_lo && base < s_hi) {
       const unsigned long long rid = base - s_lo + lane;
       if (rid < a.n) {
-        start_lane(a, L, st, rid, OWN);
+        start_lane<OWN, PREC, SOA>(a, L, st, rid);
         while (L.cur != kEmptyRef) {
           if (++L.steps > a.max_steps) {
             L.err = kErrIter;
@@ -126,7 +127,7 @@ __device__ __noinline__ unsigned long long run_scene(const BatchScene &S, unsign
         if (!has_ray) {
           const unsigned long long rid = next + __popc(idle & below);
           if (rid < hi) {
-            start_lane(a, L, st, rid, OWN);
+            start_lane<OWN, PREC, SOA>(a, L, st, rid);
             has_ray = true;
           }
         }

@@ -256,61 +256,6 @@ __device__ __forceinline__ void cp_step_wide(const TraceArgs &a, CpLane &L, Stac
   L.cur = next != kEmptyRef ? next : cp_pop(L, st);
 }
 
-// own box of node x of an own-box layout (every codec), and its word
-template <int PREC, int SOA>
-__device__ __forceinline__ void own_node(const TraceArgs &a, uint32_t x, float (&lo)[3], float (&hi)[3],
-                                         uint32_t &count, uint32_t &field) {
-  if (PREC == PREC_F32) {
-    uint32_t ref, meta;
-    if (SOA) {
-      const uint2 *bp = reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(a.nodes) +
-                                                        (size_t)x * a.node_stride);
-      const uint2 b0 = __ldg(bp), b1 = __ldg(bp + 1), b2 = __ldg(bp + 2);
-      const uint2 rm = __ldg(a.nodes2 + x);
-      lo[0] = __uint_as_float(b0.x); lo[1] = __uint_as_float(b0.y); lo[2] = __uint_as_float(b1.x);
-      hi[0] = __uint_as_float(b1.y); hi[1] = __uint_as_float(b2.x); hi[2] = __uint_as_float(b2.y);
-      ref = rm.x; meta = rm.y;
-    } else {
-      uint4 q0, q1;
-      ldg8(a.nodes + 2 * (size_t)x, q0, q1);
-      lo[0] = __uint_as_float(q0.x); lo[1] = __uint_as_float(q0.y); lo[2] = __uint_as_float(q0.z);
-      hi[0] = __uint_as_float(q0.w); hi[1] = __uint_as_float(q1.x); hi[2] = __uint_as_float(q1.y);
-      ref = q1.z; meta = q1.w;
-    }
-    count = bin_meta_count(meta);
-    field = ref;
-    return;
-  }
-  const char *np = reinterpret_cast<const char *>(a.nodes) + (size_t)x * a.node_stride;
-  uint32_t w0, w1, w2, w3 = 0;
-  if (a.node_stride == 16) {
-    const uint4 v = ldg4(reinterpret_cast<const uint4 *>(np));
-    w0 = v.x; w1 = v.y; w2 = v.z; w3 = v.w;
-  } else {
-    const uint32_t *wp = reinterpret_cast<const uint32_t *>(np);
-    w0 = __ldg(wp); w1 = __ldg(wp + 1); w2 = __ldg(wp + 2);
-  }
-  uint32_t word;
-  if (PREC == PREC_Q16) {
-    word = SOA ? __ldg(reinterpret_cast<const uint32_t *>(a.nodes2) + x) : w3;
-    lo[0] = fmaf(u16lo_f(w0), a.frame[3], a.frame[0]);
-    lo[1] = fmaf(u16hi_f(w0), a.frame[4], a.frame[1]);
-    lo[2] = fmaf(u16lo_f(w1), a.frame[5], a.frame[2]);
-    hi[0] = fmaf(u16hi_f(w1), a.frame[3], a.frame[0]);
-    hi[1] = fmaf(u16lo_f(w2), a.frame[4], a.frame[1]);
-    hi[2] = fmaf(u16hi_f(w2), a.frame[5], a.frame[2]);
-  } else {
-    word = w2;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      lo[c] = __fmaf_rd(eq10_f(w0, c), a.frame[6 + c], a.frame[c]);
-      hi[c] = __fmaf_ru(-eq10_f(w1, c), a.frame[6 + c], a.frame[3 + c]);
-    }
-  }
-  count = qbin_count(word);
-  field = count > 0 ? qbin_first(word) : qbin_field(word);
-}
-
 // Own-box binary node: the entered node's box was bounded by its parent; a
 // leaf tests its triangles, an interior node bounds both children's boxes
 // (the paper's children sorting), enters the nearer and stacks the other.
@@ -318,9 +263,8 @@ template <int PREC, int SOA, int CREF, bool STATS>
 __device__ __forceinline__ void cp_step_bin(const TraceArgs &a, CpLane &L, Stack &st, Counts &cnt) {
   const uint32_t cur = L.cur;
   if (STATS) cnt.nodes++;
-  float lo[3], hi[3];
   uint32_t n, field;
-  own_node<PREC, SOA>(a, cur, lo, hi, n, field);
+  own_ref<PREC, SOA>(a, cur, n, field);
   if (n > 0) {
     cp_leaf<STATS>(a, L, field, n, cnt);
     L.cur = cp_pop(L, st);
