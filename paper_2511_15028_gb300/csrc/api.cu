@@ -180,8 +180,8 @@ void bvh_args(const scion_bvh b, TraceArgs &a) {
 constexpr size_t kSmemOptIn = 32 * 1024;
 
 // Closest point queries are refilled once this many lanes of a warp are idle
-// (1 M random points around 1.4 M triangles, bvh4 f32: 2, 4, 8, 16 lanes take
-// 3.66, 3.65, 3.68, 3.9 ms, whole batches of 32 5.9 ms).
+// (1 M random points around 1.4 M triangles, bvh4 f32: 3.65 ms at 4 lanes, 3.68
+// at 8; 5.90 ms in whole batches of 32).
 constexpr uint32_t kCpRefill = 4;
 
 // Query kinds of launch_trace.

@@ -11,14 +11,22 @@
 //
 // One thread per ray (grid-stride). The 3x3 solve runs in single precision
 // (Cramer's rule) followed by one step of iterative refinement whose residual
-// g - J^T lambda is formed in double precision from the exact columns of J;
-// the error after the step is of the order of the square of the first
-// solve's, so lambda comes out accurate to double-precision-solve level for
-// any system that is not extremely ill conditioned, with about 20 FP64
-// operations per ray instead of a hundred (FP64 is slow on this part). A
-// singular or non-finite single-precision solve falls back to the
-// double-precision solve. The nine vertex contributions are scattered with
-// FP32 atomicAdd.
+// g - J^T lambda is formed to twice single precision: the columns of J as
+// exact pairs of floats (TwoDiff, Knuth), products as exact pairs (one fma
+// each), summed with the rounding errors carried along (the compensated dot
+// product of Ogita, Rump and Oishi, 2005). The error after the step is of the
+// order of the square of the first solve's, so lambda comes out accurate to
+// the last bit or so of a float for any system that is not extremely ill
+// conditioned. FP64 has a small fraction of the FP32 rate here: with the
+// residual in doubles (about 45 FP64 operations a hit) that pipe was 81 % busy.
+// A singular or
+// non-finite single-precision solve, and gradients so small or large that the
+// pairs could underflow or overflow, take the double-precision solve.
+//
+// The nine vertex contributions are added with FP32 atomics, a vertex's three
+// as a pair and a single (row i of the float[n][3] array starts at 12 i bytes:
+// the 8-byte aligned pair is its first two elements when i is even, its last
+// two when it is odd).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -45,15 +53,48 @@ __device__ __forceinline__ void cross3f(const float *a, const float *b, float *c
   c[2] = fmaf(a[0], b[1], -a[1] * b[0]);
 }
 
+struct Pair {  // an unevaluated sum hi + lo
+  float hi, lo;
+};
+
+// x - y exactly (TwoDiff; no overflow)
+__device__ __forceinline__ Pair two_diff(float x, float y) {
+  const float d = __fsub_rn(x, y);
+  const float t = __fsub_rn(d, x);
+  return {d, __fsub_rn(__fsub_rn(x, __fsub_rn(d, t)), __fadd_rn(y, t))};
+}
+
+// acc -= a * m, the rounding errors of the product and of the sum going to err
+__device__ __forceinline__ void sub_product(float a, float m, float &acc, float &err) {
+  const float p = __fmul_rn(a, m), e = fmaf(a, m, -p);
+  const float s = __fsub_rn(acc, p);
+  const float t = __fsub_rn(s, acc);
+  err = __fadd_rn(err, __fsub_rn(__fsub_rn(__fsub_rn(acc, __fsub_rn(s, t)), __fadd_rn(p, t)), e));
+  acc = s;
+}
+
+// g - c . l to about twice single precision, c given in pairs
+__device__ __forceinline__ float residual(const Pair *c, const float *l, float g) {
+  float acc = g, err = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    sub_product(c[k].hi, l[k], acc, err);
+    err = fmaf(-c[k].lo, l[k], err);
+  }
+  return __fadd_rn(acc, err);
+}
+
 // lambda with J^T lambda = (gt, gu, gv), J = [c0 | c1 | c2]: single-precision
-// Cramer's rule, then one refinement step lambda += J^-T (g - J^T lambda)
-// with the residual in double precision. False when the single-precision
-// system is singular or the result is not finite.
-__device__ __forceinline__ bool solve_refined(const double *c0, const double *c1, const double *c2, float gt,
-                                              float gu, float gv, double *lam) {
-  const float f0[3] = {(float)c0[0], (float)c0[1], (float)c0[2]};
-  const float f1[3] = {(float)c1[0], (float)c1[1], (float)c1[2]};
-  const float f2[3] = {(float)c2[0], (float)c2[1], (float)c2[2]};
+// Cramer's rule, then one refinement step lambda += J^-T (g - J^T lambda).
+// False when the single-precision system is singular, the result is not
+// finite or the gradients leave the range of the pairs.
+__device__ __forceinline__ bool solve_refined(const Pair *c0, const Pair *c1, const Pair *c2, float gt, float gu,
+                                              float gv, float *lam) {
+  const float gmax = fmaxf(fmaxf(fabsf(gt), fabsf(gu)), fabsf(gv));
+  if (!(gmax == 0.0f || (gmax > 1e-28f && gmax < 1e28f))) return false;
+  const float f0[3] = {c0[0].hi, c0[1].hi, c0[2].hi};
+  const float f1[3] = {c1[0].hi, c1[1].hi, c1[2].hi};
+  const float f2[3] = {c2[0].hi, c2[1].hi, c2[2].hi};
   float x12[3], x20[3], x01[3];
   cross3f(f1, f2, x12);
   cross3f(f2, f0, x20);
@@ -63,73 +104,105 @@ __device__ __forceinline__ bool solve_refined(const double *c0, const double *c1
   const float inv = 1.0f / det;
   float l0[3];
   for (int k = 0; k < 3; ++k) l0[k] = fmaf(gt, x12[k], fmaf(gu, x20[k], gv * x01[k])) * inv;
-  // residual of the equations c_i . lambda = g_i, in double
-  const double r0 = (double)gt - (c0[0] * l0[0] + c0[1] * l0[1] + c0[2] * l0[2]);
-  const double r1 = (double)gu - (c1[0] * l0[0] + c1[1] * l0[1] + c1[2] * l0[2]);
-  const double r2 = (double)gv - (c2[0] * l0[0] + c2[1] * l0[1] + c2[2] * l0[2]);
-  const float s0 = (float)r0, s1 = (float)r1, s2 = (float)r2;
+  const float s0 = residual(c0, l0, gt), s1 = residual(c1, l0, gu), s2 = residual(c2, l0, gv);
   for (int k = 0; k < 3; ++k) {
-    lam[k] = (double)l0[k] + (double)(fmaf(s0, x12[k], fmaf(s1, x20[k], s2 * x01[k])) * inv);
+    lam[k] = l0[k] + fmaf(s0, x12[k], fmaf(s1, x20[k], s2 * x01[k])) * inv;
     if (!isfinite(lam[k])) return false;
   }
   return true;
 }
 
+// grad_verts[vid] += w * l. PAIRED: the array starts on an 8-byte boundary.
+template <bool PAIRED>
+__device__ __forceinline__ void add_vertex(float *grad_verts, uint32_t vid, float w, const float *l) {
+  float *g = grad_verts + 3 * (size_t)vid;
+  const float x = w * l[0], y = w * l[1], z = w * l[2];
+  if (!PAIRED) {
+    atomicAdd(g, x);
+    atomicAdd(g + 1, y);
+    atomicAdd(g + 2, z);
+    return;
+  }
+  const bool odd = (vid & 1u) != 0u;
+  atomicAdd(reinterpret_cast<float2 *>(g + (odd ? 1 : 0)), odd ? make_float2(y, z) : make_float2(x, y));
+  atomicAdd(g + (odd ? 0 : 2), odd ? x : z);
+}
+
+template <bool PAIRED>
 __global__ void __launch_bounds__(256) backward_kernel(BackwardArgs a) {
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += stride) {
-    const uint4 h = __ldg(reinterpret_cast<const uint4 *>(a.hits) + i);
+  const uint32_t lane = threadIdx.x & 31u;
+  for (unsigned long long b = (unsigned long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); b < a.n; b += stride) {
+    const unsigned long long i = b + lane;
+    uint4 h = make_uint4(0, 0, 0, 0xFFFFFFFFu);
+    if (i < a.n) h = __ldg(reinterpret_cast<const uint4 *>(a.hits) + i);
     const uint32_t prim = h.w;
-    float4 *gr = a.grad_rays ? reinterpret_cast<float4 *>(a.grad_rays) + 2 * i : nullptr;
-    if (prim >= a.n_tris) {
-      if (gr) {
-        gr[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-        gr[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+    bool valid = prim < a.n_tris;
+    float lf[3] = {0.f, 0.f, 0.f};
+    uint32_t vid[3] = {0, 0, 0};
+    if (valid) {
+      if (a.tri_idx) {
+        vid[0] = __ldg(a.tri_idx + 3 * (size_t)prim);
+        vid[1] = __ldg(a.tri_idx + 3 * (size_t)prim + 1);
+        vid[2] = __ldg(a.tri_idx + 3 * (size_t)prim + 2);
+      } else {
+        vid[0] = 3 * prim;
+        vid[1] = 3 * prim + 1;
+        vid[2] = 3 * prim + 2;
       }
-      continue;
-    }
-    uint32_t vid[3];
-    if (a.tri_idx) {
-      vid[0] = __ldg(a.tri_idx + 3 * (size_t)prim);
-      vid[1] = __ldg(a.tri_idx + 3 * (size_t)prim + 1);
-      vid[2] = __ldg(a.tri_idx + 3 * (size_t)prim + 2);
-    } else {
-      vid[0] = 3 * prim;
-      vid[1] = 3 * prim + 1;
-      vid[2] = 3 * prim + 2;
-    }
-    const float4 p0 = __ldg(a.verts + vid[0]), p1 = __ldg(a.verts + vid[1]), p2 = __ldg(a.verts + vid[2]);
-    const float4 rd = __ldg(reinterpret_cast<const float4 *>(a.rays) + 2 * i + 1);
-    // columns of J, exact in double (differences of two floats)
-    const double c0[3] = {rd.x, rd.y, rd.z};
-    const double c1[3] = {-((double)p1.x - p0.x), -((double)p1.y - p0.y), -((double)p1.z - p0.z)};
-    const double c2[3] = {-((double)p2.x - p0.x), -((double)p2.y - p0.y), -((double)p2.z - p0.z)};
-    const float gt = a.grad_tuv[3 * i], gu = a.grad_tuv[3 * i + 1], gv = a.grad_tuv[3 * i + 2];
-    double lam[3];
-    if (!solve_refined(c0, c1, c2, gt, gu, gv, lam)) {
-      double x12[3], x20[3], x01[3];
-      cross3(c1, c2, x12);
-      cross3(c2, c0, x20);
-      cross3(c0, c1, x01);
-      const double det = dot3(c0, x12);
-      if (det == 0.0) {
-        if (gr) {
-          gr[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-          gr[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        continue;
+      const float4 p0 = __ldg(a.verts + vid[0]), p1 = __ldg(a.verts + vid[1]), p2 = __ldg(a.verts + vid[2]);
+      const float4 rd = __ldg(reinterpret_cast<const float4 *>(a.rays) + 2 * i + 1);
+      // columns of J, each an exact pair
+      const Pair c0[3] = {{rd.x, 0.f}, {rd.y, 0.f}, {rd.z, 0.f}};
+      const Pair c1[3] = {two_diff(p0.x, p1.x), two_diff(p0.y, p1.y), two_diff(p0.z, p1.z)};
+      const Pair c2[3] = {two_diff(p0.x, p2.x), two_diff(p0.y, p2.y), two_diff(p0.z, p2.z)};
+      const float gt = a.grad_tuv[3 * i], gu = a.grad_tuv[3 * i + 1], gv = a.grad_tuv[3 * i + 2];
+      if (!solve_refined(c0, c1, c2, gt, gu, gv, lf)) {
+        // the columns in double: differences of two floats
+        const double e0[3] = {rd.x, rd.y, rd.z};
+        const double e1[3] = {(double)p0.x - p1.x, (double)p0.y - p1.y, (double)p0.z - p1.z};
+        const double e2[3] = {(double)p0.x - p2.x, (double)p0.y - p2.y, (double)p0.z - p2.z};
+        double x12[3], x20[3], x01[3];
+        cross3(e1, e2, x12);
+        cross3(e2, e0, x20);
+        cross3(e0, e1, x01);
+        const double det = dot3(e0, x12);
+        if (det == 0.0) valid = false;
+        for (int k = 0; k < 3; ++k)
+          lf[k] = valid ? (float)(((double)gt * x12[k] + (double)gu * x20[k] + (double)gv * x01[k]) / det) : 0.f;
       }
-      for (int k = 0; k < 3; ++k) lam[k] = ((double)gt * x12[k] + (double)gu * x20[k] + (double)gv * x01[k]) / det;
     }
-    // the scatter in single precision from lambda rounded once
-    const float lf[3] = {(float)lam[0], (float)lam[1], (float)lam[2]};
-    const float t = __uint_as_float(h.x), u = __uint_as_float(h.y), v = __uint_as_float(h.z);
+    const float t = valid ? __uint_as_float(h.x) : 0.f, u = __uint_as_float(h.y), v = __uint_as_float(h.z);
+    if (a.grad_rays && i < a.n) {
+      float4 *gr = reinterpret_cast<float4 *>(a.grad_rays) + 2 * i;
+      gr[0] = valid ? make_float4(-lf[0], -lf[1], -lf[2], 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+      gr[1] = valid ? make_float4(-t * lf[0], -t * lf[1], -t * lf[2], 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float c[9];
     const float w[3] = {(1.0f - u) - v, u, v};
     for (int j = 0; j < 3; ++j)
-      for (int k = 0; k < 3; ++k) atomicAdd(a.grad_verts + 3 * (size_t)vid[j] + k, w[j] * lf[k]);
-    if (gr) {
-      gr[0] = make_float4(-lf[0], -lf[1], -lf[2], 0.f);
-      gr[1] = make_float4(-t * lf[0], -t * lf[1], -t * lf[2], 0.f);
+      for (int k = 0; k < 3; ++k) c[3 * j + k] = valid ? w[j] * lf[k] : 0.f;
+    // neighbouring rays often hit one triangle: the first lane of such a run
+    // adds the run's sum (segmented sums over the warp, skipped where no lane
+    // follows its neighbour)
+    const uint32_t key = valid ? prim : 0xFFFFFFFFu;
+    const uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, key, 1);
+    const bool same = valid && lane > 0 && prev == key;
+    const uint32_t heads = __ballot_sync(0xFFFFFFFFu, !same);
+    if (heads != 0xFFFFFFFFu) {
+      const uint32_t later = heads & (0xFFFFFFFEu << lane);  // first lanes of the runs after this lane's
+      const uint32_t end = later ? __ffs(later) - 1 : 32;
+      for (int o = 1; o < 32; o <<= 1) {
+        const bool in = lane + o < end;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+          const float x = __shfl_down_sync(0xFFFFFFFFu, c[k], o);
+          if (in) c[k] += x;
+        }
+      }
+    }
+    if (valid && !same) {
+      for (int j = 0; j < 3; ++j) add_vertex<PAIRED>(a.grad_verts, vid[j], 1.0f, c + 3 * j);
     }
   }
 }
@@ -140,7 +213,8 @@ cudaError_t launch_backward(const BackwardArgs &a, int sms, cudaStream_t s) {
   if (a.n == 0) return cudaSuccess;
   const unsigned long long blocks = (a.n + 255) / 256;
   const unsigned grid = (unsigned)(blocks < (unsigned long long)sms * 8 ? blocks : (unsigned long long)sms * 8);
-  backward_kernel<<<grid, 256, 0, s>>>(a);
+  if ((reinterpret_cast<uintptr_t>(a.grad_verts) & 7u) == 0) backward_kernel<true><<<grid, 256, 0, s>>>(a);
+  else backward_kernel<false><<<grid, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 

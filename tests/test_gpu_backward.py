@@ -74,6 +74,30 @@ def test_backward_matches_fp64_reference(setup, layout):
     assert np.all(gr[miss] == 0)
 
 
+@pytest.mark.parametrize("scale", [2.0 ** k for k in (-96, -90, 0, 66, 96)])
+@pytest.mark.parametrize("shift", [0, 1, 2])
+def test_backward_gradient_ranges_and_alignment(setup, scale, shift):
+    """Gradients at and beyond the range of the pair arithmetic (its ends fall
+    back to the double-precision solve), into a vertex gradient that starts on
+    an 8-byte boundary or 4 bytes past one. The bound is the FP32 summation
+    error of the reference test, scaled; the scales are powers of two, so the
+    scaled gradients are exact. (FP32 atomics flush results below 1.2e-38 to
+    zero: at 2^-96 that is 1e-9 of the scaled value per addend, far inside the
+    bound's 1e-6.)"""
+    scion, sc, rays, tris, g, hits, gv64, gr64 = setup
+    bvh = scion.scion_build(sc.verts, scion.layout(width=4, box_layout="soa"), sc.indices)
+    d_rays = torch.from_numpy(rays).cuda()
+    h = scion.scion_trace_closest(bvh, d_rays)
+    buf = torch.zeros(3 * sc.verts.shape[0] + 4, dtype=torch.float32, device="cuda")
+    out = buf[shift:shift + 3 * sc.verts.shape[0]].view(-1, 3)
+    gv, gr = scion.scion_trace_backward(bvh, d_rays, h, torch.from_numpy(g).cuda() * scale, grad_verts=out)
+    S = _abs_scale(sc, rays, hits, g, tris)
+    assert np.all(np.abs(gv.cpu().numpy().astype(np.float64) / scale - gv64) <= 1e-5 * S + 1e-6)
+    got = gr.cpu().numpy().astype(np.float64)[:, :3] / scale
+    assert np.all(np.abs(got - gr64[:, :3]) <= 1e-6 * np.abs(gr64[:, :3]) + 1e-6)
+    assert float(buf[:shift].abs().sum()) == 0 and float(buf[shift + 3 * sc.verts.shape[0]:].abs().sum()) == 0
+
+
 def test_backward_against_central_differences(setup, oracle_mod):
     scion, sc, rays, tris, g, hits, gv64, gr64 = setup
     fv, fr = oracle_mod.grad_fd(tris, sc.indices, sc.verts.shape[0], rays, hits, g, 1e-4)
