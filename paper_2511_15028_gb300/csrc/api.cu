@@ -911,12 +911,13 @@ scion_status scion_refit(scion_bvh bvh, const float *d_verts, uint64_t n_verts, 
   if (!on_bvh_device(bvh)) return SCION_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   scion_bvh b = bvh;
-  if (!b->d_refit_parent && b->n_nodes > 0) {
+  const bool first = !b->d_refit_parent;
+  if (first && b->n_nodes > 0) {
     const size_t n = b->n_nodes;
     cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&b->d_refit_parent), n * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&b->d_refit_pending), n * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_refit_boxes, n * 6 * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&b->d_refit_frame), 16 * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&b->d_refit_frame), kRefitFrameFloats * sizeof(float));
     if (e != cudaSuccess) {
       cudaFree(b->d_refit_parent);
       cudaFree(b->d_refit_pending);
@@ -941,6 +942,7 @@ scion_status scion_refit(scion_bvh bvh, const float *d_verts, uint64_t n_verts, 
   rb.n_verts = b->n_verts;
   rb.own_box = b->own_box;
   rb.desc = b->desc;
+  rb.first = first;
   rb.parent = b->d_refit_parent;
   rb.pending = b->d_refit_pending;
   rb.boxes = b->d_refit_boxes;

@@ -1,6 +1,6 @@
-// Box codecs of the physical layouts, compiled for the host packer and for
-// the device refit alike (one implementation, identical IEEE arithmetic on
-// both sides: no contraction, correctly rounded double and float ops).
+// Box codecs of the physical layouts: the host packer's, and the definition of
+// the bytes that the device encoders (codec_fast.h) write too (identical IEEE
+// arithmetic: no contraction, correctly rounded double and float ops).
 //
 // Every encoder writes a box that encloses its input: f32 as is, f16 and
 // world-grid codes rounded outward, u8 codes verified against the device

@@ -10,6 +10,8 @@
 
 namespace scion {
 
+constexpr uint32_t kRefitFrameFloats = 18;
+
 struct RefitBuffers {
   void *nodes, *nodes2, *prims, *verts4;  // the BVH's device buffers
   const uint32_t *prim_ids, *tri_idx;
@@ -17,8 +19,10 @@ struct RefitBuffers {
   uint64_t n_verts;
   bool own_box;
   scion_layout_desc desc;
-  // refit scratch (device): n_nodes parents and counters, n_nodes boxes of
-  // 24 bytes, 12 floats of world grid (q16/eq10)
+  // refit scratch (device): n_nodes parents and counters (written by the
+  // BVH's first refit and kept), n_nodes boxes of 24 bytes, 18 floats of world
+  // grid (q16/eq10)
+  bool first;
   uint32_t *parent, *pending;
   void *boxes;
   float *frame;
