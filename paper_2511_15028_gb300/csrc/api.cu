@@ -45,7 +45,9 @@ struct scion_bvh_s {
   cudaStream_t slot_stream[kStreamSlotCount] = {};
   double build_ms = 0.0, logical_ms = 0.0, pack_ms = 0.0;
   int device = 0;
-  // refit scratch, allocated by the first scion_refit
+  // refit scratch, allocated by the first scion_refit; refit_linked: it holds
+  // the nodes' parents and counters
+  bool refit_linked = false;
   uint32_t *d_refit_parent = nullptr, *d_refit_pending = nullptr;
   void *d_refit_boxes = nullptr;
   float *d_refit_frame = nullptr;
@@ -911,8 +913,7 @@ scion_status scion_refit(scion_bvh bvh, const float *d_verts, uint64_t n_verts, 
   if (!on_bvh_device(bvh)) return SCION_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   scion_bvh b = bvh;
-  const bool first = !b->d_refit_parent;
-  if (first && b->n_nodes > 0) {
+  if (!b->d_refit_parent && b->n_nodes > 0) {
     const size_t n = b->n_nodes;
     cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&b->d_refit_parent), n * sizeof(uint32_t));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&b->d_refit_pending), n * sizeof(uint32_t));
@@ -942,13 +943,14 @@ scion_status scion_refit(scion_bvh bvh, const float *d_verts, uint64_t n_verts, 
   rb.n_verts = b->n_verts;
   rb.own_box = b->own_box;
   rb.desc = b->desc;
-  rb.first = first;
+  rb.first = !b->refit_linked;
   rb.parent = b->d_refit_parent;
   rb.pending = b->d_refit_pending;
   rb.boxes = b->d_refit_boxes;
   rb.frame = b->d_refit_frame;
   rb.status = b->d_scratch + 3;
   SCION_CUDA(refit_launch(rb, d_verts, s));
+  b->refit_linked = true;
   if (prec_has_frame(b->desc.box_prec) && b->n_nodes > 0) {
     // the traversal takes the grid as a launch argument: read it back
     SCION_CUDA(cudaMemcpyAsync(b->frame, b->d_refit_frame, 9 * sizeof(float), cudaMemcpyDeviceToHost, s));
