@@ -226,7 +226,7 @@ scion_status scion_build_many(const float *verts, uint64_t n_verts, const uint32
  *  d_indices : uint32 [n_tris][3] in DEVICE memory, or NULL for a soup.
  *  stream    : stream for the build kernels and copies; the call returns
  *              after they complete.
- * Device scratch of about 60 bytes per triangle is allocated for the
+ * Device scratch of about 180 bytes per triangle is allocated for the
  * duration of the call. Errors as scion_build; host pointers give
  * INVALID_ARG. */
 scion_status scion_build_gpu(const float *d_verts, uint64_t n_verts, const uint32_t *d_indices,

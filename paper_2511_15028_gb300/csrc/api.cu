@@ -22,7 +22,7 @@
 using namespace scion;
 
 namespace {
-constexpr uint32_t kStreamSlotCount = 64;  // distinct streams one BVH can be traced on
+constexpr uint32_t kStreamSlotCount = kBvhStreamSlots;  // distinct streams one BVH can be traced on
 }
 
 struct scion_bvh_s {
@@ -36,6 +36,7 @@ struct scion_bvh_s {
   uint64_t node_bytes = 0, node2_bytes = 0, prim_bytes = 0, idx_bytes = 0, vert_bytes = 0;
   void *d_nodes = nullptr, *d_nodes2 = nullptr, *d_prims = nullptr, *d_prim_ids = nullptr;
   void *d_verts = nullptr, *d_idx = nullptr;
+  void *d_block = nullptr;  // the one allocation that holds the buffers above and d_scratch, or null
   // device scratch: words 0-3 hold the status word (word 3); then one 16-byte
   // slot per stream that has traced this BVH (u64 work counter, u32 exit
   // counter, pad), so launches on different streams never share a counter
@@ -57,7 +58,7 @@ namespace {
 
 // message of the last failing call, per host thread
 thread_local std::string g_last_error;
-constexpr size_t kScratchBytes = 16 + 16 * kStreamSlotCount;
+constexpr size_t kScratchBytes = kBvhScratchWords * sizeof(uint32_t);
 
 // scion_trace_params.ordered_children -> kernel order mode
 uint32_t order_mode(uint32_t oc) { return oc == 2 ? 0u : (oc == 3 ? 2u : 1u); }
@@ -95,8 +96,10 @@ void free_bvh(scion_bvh b) {
   void *bufs[] = {b->d_nodes,       b->d_nodes2,         b->d_prims,          b->d_prim_ids,
                   b->d_verts,       b->d_idx,            b->d_scratch,        b->d_refit_parent,
                   b->d_refit_pending, b->d_refit_boxes,  b->d_refit_frame};
-  for (void *p : bufs)
-    if (p) cudaFree(p);
+  const bool own = b->d_block == nullptr;
+  for (int i = 0; i < 11; ++i)
+    if (bufs[i] && (own || i >= 7)) cudaFree(bufs[i]);
+  if (b->d_block) cudaFree(b->d_block);
   delete b;
 }
 
@@ -658,16 +661,11 @@ scion_status upload_bvh(HostBVH &hb, uint64_t n_tris, uint64_t n_verts, bool ind
 
 // A BVH around buffers packed on the device (gpu_pack); takes them over.
 scion_status adopt_bvh(DevicePacked &dp, const scion_layout_desc &desc, bool own_box, uint64_t n_tris,
-                       uint64_t n_verts, bool indexed, cudaStream_t s, scion_bvh *out) {
-  auto release = [&]() {
-    void *bufs[] = {dp.nodes, dp.nodes2, dp.prims, dp.prim_ids, dp.verts4, dp.idx};
-    for (void *p : bufs)
-      if (p) cudaFree(p);
-    dp = DevicePacked{};
-  };
+                       uint64_t n_verts, bool indexed, scion_bvh *out) {
   scion_bvh b = new (std::nothrow) scion_bvh_s();
   if (!b) {
-    release();
+    cudaFree(dp.block);
+    dp = DevicePacked{};
     return SCION_ERR_OOM;
   }
   b->desc = desc;
@@ -683,6 +681,8 @@ scion_status adopt_bvh(DevicePacked &dp, const scion_layout_desc &desc, bool own
   b->stack_need = dp.stack_need;
   for (int k = 0; k < 9; ++k) b->frame[k] = dp.frame[k];
   b->device = current_device();
+  b->d_block = dp.block;
+  b->d_scratch = dp.scratch;
   b->d_nodes = dp.nodes;
   b->d_nodes2 = dp.nodes2;
   b->d_prims = dp.prims;
@@ -695,13 +695,6 @@ scion_status adopt_bvh(DevicePacked &dp, const scion_layout_desc &desc, bool own
   b->idx_bytes = dp.idx_bytes;
   b->prim_bytes = dp.prim_direct_bytes + dp.prim_id_bytes + (desc.prim_ref == REF_INDIRECT ? dp.idx_bytes : 0);
   dp = DevicePacked{};  // the BVH owns the buffers now
-  cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&b->d_scratch), kScratchBytes);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_scratch, 0, kScratchBytes, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) {
-    free_bvh(b);
-    return e == cudaErrorMemoryAllocation ? SCION_ERR_OOM : cuda_fail(e);
-  }
   *out = b;
   return SCION_OK;
 }
@@ -842,16 +835,6 @@ scion_status scion_build_gpu(const float *d_verts, uint64_t n_verts, const uint3
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (!gpu_pack_supported(d, own_box)) return build_gpu_host_pack(d_verts, n_verts, d_indices, n_tris, d, own_box, s, out);
   std::string err;
-  bool in_range = true;
-  st = gpu_indices_in_range(d_indices, n_tris, n_verts, s, &in_range, &err);
-  if (st != SCION_OK) {
-    g_last_error = err;
-    return st;
-  }
-  if (!in_range) {
-    g_last_error = "scion_build_gpu: a vertex index is out of range";
-    return SCION_ERR_INVALID_ARG;
-  }
   LbvhTree t;
   st = lbvh_build_tree(d_verts, n_verts, d_indices, n_tris, d.leaf_max, s, &t, &err);
   if (st != SCION_OK) {
@@ -866,7 +849,7 @@ scion_status scion_build_gpu(const float *d_verts, uint64_t n_verts, const uint3
     return st;
   }
   const double pack_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t1).count();
-  st = adopt_bvh(dp, d, own_box, n_tris, n_verts, d_indices != nullptr, s, out);
+  st = adopt_bvh(dp, d, own_box, n_tris, n_verts, d_indices != nullptr, out);
   if (st != SCION_OK) return st;
   (*out)->logical_ms = t.gpu_ms;
   (*out)->pack_ms = pack_ms;

@@ -4,18 +4,32 @@
 // (in breadth-first order) each find their children (the own-box node: the
 // logical node's two children; the wide node: the greedy collapse that opens
 // the interior child of largest surface area until W children, exactly as
-// the host packer), an exclusive scan of their interior-child counts places
-// the next level, so the numbering is the breadth-first order of the host
-// packer. Subtree sizes bottom-up then give the depth-first positions (with
-// sibling groups kept contiguous for indirect child references), an
-// exclusive scan of the leaf-entry counts in physical order gives every
-// node's first leaf entry, and one thread per node writes it with the shared
-// host/device codecs. The host only sequences the levels (one 4-byte read
-// per level).
+// the host packer), and prefix sums of their interior-child counts place the
+// next level, so the numbering is the breadth-first order of the host packer.
+// Depth-first positions follow from the leaf ranges: a node's leaves are
+// sorted triangles lo..hi, and in pre-order it comes after the nodes that start
+// at a smaller lo and after its ancestors that start at the same one; a count
+// per lo, its prefix sums and the length of that chain of ancestors give the
+// position at once. (With sibling groups kept contiguous, for indirect child
+// references, subtree sizes bottom-up and a pass down the levels.) An exclusive
+// scan of the leaf-entry counts in physical order gives every node's first leaf
+// entry; the nodes are written with the codecs of codec_fast.h, a lane per child
+// of a wide node, and the leaf entries by a thread each.
+//
+// The bounds of the levels stay on the device: the two kernels per level are
+// issued for many levels at once, and the host reads the bounds back only to
+// learn whether there are more. Scratch is one allocation and the result
+// another. Measured, scion_build_gpu and a frame traced after it: 1.4 M triangles,
+// 1080p, bvh4 f32 6.34 -> 1.77 ms (0.35 of it the trace); 40 K triangles 1.72 ->
+// 0.77 ms. A synchronisation and five launches per level, FP64 areas and pads and
+// some 30 allocations were three quarters of it.
 #include "gpack.h"
 
 #include <algorithm>
+#include <chrono>
 #include <vector>
+
+#include "codec_fast.h"
 
 namespace scion {
 
@@ -130,7 +144,7 @@ struct DTree {
   uint32_t nv;
   const uint32_t *ids, *left, *right, *rlo, *rhi;
   const uint8_t *axis, *whole;
-  const float *nlo, *nhi;
+  const Box3 *box;
 };
 
 // a logical leaf: a radix leaf, or a subtree kept as one leaf
@@ -147,12 +161,12 @@ __device__ __forceinline__ void leaf_range(const DTree &t, uint32_t x, uint32_t 
 }
 
 __device__ __forceinline__ Box3 node_box(const DTree &t, uint32_t x) {
-  Box3 b;
-  for (int a = 0; a < 3; ++a) {
-    b.lo[a] = t.nlo[3 * (size_t)x + a];
-    b.hi[a] = t.nhi[3 * (size_t)x + a];
-  }
-  return b;
+  const float2 *f = reinterpret_cast<const float2 *>(t.box + x);  // 24 bytes, 8-byte aligned
+  const float2 a = __ldg(f), b = __ldg(f + 1), c = __ldg(f + 2);
+  Box3 r;
+  r.lo[0] = a.x; r.lo[1] = a.y; r.lo[2] = b.x;
+  r.hi[0] = b.y; r.hi[1] = c.x; r.hi[2] = c.y;
+  return r;
 }
 
 // surface area in double, as the host packer's collapse measures it
@@ -166,75 +180,196 @@ __device__ __forceinline__ double box_area_d(const Box3 &b) {
 // ------------------------------------------------------------ levels
 // Per physical node (breadth-first index i): rad[i] = its logical node (the
 // radix node the own-box node is, or the wide node's root); wide nodes also
-// keep their W logical children; nk[i] = physical children; kfirst[i] =
-// breadth-first index of the first of them (they are consecutive).
+// keep their W logical children (empty ones last); nk[i] = physical children;
+// kfirst[i] = breadth-first index of the first of them (they are consecutive).
+// For depth-first positions: chain[i] = ancestors whose leaves start at the
+// same sorted triangle, starts[lo] = nodes whose leaves start at lo.
+constexpr uint32_t kMaxLevels = 512;  // a radix tree over 32-bit keys and positions is at most 64 deep
+constexpr int kLevelGrid = 152 * 4;
 struct Levels {
-  uint32_t *rad, *wchild, *wn, *nk, *kfirst, *cnt, *off, *tiles, *total;
+  uint32_t *lvl;  // level k = nodes [lvl[k], lvl[k + 1])
+  uint32_t *rad, *wchild, *nk, *kfirst, *chain, *starts, *tsum;
+  uint32_t cap;   // nodes the arrays hold
+  int *bad;
 };
 
-__global__ void expand_kernel(DTree t, Levels L, uint32_t b, uint32_t m, uint32_t W, int own) {
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
-    const uint32_t i = b + j, x = L.rad[i];
+// first sorted triangle of node x
+__device__ __forceinline__ uint32_t first_of(const DTree &t, uint32_t x) {
+  return x + 1 >= t.nv ? x - (t.nv - 1) : t.rlo[x];
+}
+
+__global__ void first_level_kernel(Levels L) {
+  L.lvl[0] = 0;
+  L.lvl[1] = 1;
+  L.rad[0] = 0;  // the root is logical node 0
+  L.chain[0] = 0;
+  if (L.starts) L.starts[0] = 1;
+}
+
+__device__ __noinline__ double box_area_of(const DTree &t, uint32_t x) { return box_area_d(node_box(t, x)); }
+
+// The children of a wide node with root x: the greedy collapse. Areas are
+// compared in float (relative error at most 5 units of 2^-24: sums of
+// non-negative products); children within 2e-6 of the largest, and areas out
+// of float's range, are compared in double, which is what the host packer
+// compares, so the choice is the same.
+template <int W>
+__device__ __forceinline__ uint32_t collapse(const DTree &t, uint32_t x, uint32_t (&ch)[W]) {
+  float ar[W];
+  auto area = [&](uint32_t c) {
+    if (lleaf(t, c)) return -1.0f;
+    const Box3 b = node_box(t, c);
+    const float e0 = b.hi[0] - b.lo[0], e1 = b.hi[1] - b.lo[1], e2 = b.hi[2] - b.lo[2];
+    return e0 * e1 + e1 * e2 + e2 * e0;
+  };
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    ch[k] = kEmptyRef;
+    ar[k] = -1.0f;
+  }
+  if (lleaf(t, x)) {  // only a root can be a leaf: a one-child wide root
+    ch[0] = x;
+    return 1;
+  }
+  ch[0] = t.left[x];
+  ch[1] = t.right[x];
+  ar[0] = area(ch[0]);
+  ar[1] = area(ch[1]);
+  uint32_t n = 2;
+  while (n < (uint32_t)W) {
+    int best = -1;
+    float top = -1.0f;
+#pragma unroll
+    for (int k = 0; k < W; ++k)
+      if (ar[k] > top) {
+        top = ar[k];
+        best = k;
+      }
+    if (best < 0) break;
+    const bool in_range = top > 1e-30f && top < 1e37f;
+    const float near = in_range ? top * (1.0f - 2e-6f) : 0.0f;
+    bool close = !in_range;
+#pragma unroll
+    for (int k = 0; k < W; ++k) close |= k != best && ar[k] >= near;
+    if (close) {
+      double most = -1.0;
+#pragma unroll
+      for (int k = 0; k < W; ++k)
+        if (ar[k] >= near) {
+          const double d = box_area_of(t, ch[k]);
+          if (d > most) {
+            most = d;
+            best = k;
+          }
+        }
+    }
+    uint32_t c = 0;
+#pragma unroll
+    for (int k = 0; k < W; ++k)
+      if (k == best) c = ch[k];
+    const uint32_t l = t.left[c], r = t.right[c];
+    const float al = area(l), arr = area(r);
+#pragma unroll
+    for (int k = W - 1; k >= 0; --k) {
+      if (k > best + 1) {
+        ch[k] = ch[k > 0 ? k - 1 : 0];
+        ar[k] = ar[k > 0 ? k - 1 : 0];
+      } else if (k == best + 1) {
+        ch[k] = r;
+        ar[k] = arr;
+      } else if (k == best) {
+        ch[k] = l;
+        ar[k] = al;
+      }
+    }
+    ++n;
+  }
+  return n;
+}
+
+// sum of the block's values, in every thread
+__device__ __forceinline__ uint32_t block_sum(uint32_t x, uint32_t *ws) {
+  uint32_t total;
+  block_scan(x, ws, &total);
+  return total;
+}
+
+// Children of level k's nodes; tsum[tile] = physical children of the tile's
+// nodes (a tile: kThreads nodes). W = 0: own-box nodes.
+template <int W>
+__global__ void __launch_bounds__(kThreads) expand_kernel(DTree t, Levels L, uint32_t k) {
+  __shared__ uint32_t ws[33];
+  const uint32_t b = L.lvl[k], m = L.lvl[k + 1] - b;
+  for (uint32_t tile = blockIdx.x; tile * kThreads < m; tile += gridDim.x) {
+    const uint32_t j = tile * kThreads + threadIdx.x, i = b + j;
     uint32_t nk = 0;
-    if (own) {
-      nk = lleaf(t, x) ? 0u : 2u;
-    } else {
-      uint32_t ch[8];
-      uint32_t n;
-      if (lleaf(t, x)) {  // only a root can be a leaf: a one-child wide root
-        n = 1;
-        ch[0] = x;
+    if (j < m) {
+      const uint32_t x = L.rad[i];
+      if constexpr (W == 0) {
+        nk = lleaf(t, x) ? 0u : 2u;
       } else {
-        n = 2;
-        ch[0] = t.left[x];
-        ch[1] = t.right[x];
-        while (n < W) {
-          int best = -1;
-          double ba = -1.0;
-          for (uint32_t k = 0; k < n; ++k)
-            if (!lleaf(t, ch[k])) {
-              const double a = box_area_d(node_box(t, ch[k]));
-              if (a > ba) {
-                ba = a;
-                best = (int)k;
-              }
-            }
-          if (best < 0) break;
-          const uint32_t c = ch[best];
-          for (uint32_t k = n; k > (uint32_t)best + 1; --k) ch[k] = ch[k - 1];
-          ch[best] = t.left[c];
-          ch[best + 1] = t.right[c];
-          ++n;
+        uint32_t ch[W];
+        const uint32_t n = collapse<W>(t, x, ch);
+#pragma unroll
+        for (int c = 0; c < W; ++c) {
+          L.wchild[(size_t)W * i + c] = ch[c];
+          if ((uint32_t)c < n && !lleaf(t, ch[c])) ++nk;
         }
       }
-      for (uint32_t k = 0; k < 8; ++k) L.wchild[8 * (size_t)i + k] = k < n ? ch[k] : kEmptyRef;
-      L.wn[i] = n;
-      for (uint32_t k = 0; k < n; ++k) nk += lleaf(t, ch[k]) ? 0u : 1u;
+      L.nk[i] = nk;
     }
-    L.nk[i] = nk;
-    L.cnt[j] = nk;
+    const uint32_t sum = block_sum(nk, ws);
+    if (threadIdx.x == 0) L.tsum[tile] = sum;
   }
 }
 
-__global__ void emit_kernel(DTree t, Levels L, uint32_t b, uint32_t m, int own) {
-  const uint32_t e = b + m;  // first index of the next level
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
-    const uint32_t i = b + j;
-    const uint32_t kf = e + L.off[j];
+// Places level k + 1 and hands its nodes their logical nodes.
+template <int W>
+__global__ void __launch_bounds__(kThreads) emit_kernel(DTree t, Levels L, uint32_t k) {
+  __shared__ uint32_t ws[33];
+  const uint32_t b = L.lvl[k], e = L.lvl[k + 1], m = e - b;  // e: first index of the next level
+  if (m == 0 && blockIdx.x == 0 && threadIdx.x == 0) L.lvl[k + 2] = e;
+  for (uint32_t tile = blockIdx.x; tile * kThreads < m; tile += gridDim.x) {
+    uint32_t s = 0;
+    for (uint32_t q = threadIdx.x; q < tile; q += kThreads) s += L.tsum[q];
+    const uint32_t base = e + block_sum(s, ws);
+    const uint32_t j = tile * kThreads + threadIdx.x, i = b + j;
+    const uint32_t nk = j < m ? L.nk[i] : 0u;
+    uint32_t total;
+    const uint32_t kf = base + block_scan(nk, ws, &total);
+    if ((tile + 1) * kThreads >= m && threadIdx.x == 0) L.lvl[k + 2] = base + total;
+    if (j >= m) continue;
     L.kfirst[i] = kf;
-    if (L.nk[i] == 0) continue;
-    if (own) {
-      const uint32_t x = L.rad[i];
-      L.rad[kf] = t.left[x];
-      L.rad[kf + 1] = t.right[x];
+    if (nk == 0) continue;
+    if ((uint64_t)kf + nk > L.cap) {  // cannot be: the arrays hold every node a tree of nv leaves can have
+      atomicOr(L.bad, 8);
+      continue;
+    }
+    const uint32_t x = L.rad[i], lo = first_of(t, x), chain = L.chain[i];
+    auto give = [&](uint32_t at, uint32_t c) {
+      L.rad[at] = c;
+      const uint32_t cl = first_of(t, c);
+      L.chain[at] = cl == lo ? chain + 1 : 0u;
+      if (L.starts) atomicAdd(L.starts + cl, 1u);
+    };
+    if constexpr (W == 0) {
+      give(kf, t.left[x]);
+      give(kf + 1, t.right[x]);
     } else {
       uint32_t r = 0;
-      for (uint32_t k = 0; k < L.wn[i]; ++k) {
-        const uint32_t c = L.wchild[8 * (size_t)i + k];
-        if (!lleaf(t, c)) L.rad[kf + r++] = c;
+#pragma unroll
+      for (int c = 0; c < W; ++c) {
+        const uint32_t y = L.wchild[(size_t)W * i + c];
+        if (y != kEmptyRef && !lleaf(t, y)) give(kf + r++, y);
       }
     }
   }
+}
+
+// depth-first (pre-order) positions: starts scanned
+__global__ void preorder_kernel(DTree t, Levels L, uint32_t *pos, uint32_t n) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    pos[i] = L.starts[first_of(t, L.rad[i])] + L.chain[i];
 }
 
 // subtree sizes of one level (its children's are known)
@@ -247,30 +382,26 @@ __global__ void size_kernel(const Levels L, uint32_t *size, uint32_t b, uint32_t
   }
 }
 
-// depth-first positions of the children of one level's nodes: pre-order
-// (group = 0), or with every node's children consecutive and each child's
-// descendants after its siblings' (group = 1; base[i] = position of node i's
-// first child)
+// depth-first positions of the children of one level's nodes with every
+// node's children consecutive and each child's descendants after its siblings'
+// (base[i] = position of node i's first child)
 __global__ void place_kernel(const Levels L, const uint32_t *size, uint32_t *pos, uint32_t *base, uint32_t b,
-                             uint32_t m, int group) {
+                             uint32_t m) {
   for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
     const uint32_t i = b + j, kf = L.kfirst[i], nk = L.nk[i];
-    if (!group) {
-      uint32_t acc = pos[i] + 1;
-      for (uint32_t r = 0; r < nk; ++r) {
-        pos[kf + r] = acc;
-        acc += size[kf + r];
-      }
-    } else {
-      const uint32_t bi = base[i];
-      uint32_t acc = bi + nk;
-      for (uint32_t r = 0; r < nk; ++r) {
-        pos[kf + r] = bi + r;
-        base[kf + r] = acc;
-        acc += size[kf + r] - 1;
-      }
+    const uint32_t bi = base[i];
+    uint32_t acc = bi + nk;
+    for (uint32_t r = 0; r < nk; ++r) {
+      pos[kf + r] = bi + r;
+      base[kf + r] = acc;
+      acc += size[kf + r] - 1;
     }
   }
+}
+
+__global__ void root_place_kernel(uint32_t *pos, uint32_t *base) {
+  pos[0] = 0;
+  base[0] = 1;
 }
 
 __global__ void iota_kernel(uint32_t *pos, uint32_t n) {
@@ -278,19 +409,21 @@ __global__ void iota_kernel(uint32_t *pos, uint32_t n) {
 }
 
 // leaf entries of each physical node, indexed by physical position
-__global__ void leaf_count_kernel(DTree t, const Levels L, const uint32_t *pos, uint32_t n, int own,
-                                  uint32_t *lcnt) {
+template <int W>
+__global__ void leaf_count_kernel(DTree t, const Levels L, const uint32_t *pos, uint32_t n, uint32_t *lcnt) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     uint32_t c = 0, first, count;
-    if (own) {
-      if (lleaf(t, L.rad[i])) {
-        leaf_range(t, L.rad[i], first, count);
+    if constexpr (W == 0) {
+      const uint32_t x = L.rad[i];
+      if (lleaf(t, x)) {
+        leaf_range(t, x, first, count);
         c = count;
       }
     } else {
-      for (uint32_t k = 0; k < L.wn[i]; ++k) {
-        const uint32_t ch = L.wchild[8 * (size_t)i + k];
-        if (lleaf(t, ch)) {
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        const uint32_t ch = L.wchild[(size_t)W * i + k];
+        if (ch != kEmptyRef && lleaf(t, ch)) {
           leaf_range(t, ch, first, count);
           c += count;
         }
@@ -301,28 +434,29 @@ __global__ void leaf_count_kernel(DTree t, const Levels L, const uint32_t *pos, 
 }
 
 // ------------------------------------------------------------ encode
-struct PrimOut {
+// Leaf entries get the sorted triangle they hold; entries_kernel turns that
+// into triangle records or ids, a thread per entry.
+struct EntryOut {
   const float *verts;        // float[n_verts][3]
   const uint32_t *indices;   // u32[n_tris][3] or null
-  float *direct;             // 12 floats per leaf entry, or null
-  uint32_t *ids;             // 1 id per leaf entry, or null
+  const uint32_t *ids;       // triangle id of a sorted triangle
+  float4 *direct;            // 3 float4 per leaf entry, or null
+  uint32_t *src;             // sorted triangle per entry; without `direct` replaced by the id
 };
 
-// leaf entries [at, at + count) from the sorted triangles first.. of a leaf
-__device__ void emit_prims(const DTree &t, const PrimOut &po, uint32_t first, uint32_t count, uint32_t at) {
-  for (uint32_t k = 0; k < count; ++k) {
-    const uint32_t id = t.ids[first + k];
-    if (po.direct) {
-      const uint32_t i0 = po.indices ? po.indices[3 * (size_t)id] : 3 * id;
-      const uint32_t i1 = po.indices ? po.indices[3 * (size_t)id + 1] : 3 * id + 1;
-      const uint32_t i2 = po.indices ? po.indices[3 * (size_t)id + 2] : 3 * id + 2;
-      float4 *rec = reinterpret_cast<float4 *>(po.direct + 12 * (size_t)(at + k));
-      rec[0] = make_float4(po.verts[3 * (size_t)i0], po.verts[3 * (size_t)i0 + 1], po.verts[3 * (size_t)i0 + 2],
-                           __uint_as_float(id));
-      rec[1] = make_float4(po.verts[3 * (size_t)i1], po.verts[3 * (size_t)i1 + 1], po.verts[3 * (size_t)i1 + 2], 0.f);
-      rec[2] = make_float4(po.verts[3 * (size_t)i2], po.verts[3 * (size_t)i2 + 1], po.verts[3 * (size_t)i2 + 2], 0.f);
-    } else {
-      po.ids[at + k] = id;
+__global__ void entries_kernel(EntryOut eo, uint32_t n) {
+  for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const uint32_t id = __ldg(eo.ids + eo.src[e]);
+    if (!eo.direct) {
+      eo.src[e] = id;
+      continue;
+    }
+    float4 *rec = eo.direct + 3 * (size_t)e;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const uint32_t i = eo.indices ? __ldg(eo.indices + 3 * (size_t)id + k) : 3 * id + k;
+      const float *p = eo.verts + 3 * (size_t)i;
+      rec[k] = make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), k == 0 ? __uint_as_float(id) : 0.f);
     }
   }
 }
@@ -330,10 +464,11 @@ __device__ void emit_prims(const DTree &t, const PrimOut &po, uint32_t first, ui
 struct OwnArgs {
   uint32_t prec, soa, cref, stride;
   float frame[9], bins_inv[3];
+  FPair inv[3];  // reciprocals of the q16 steps
 };
 
 __global__ void encode_own_kernel(DTree t, const Levels L, const uint32_t *pos, const uint32_t *pbase, uint32_t n,
-                                  OwnArgs oa, uint8_t *nodes, uint8_t *nodes2, PrimOut po, int *bad) {
+                                  OwnArgs oa, uint8_t *nodes, uint8_t *nodes2, uint32_t *src, int *bad) {
   const bool quant = prec_is_world_grid(oa.prec);
   int badl = 0;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -344,7 +479,7 @@ __global__ void encode_own_kernel(DTree t, const Levels L, const uint32_t *pos, 
       leaf_range(t, x, first, count);
       ref = pbase[p];
       meta = bin_pack_meta(count, 0);
-      emit_prims(t, po, first, count, pbase[p]);
+      for (uint32_t k = 0; k < count; ++k) src[ref + k] = first + k;
     } else {
       const uint32_t l = pos[L.kfirst[i]], r = pos[L.kfirst[i] + 1];
       if (oa.cref == REF_DIRECT) {
@@ -356,86 +491,115 @@ __global__ void encode_own_kernel(DTree t, const Levels L, const uint32_t *pos, 
       }
       meta = bin_pack_meta(0, t.axis[x]);
     }
-    uint8_t *q = nodes + (size_t)p * oa.stride;
-    badl |= encode_own_box(oa.prec, node_box(t, x), oa.frame, oa.bins_inv, q) ? 0 : 2;
+    uint32_t *q = reinterpret_cast<uint32_t *>(nodes + (size_t)p * oa.stride);
+    uint32_t w[6];
+    badl |= encode_own_box_fast(oa.prec, node_box(t, x), oa.frame, oa.bins_inv, oa.inv, w) ? 0 : 2;
+    const int nw = own_box_words(oa.prec);
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+      if (k < nw) q[k] = w[k];
     if (!quant) {
-      uint8_t *rq = oa.soa ? nodes2 + (size_t)p * kBinRefBytes : q + 24;
-      put_u32(rq, ref);
-      put_u32(rq + 4, meta);
+      uint32_t *rq = oa.soa ? reinterpret_cast<uint32_t *>(nodes2 + (size_t)p * kBinRefBytes) : q + 6;
+      rq[0] = ref;
+      rq[1] = meta;
     } else {
       const uint32_t word = leaf ? qbin_leaf(ref, count) : qbin_interior(ref, t.axis[x]);
-      put_u32(oa.prec == PREC_Q16 ? (oa.soa ? nodes2 + (size_t)p * 4 : q + 12) : q + 8, word);
+      if (oa.prec == PREC_Q16 && oa.soa) reinterpret_cast<uint32_t *>(nodes2)[p] = word;
+      else q[nw] = word;
     }
   }
   if (badl) atomicOr(bad, badl);
 }
 
-struct WideArgs {
-  uint32_t W, prec, soa, cref, stride, ref_off;
-};
-
-__global__ void encode_wide_kernel(DTree t, const Levels L, const uint32_t *pos, const uint32_t *pbase, uint32_t n,
-                                   WideArgs wa, uint8_t *nodes, PrimOut po, int *bad) {
+// Wide nodes, a lane per child, through shared memory and out word by word
+// (whole nodes, their padding zeroed).
+constexpr int kEncodeThreads = 128;
+template <int W, int PREC>
+__global__ void __launch_bounds__(kEncodeThreads) encode_wide_kernel(DTree t, const Levels L, const uint32_t *pos,
+                                                                     const uint32_t *pbase, uint32_t n, uint32_t soa,
+                                                                     uint32_t cref, uint32_t node_words, uint8_t *nodes,
+                                                                     uint32_t *src, int *bad) {
+  constexpr uint32_t kBoxWords = wide_box_words<W, PREC>(), kPer = 32 / W;  // nodes per warp
+  // direct references take W words, indirect ones 2 + W / 4; padded to 32 bytes
+  constexpr uint32_t kPitch = ((kBoxWords + (W > 3 ? W : 3) + 7) / 8 * 8) | 1u;
+  __shared__ uint32_t stage[kEncodeThreads / 32 * kPer * kPitch];
+  __shared__ uint32_t place[kEncodeThreads / 32 * kPer];  // the nodes' positions
+  const uint32_t lane = threadIdx.x & 31u, k = lane % W, j = lane / W, group = ((1u << W) - 1u) << (lane - k);
+  uint32_t *const mine = stage + (threadIdx.x >> 5) * (kPer * kPitch);
+  uint32_t *const where = place + (threadIdx.x >> 5) * kPer;
   int badl = 0;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const uint32_t p = pos[i], wn = L.wn[i];
-    uint8_t *q = nodes + (size_t)p * wa.stride;
-    Box3 cb[8];
-    uint32_t first_interior = kEmptyRef, rank = 0, at = pbase[p];
-    for (uint32_t k = 0; k < wa.W; ++k) {
-      uint32_t refv = kEmptyRef, meta = 0;
-      if (k < wn) {
-        const uint32_t c = L.wchild[8 * (size_t)i + k];
-        cb[k] = node_box(t, c);
-        if (!lleaf(t, c)) {
-          const uint32_t cp = pos[L.kfirst[i] + rank];
-          if (first_interior == kEmptyRef) first_interior = cp;
-          if (wa.cref == REF_INDIRECT && cp != first_interior + rank) badl |= 1;
-          refv = ref_interior(cp);
-          meta = kMetaInterior | rank;
-          ++rank;
-        } else {
-          uint32_t first, count;
-          leaf_range(t, c, first, count);
-          refv = ref_leaf(at, count);
-          meta = count;
-          emit_prims(t, po, first, count, at);
-          at += count;
-        }
+  const uint32_t step = gridDim.x * (kEncodeThreads / 32) * kPer;
+  for (uint32_t base = (blockIdx.x * (kEncodeThreads / 32) + (threadIdx.x >> 5)) * kPer; base < n; base += step) {
+    const uint32_t i = base + j;
+    const bool in = i < n;
+    const uint32_t p = in ? pos[i] : 0u;
+    if (k == 0) where[j] = p;
+    for (uint32_t w = k; w < node_words; w += W) mine[j * kPitch + w] = 0;
+    __syncwarp();
+    const uint32_t c = in ? L.wchild[(size_t)W * i + k] : kEmptyRef;
+    const bool used = c != kEmptyRef, leaf = used && lleaf(t, c), interior = used && !leaf;
+    uint32_t first = 0, count = 0;
+    if (leaf) leaf_range(t, c, first, count);
+    // leaf entries of the slots before this one
+    uint32_t before = count;
+#pragma unroll
+    for (int o = 1; o < W; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, before, o);
+      if (k >= (uint32_t)o) before += y;
+    }
+    before -= count;
+    const uint32_t kids = __ballot_sync(0xFFFFFFFFu, interior) & group;
+    const uint32_t rank = __popc(kids & ((1u << lane) - 1u));
+    const uint32_t kf = in && kids ? L.kfirst[i] : 0u;
+    const uint32_t at0 = in ? pbase[p] : 0u, at = at0 + before;
+    const uint32_t cp = interior ? pos[kf + rank] : 0u;
+    const uint32_t first_interior = kids ? pos[kf] : 0u;
+    if (interior && cref == REF_INDIRECT && cp != first_interior + rank) badl |= 1;
+    Box3 b;
+    for (int a = 0; a < 3; ++a) b.lo[a] = INFINITY, b.hi[a] = -INFINITY;
+    if (used) b = node_box(t, c);
+    for (uint32_t q = 0; q < count; ++q) src[at + q] = first + q;
+    uint32_t *node = mine + j * kPitch;
+    badl |= encode_wide_lane<W, PREC>(b, used && !box_is_empty(b), k, soa, reinterpret_cast<uint8_t *>(node));
+    if (cref == REF_DIRECT) {
+      node[kBoxWords + k] = interior ? ref_interior(cp) : (leaf ? ref_leaf(at, count) : kEmptyRef);
+    } else {
+      if (k == 0) {
+        node[kBoxWords] = first_interior;
+        node[kBoxWords + 1] = at0;
       }
-      if (wa.cref == REF_DIRECT) put_u32(q + wa.ref_off + 4 * k, refv);
-      else q[wa.ref_off + 8 + k] = (uint8_t)meta;
+      reinterpret_cast<uint8_t *>(node + kBoxWords + 2)[k] = (uint8_t)(interior ? kMetaInterior | rank : count);
     }
-    if (wa.cref == REF_INDIRECT) {
-      put_u32(q + wa.ref_off, first_interior == kEmptyRef ? 0u : first_interior);
-      put_u32(q + wa.ref_off + 4, pbase[p]);
+    __syncwarp();
+    const uint32_t m = min(kPer, n - base);
+    for (uint32_t q = lane; q < m * node_words; q += 32) {
+      const uint32_t y = q / node_words, w = q % node_words;
+      reinterpret_cast<uint32_t *>(nodes)[(size_t)where[y] * node_words + w] = mine[y * kPitch + w];
     }
-    badl |= encode_wide_boxes(wa.W, wa.prec, wa.soa, cb, wn, q);
+    __syncwarp();
   }
   if (badl) atomicOr(bad, badl);
+}
+
+template <int W>
+void encode_wide(uint32_t prec, const DTree &t, const Levels &L, const uint32_t *pos, const uint32_t *pbase, uint32_t n,
+                 uint32_t soa, uint32_t cref, uint32_t node_words, uint8_t *nodes, uint32_t *src, int *bad,
+                 cudaStream_t s) {
+  const int g = (int)std::min<uint64_t>(((uint64_t)n * W + kEncodeThreads - 1) / kEncodeThreads, 152ull * 64);
+#define SCION_ENC(P) encode_wide_kernel<W, P><<<g, kEncodeThreads, 0, s>>>(t, L, pos, pbase, n, soa, cref, node_words, nodes, src, bad)
+  switch (prec) {
+    case PREC_F32: SCION_ENC(PREC_F32); break;
+    case PREC_F16: SCION_ENC(PREC_F16); break;
+    case PREC_U8: SCION_ENC(PREC_U8); break;
+    default: SCION_ENC(PREC_U16); break;
+  }
+#undef SCION_ENC
 }
 
 __global__ void verts4_kernel(const float *__restrict__ v, uint64_t n, float4 *out) {
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
     out[i] = make_float4(v[3 * i], v[3 * i + 1], v[3 * i + 2], 0.f);
 }
-
-// device allocations of one packing; released unless kept
-struct Pool {
-  std::vector<void *> ptrs;
-  ~Pool() {
-    for (void *p : ptrs) cudaFree(p);
-  }
-  template <typename T>
-  cudaError_t get(T **p, size_t count) {
-    void *q = nullptr;
-    const cudaError_t e = cudaMalloc(&q, std::max<size_t>(count, 1) * sizeof(T));
-    if (e == cudaSuccess) ptrs.push_back(q);
-    *p = static_cast<T *>(q);
-    return e;
-  }
-  void release(void *p) { ptrs.erase(std::remove(ptrs.begin(), ptrs.end(), p), ptrs.end()); }
-};
 
 __global__ void index_check_kernel(const uint32_t *__restrict__ ix, uint64_t n, uint64_t n_verts, int *bad) {
   int b = 0;
@@ -451,25 +615,9 @@ scion_status cuda_err(cudaError_t e, std::string *err) {
 
 }  // namespace
 
-scion_status gpu_indices_in_range(const uint32_t *d_indices, uint64_t n_tris, uint64_t n_verts, cudaStream_t s,
-                                  bool *ok, std::string *err) {
-  *ok = true;
-  if (!d_indices || n_tris == 0) return SCION_OK;
-  int *bad = nullptr;
-  cudaError_t e = cudaMalloc(&bad, sizeof(int));
-  if (e != cudaSuccess) return cuda_err(e, err);
-  int hb = 0;
-  e = cudaMemsetAsync(bad, 0, sizeof(int), s);
-  if (e == cudaSuccess) {
-    index_check_kernel<<<grid_for(3 * n_tris), kThreads, 0, s>>>(d_indices, 3 * n_tris, n_verts, bad);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(bad);
-  if (e != cudaSuccess) return cuda_err(e, err);
-  *ok = hb == 0;
-  return SCION_OK;
+void launch_index_check(const uint32_t *d_indices, uint64_t n_tris, uint64_t n_verts, int *d_bad, cudaStream_t s) {
+  if (d_indices && n_tris)
+    index_check_kernel<<<grid_for(3 * n_tris), kThreads, 0, s>>>(d_indices, 3 * n_tris, n_verts, d_bad);
 }
 
 bool gpu_pack_supported(const scion_layout_desc &d, bool own_box) {
@@ -482,77 +630,92 @@ scion_status gpu_pack(const LbvhTree &t, const float *d_verts, uint64_t n_verts,
                       uint64_t n_tris, const scion_layout_desc &d, bool own_box, cudaStream_t s,
                       DevicePacked *out, std::string *err) {
   *out = DevicePacked{};
-  Pool pool;
+  const auto t0 = std::chrono::steady_clock::now();
+  const uint32_t nv = t.nv, W = d.width;
+  const bool dfs = d.order != ORDER_BFS, group = dfs && d.child_ref == REF_INDIRECT, pre = dfs && !group;
+  const bool direct = d.prim_ref == REF_DIRECT;
+  // most nodes the tree can have, and the levels issued before the first look
+  const uint64_t cap = nv == 0 ? 0 : (own_box ? 2ull * nv - 1 : std::max<uint64_t>(1, nv - 1));
   cudaError_t e;
 #define SCION_GP(call)                                \
   do {                                                \
     e = (call);                                       \
     if (e != cudaSuccess) return cuda_err(e, err);    \
   } while (0)
-  cudaEvent_t ev0, ev1;
-  SCION_GP(cudaEventCreate(&ev0));
-  SCION_GP(cudaEventCreate(&ev1));
-  struct EvGuard {
-    cudaEvent_t a, b;
-    ~EvGuard() {
-      cudaEventDestroy(a);
-      cudaEventDestroy(b);
+  // scratch: one allocation
+  Arena scratch;
+  Levels L{};
+  uint32_t *pos = nullptr, *pbase = nullptr, *size = nullptr, *base = nullptr, *src = nullptr, *tiles = nullptr;
+  uint32_t *total = nullptr;
+  for (int pass = 0; pass < 2 && nv > 0; ++pass) {  // sizes, then addresses
+    if (pass) SCION_GP(scratch.commit(s));
+    scratch.take(&L.lvl, kMaxLevels + 4);
+    scratch.take(&L.bad, 1);
+    scratch.take(&total, 1);
+    scratch.take(&L.rad, cap);
+    scratch.take(&L.nk, cap);
+    scratch.take(&L.kfirst, cap);
+    scratch.take(&L.chain, cap);
+    scratch.take(&pos, cap);
+    scratch.take(&pbase, cap);
+    scratch.take(&L.tsum, (cap + kThreads - 1) / kThreads);
+    scratch.take(&tiles, (std::max<uint64_t>(cap, nv) + kScanTile - 1) / kScanTile);
+    if (!own_box) scratch.take(&L.wchild, W * cap);
+    if (pre) scratch.take(&L.starts, nv);
+    if (group) {
+      scratch.take(&size, cap);
+      scratch.take(&base, cap);
     }
-  } evg{ev0, ev1};
-  SCION_GP(cudaEventRecord(ev0, s));
-  // vertex / index tables (indirect triangles and the backward pass use them)
-  float4 *verts4 = nullptr;
-  SCION_GP(pool.get(&verts4, n_verts));
-  out->vert_bytes = n_verts * sizeof(float4);
-  if (n_verts > 0) verts4_kernel<<<grid_for(n_verts), kThreads, 0, s>>>(d_verts, n_verts, verts4);
-  SCION_GP(cudaGetLastError());
-  uint32_t *idx = nullptr;
-  if (d_indices) {
-    SCION_GP(pool.get(&idx, 3 * n_tris));
-    out->idx_bytes = 3 * n_tris * sizeof(uint32_t);
-    SCION_GP(cudaMemcpyAsync(idx, d_indices, out->idx_bytes, cudaMemcpyDeviceToDevice, s));
+    if (direct) scratch.take(&src, nv);
   }
-  const uint32_t nv = t.nv;
-  const uint32_t W = d.width;
-  void *nodes = nullptr, *nodes2 = nullptr, *prims = nullptr, *prim_ids = nullptr;
+  const DTree dt{nv, t.ids, t.left, t.right, t.rlo, t.rhi, t.axis, t.whole, t.box};
+  std::vector<uint32_t> lvl{0, 0};
+  uint32_t nn = 0, levels = 0;
   if (nv > 0) {
-    const DTree dt{nv, t.ids, t.left, t.right, t.rlo, t.rhi, t.axis, t.whole, t.nlo, t.nhi};
-    const uint64_t cap = own_box ? 2ull * nv - 1 : std::max<uint64_t>(1, nv - 1);
-    Levels L{};
-    SCION_GP(pool.get(&L.rad, cap));
-    SCION_GP(pool.get(&L.nk, cap));
-    SCION_GP(pool.get(&L.kfirst, cap));
-    SCION_GP(pool.get(&L.cnt, cap));
-    SCION_GP(pool.get(&L.off, cap));
-    SCION_GP(pool.get(&L.tiles, (cap + kScanTile - 1) / kScanTile));
-    SCION_GP(pool.get(&L.total, 1));
-    if (!own_box) {
-      SCION_GP(pool.get(&L.wchild, 8 * cap));
-      SCION_GP(pool.get(&L.wn, cap));
-    }
-    // levels, breadth first from the root (logical node 0)
-    const uint32_t root = 0;
-    SCION_GP(cudaMemcpyAsync(L.rad, &root, sizeof(uint32_t), cudaMemcpyHostToDevice, s));
-    std::vector<uint32_t> lvl{0, 1};  // level k = [lvl[k], lvl[k+1])
-    for (;;) {
-      const uint32_t b = lvl[lvl.size() - 2], m = lvl.back() - b;
-      expand_kernel<<<grid_for(m), kThreads, 0, s>>>(dt, L, b, m, W, own_box ? 1 : 0);
+    L.cap = (uint32_t)std::min<uint64_t>(cap, 0xFFFFFFFFull);
+    SCION_GP(cudaMemsetAsync(L.bad, 0, sizeof(int), s));
+    if (pre) SCION_GP(cudaMemsetAsync(L.starts, 0, nv * sizeof(uint32_t), s));
+    first_level_kernel<<<1, 1, 0, s>>>(L);
+    // a binary tree over n leaves is rarely deeper than 1.6 log2 n; W-wide ones
+    // have log2 W levels of it in one
+    uint32_t log2n = 1;
+    while (log2n < 31 && (1u << log2n) < nv) ++log2n;
+    uint32_t issue = (own_box || W == 2) ? log2n * 8 / 5 + 2 : (W == 4 ? log2n * 4 / 5 + 3 : log2n * 3 / 5 + 3);
+    for (uint32_t k = 0;;) {
+      for (uint32_t q = 0; q < issue; ++q, ++k) {
+        switch (own_box ? 0u : W) {
+          case 0:
+            expand_kernel<0><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            emit_kernel<0><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            break;
+          case 2:
+            expand_kernel<2><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            emit_kernel<2><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            break;
+          case 4:
+            expand_kernel<4><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            emit_kernel<4><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            break;
+          default:
+            expand_kernel<8><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            emit_kernel<8><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            break;
+        }
+      }
       SCION_GP(cudaGetLastError());
-      SCION_GP(exclusive_scan(L.cnt, L.off, m, L.tiles, L.total, s));
-      emit_kernel<<<grid_for(m), kThreads, 0, s>>>(dt, L, b, m, own_box ? 1 : 0);
-      SCION_GP(cudaGetLastError());
-      uint32_t next = 0;
-      SCION_GP(cudaMemcpyAsync(&next, L.total, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+      lvl.resize(k + 2);
+      SCION_GP(cudaMemcpyAsync(lvl.data(), L.lvl, (k + 2) * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
       SCION_GP(cudaStreamSynchronize(s));
-      if (next == 0) break;
-      if (lvl.back() + (uint64_t)next > cap) {
-        *err = "GPU packer: level sizes exceed the node count";
+      if (lvl[k + 1] == lvl[k]) break;  // the last level issued placed no further nodes
+      issue = 8;
+      if (k + issue + 2 > kMaxLevels) {
+        *err = "GPU packer: the tree has too many levels";
         return SCION_ERR_CUDA;
       }
-      lvl.push_back(lvl.back() + next);
     }
-    const uint32_t nn = lvl.back();
-    const uint32_t levels = (uint32_t)lvl.size() - 1;
+    nn = lvl.back();
+    while (lvl.size() > 2 && lvl[lvl.size() - 2] == nn) lvl.pop_back();
+    levels = (uint32_t)lvl.size() - 1;
     if (own_box && prec_is_world_grid(d.box_prec) && nn >= kQMaxNodes) {
       *err = "too many nodes for the quantised own-box node";
       return SCION_ERR_UNSUPPORTED_LAYOUT;
@@ -561,118 +724,115 @@ scion_status gpu_pack(const LbvhTree &t, const float *d_verts, uint64_t n_verts,
       *err = "too many nodes";
       return SCION_ERR_INVALID_ARG;
     }
-    // physical positions
-    uint32_t *pos = nullptr;
-    SCION_GP(pool.get(&pos, nn));
-    if (d.order == ORDER_BFS) {
-      iota_kernel<<<grid_for(nn), kThreads, 0, s>>>(pos, nn);
+  }
+  // sizes of the result, and its one allocation
+  OwnArgs oa{};
+  uint32_t stride = 0, ref_bytes = 0;
+  if (own_box) {
+    oa.prec = d.box_prec;
+    oa.soa = d.box_layout;
+    oa.cref = d.child_ref;
+    const bool soa = d.box_layout == LAYOUT_SOA, a16 = d.align == 16;
+    if (oa.prec == PREC_F32) {
+      stride = soa ? (a16 ? 32u : kBinBoxBytes) : kBinNodeBytes;
+      ref_bytes = soa ? kBinRefBytes : 0u;
+    } else if (oa.prec == PREC_Q16) {
+      stride = soa ? (a16 ? 16u : kQBoxBytes) : 16u;
+      ref_bytes = soa ? 4u : 0u;
     } else {
-      const int group = d.child_ref == REF_INDIRECT ? 1 : 0;
-      uint32_t *size = nullptr, *base = nullptr;
-      SCION_GP(pool.get(&size, nn));
+      stride = a16 ? 16u : kQBoxBytes;
+    }
+    oa.stride = stride;
+  } else {
+    stride = wide_node_stride(W, d.box_prec, d.child_ref);
+  }
+  const uint64_t entries = nv;  // every valid triangle is in one leaf
+  Arena block;
+  uint8_t *nodes = nullptr, *nodes2 = nullptr;
+  float4 *prims = nullptr, *verts4 = nullptr;
+  uint32_t *prim_ids = nullptr, *idx = nullptr;
+  for (int pass = 0; pass < 2; ++pass) {
+    if (pass) SCION_GP(block.commit());
+    if (nn) block.take(&nodes, (uint64_t)nn * stride);
+    if (nn && ref_bytes) block.take(&nodes2, (uint64_t)nn * ref_bytes);
+    if (entries && direct) block.take(&prims, 3 * entries);
+    if (entries && !direct) block.take(&prim_ids, entries);
+    if (n_verts) block.take(&verts4, n_verts);
+    if (d_indices && n_tris) block.take(&idx, 3 * n_tris);
+    block.take(&out->scratch, kBvhScratchWords);
+  }
+  SCION_GP(cudaMemsetAsync(out->scratch, 0, kBvhScratchWords * sizeof(uint32_t), s));
+  // vertex / index tables (indirect triangles and the backward pass use them)
+  if (n_verts > 0) verts4_kernel<<<grid_for(n_verts), kThreads, 0, s>>>(d_verts, n_verts, verts4);
+  SCION_GP(cudaGetLastError());
+  if (idx) SCION_GP(cudaMemcpyAsync(idx, d_indices, 3 * n_tris * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
+  out->root_ref = kEmptyRef;
+  if (nv > 0) {
+    // physical positions
+    if (!dfs) {
+      iota_kernel<<<grid_for(nn), kThreads, 0, s>>>(pos, nn);
+    } else if (pre) {
+      SCION_GP(exclusive_scan(L.starts, L.starts, nv, tiles, total, s));
+      preorder_kernel<<<grid_for(nn), kThreads, 0, s>>>(dt, L, pos, nn);
+    } else {
       for (uint32_t k = levels; k-- > 0;)
         size_kernel<<<grid_for(lvl[k + 1] - lvl[k]), kThreads, 0, s>>>(L, size, lvl[k], lvl[k + 1] - lvl[k]);
-      const uint32_t zero_one[2] = {0u, 1u};
-      SCION_GP(cudaMemcpyAsync(pos, &zero_one[0], sizeof(uint32_t), cudaMemcpyHostToDevice, s));
-      if (group) {
-        SCION_GP(pool.get(&base, nn));
-        SCION_GP(cudaMemcpyAsync(base, &zero_one[1], sizeof(uint32_t), cudaMemcpyHostToDevice, s));
-      }
+      root_place_kernel<<<1, 1, 0, s>>>(pos, base);
       for (uint32_t k = 0; k + 1 < levels; ++k)
         place_kernel<<<grid_for(lvl[k + 1] - lvl[k]), kThreads, 0, s>>>(L, size, pos, base, lvl[k],
-                                                                        lvl[k + 1] - lvl[k], group);
-      // the host values above are read by the copies before this returns
-      SCION_GP(cudaStreamSynchronize(s));
+                                                                        lvl[k + 1] - lvl[k]);
     }
     SCION_GP(cudaGetLastError());
     // leaf entries: counts in physical order, prefix sums
-    uint32_t *pbase = nullptr;
-    SCION_GP(pool.get(&pbase, nn));
-    leaf_count_kernel<<<grid_for(nn), kThreads, 0, s>>>(dt, L, pos, nn, own_box ? 1 : 0, pbase);
-    SCION_GP(cudaGetLastError());
-    SCION_GP(exclusive_scan(pbase, pbase, nn, L.tiles, L.total, s));
-    uint32_t entries = 0;
-    SCION_GP(cudaMemcpyAsync(&entries, L.total, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    SCION_GP(cudaStreamSynchronize(s));
-    // buffers
-    PrimOut po{d_verts, d_indices, nullptr, nullptr};
-    if (d.prim_ref == REF_DIRECT) {
-      float *pd = nullptr;
-      SCION_GP(pool.get(&pd, 12 * (size_t)entries));
-      po.direct = pd;
-      prims = pd;
-      out->prim_direct_bytes = 48ull * entries;
-    } else {
-      uint32_t *pi = nullptr;
-      SCION_GP(pool.get(&pi, entries));
-      po.ids = pi;
-      prim_ids = pi;
-      out->prim_id_bytes = 4ull * entries;
+    switch (own_box ? 0u : W) {
+      case 0: leaf_count_kernel<0><<<grid_for(nn), kThreads, 0, s>>>(dt, L, pos, nn, pbase); break;
+      case 2: leaf_count_kernel<2><<<grid_for(nn), kThreads, 0, s>>>(dt, L, pos, nn, pbase); break;
+      case 4: leaf_count_kernel<4><<<grid_for(nn), kThreads, 0, s>>>(dt, L, pos, nn, pbase); break;
+      default: leaf_count_kernel<8><<<grid_for(nn), kThreads, 0, s>>>(dt, L, pos, nn, pbase); break;
     }
-    int *bad = nullptr;
-    SCION_GP(pool.get(&bad, 1));
-    SCION_GP(cudaMemsetAsync(bad, 0, sizeof(int), s));
+    SCION_GP(cudaGetLastError());
+    SCION_GP(exclusive_scan(pbase, pbase, nn, tiles, total, s));
+    uint32_t *entry = direct ? src : prim_ids;
     if (own_box) {
-      OwnArgs oa{};
-      oa.prec = d.box_prec;
-      oa.soa = d.box_layout;
-      oa.cref = d.child_ref;
-      const bool soa = d.box_layout == LAYOUT_SOA, a16 = d.align == 16;
-      uint32_t ref_bytes = 0;
-      if (oa.prec == PREC_F32) {
-        oa.stride = soa ? (a16 ? 32u : kBinBoxBytes) : kBinNodeBytes;
-        ref_bytes = soa ? kBinRefBytes : 0u;
-      } else if (oa.prec == PREC_Q16) {
-        oa.stride = soa ? (a16 ? 16u : kQBoxBytes) : 16u;
-        ref_bytes = soa ? 4u : 0u;
-      } else {
-        oa.stride = a16 ? 16u : kQBoxBytes;
-      }
       if (prec_is_world_grid(oa.prec)) {
         // world grid over the padded root box, computed by the host codec
-        float rb[6];
-        SCION_GP(cudaMemcpyAsync(rb, t.nlo, 3 * sizeof(float), cudaMemcpyDeviceToHost, s));
-        SCION_GP(cudaMemcpyAsync(rb + 3, t.nhi, 3 * sizeof(float), cudaMemcpyDeviceToHost, s));
-        SCION_GP(cudaStreamSynchronize(s));
         Box3 root_box;
-        for (int a = 0; a < 3; ++a) {
-          root_box.lo[a] = rb[a];
-          root_box.hi[a] = rb[3 + a];
-        }
+        SCION_GP(cudaMemcpyAsync(&root_box, t.box, sizeof(Box3), cudaMemcpyDeviceToHost, s));
+        SCION_GP(cudaStreamSynchronize(s));
         world_frame(oa.prec, padded(root_box), oa.frame, oa.bins_inv);
+        for (int a = 0; a < 3; ++a) oa.inv[a] = reciprocal_pair(oa.prec == PREC_Q16 ? oa.frame[3 + a] : 0.0f);
         for (int k = 0; k < 9; ++k) out->frame[k] = oa.frame[k];
+        // records padded to 16 bytes have words that nothing writes
+        SCION_GP(cudaMemsetAsync(nodes, 0, (uint64_t)nn * stride, s));
+      } else if (stride == 32 && d.box_layout == LAYOUT_SOA) {
+        SCION_GP(cudaMemsetAsync(nodes, 0, (uint64_t)nn * stride, s));
       }
-      out->node_stride = oa.stride;
-      out->node_bytes = (uint64_t)nn * oa.stride;
-      SCION_GP(pool.get(reinterpret_cast<uint8_t **>(&nodes), out->node_bytes));
-      SCION_GP(cudaMemsetAsync(nodes, 0, out->node_bytes, s));
-      if (ref_bytes) {
-        out->node2_bytes = (uint64_t)nn * ref_bytes;
-        SCION_GP(pool.get(reinterpret_cast<uint8_t **>(&nodes2), out->node2_bytes));
-        SCION_GP(cudaMemsetAsync(nodes2, 0, out->node2_bytes, s));
-      }
-      encode_own_kernel<<<grid_for(nn), kThreads, 0, s>>>(dt, L, pos, pbase, nn, oa, static_cast<uint8_t *>(nodes),
-                                                           static_cast<uint8_t *>(nodes2), po, bad);
+      encode_own_kernel<<<grid_for(nn), kThreads, 0, s>>>(dt, L, pos, pbase, nn, oa, nodes, nodes2, entry, L.bad);
       out->root_ref = 0;
       out->depth = levels;
       out->stack_need = levels;
     } else {
-      WideArgs wa{W, d.box_prec, d.box_layout, d.child_ref, wide_node_stride(W, d.box_prec, d.child_ref),
-                  wide_ref_offset(W, d.box_prec)};
-      out->node_stride = wa.stride;
-      out->node_bytes = (uint64_t)nn * wa.stride;
-      SCION_GP(pool.get(reinterpret_cast<uint8_t **>(&nodes), out->node_bytes));
-      SCION_GP(cudaMemsetAsync(nodes, 0, out->node_bytes, s));
-      encode_wide_kernel<<<grid_for(nn), kThreads, 0, s>>>(dt, L, pos, pbase, nn, wa, static_cast<uint8_t *>(nodes),
-                                                            po, bad);
+      const uint32_t words = stride / 4;
+      switch (W) {
+        case 2: encode_wide<2>(d.box_prec, dt, L, pos, pbase, nn, d.box_layout, d.child_ref, words, nodes, entry, L.bad, s); break;
+        case 4: encode_wide<4>(d.box_prec, dt, L, pos, pbase, nn, d.box_layout, d.child_ref, words, nodes, entry, L.bad, s); break;
+        default: encode_wide<8>(d.box_prec, dt, L, pos, pbase, nn, d.box_layout, d.child_ref, words, nodes, entry, L.bad, s); break;
+      }
       out->root_ref = ref_interior(0);
       out->depth = levels;
       out->stack_need = (W - 1) * levels + 1;
     }
     SCION_GP(cudaGetLastError());
+    entries_kernel<<<grid_for(entries), kThreads, 0, s>>>(EntryOut{d_verts, d_indices, t.ids, prims, entry},
+                                                          (uint32_t)entries);
+    SCION_GP(cudaGetLastError());
     int hbad = 0;
-    SCION_GP(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+    SCION_GP(cudaMemcpyAsync(&hbad, L.bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     SCION_GP(cudaStreamSynchronize(s));
+    if (hbad & 8) {
+      *err = "GPU packer: level sizes exceed the node count";
+      return SCION_ERR_CUDA;
+    }
     if (hbad & 1) {
       *err = own_box ? "node order violates the child reference encoding" : "siblings not contiguous";
       return SCION_ERR_UNSUPPORTED_LAYOUT;
@@ -685,26 +845,27 @@ scion_status gpu_pack(const LbvhTree &t, const float *d_verts, uint64_t n_verts,
       *err = "u8/u16 enclosure";
       return SCION_ERR_BAD_INPUT;
     }
-    out->n_nodes = nn;
-    out->n_leaf_entries = entries;
   } else {
-    out->root_ref = kEmptyRef;
+    SCION_GP(cudaStreamSynchronize(s));
   }
-  SCION_GP(cudaEventRecord(ev1, s));
-  SCION_GP(cudaStreamSynchronize(s));
-  float ms = 0.f;
-  SCION_GP(cudaEventElapsedTime(&ms, ev0, ev1));
-  out->pack_ms = ms;
 #undef SCION_GP
-  // hand the result buffers to the caller
+  out->n_nodes = nn;
+  out->n_leaf_entries = (uint32_t)entries;
+  out->node_stride = stride;
+  out->node_bytes = (uint64_t)nn * stride;
+  out->node2_bytes = (uint64_t)nn * ref_bytes;
+  out->prim_direct_bytes = direct ? 48ull * entries : 0;
+  out->prim_id_bytes = direct ? 0 : 4ull * entries;
+  out->vert_bytes = n_verts * sizeof(float4);
+  out->idx_bytes = d_indices ? 3 * n_tris * sizeof(uint32_t) : 0;
   out->nodes = nodes;
   out->nodes2 = nodes2;
   out->prims = prims;
   out->prim_ids = prim_ids;
   out->verts4 = verts4;
   out->idx = idx;
-  for (void *p : {nodes, nodes2, prims, prim_ids, static_cast<void *>(verts4), static_cast<void *>(idx)})
-    if (p) pool.release(p);
+  out->block = block.release();  // the caller's now
+  out->pack_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
   return SCION_OK;
 }
 

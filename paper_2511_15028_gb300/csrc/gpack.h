@@ -15,22 +15,29 @@
 
 namespace scion {
 
-// A packed BVH in device memory. The buffers belong to the caller once
-// gpu_pack returns SCION_OK (cudaFree each); on error gpu_pack frees them.
+// Words of a BVH's own device scratch: status words, then the counters of the
+// streams that trace it.
+constexpr uint32_t kBvhStreamSlots = 64;
+constexpr uint32_t kBvhScratchWords = 4 + 4 * kBvhStreamSlots;
+
+// A packed BVH in device memory: parts of one allocation, `block`, which
+// belongs to the caller once gpu_pack returns SCION_OK (cudaFree); on error
+// gpu_pack frees it. scratch: kBvhScratchWords zeroed words.
 struct DevicePacked {
+  void *block = nullptr;
   void *nodes = nullptr, *nodes2 = nullptr, *prims = nullptr, *prim_ids = nullptr;
   void *verts4 = nullptr, *idx = nullptr;
+  uint32_t *scratch = nullptr;
   uint64_t node_bytes = 0, node2_bytes = 0, prim_direct_bytes = 0, prim_id_bytes = 0, vert_bytes = 0,
            idx_bytes = 0;
   uint32_t n_nodes = 0, node_stride = 0, n_leaf_entries = 0, root_ref = kEmptyRef, depth = 0, stack_need = 0;
   float frame[9] = {};
-  double pack_ms = 0.0;  // device time of the packing kernels
+  double pack_ms = 0.0;  // wall time of the packing
 };
 
-// Whether every index of the device array d_indices (u32[n_tris][3]) is
-// below n_verts, checked on the GPU (before any kernel reads through them).
-scion_status gpu_indices_in_range(const uint32_t *d_indices, uint64_t n_tris, uint64_t n_verts, cudaStream_t stream,
-                                  bool *ok, std::string *err);
+// Enqueues the check that every index of the device array d_indices
+// (u32[n_tris][3]) is below n_verts; an index that is not sets *d_bad.
+void launch_index_check(const uint32_t *d_indices, uint64_t n_tris, uint64_t n_verts, int *d_bad, cudaStream_t stream);
 
 // Layouts gpu_pack builds: every width, box precision, box layout and child
 // and primitive reference of the children-in-parent nodes and of the

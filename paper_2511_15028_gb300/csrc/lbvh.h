@@ -21,31 +21,65 @@
 
 namespace scion {
 
+// One device allocation cut into arrays: take every array (which only adds up
+// sizes), commit, take them again in the same order (which gives addresses).
+// cudaMalloc and cudaFree of a few MB cost 35 us each here, of hundreds of MB
+// 50 and 200 us: more than most kernels of a build. commit(stream) allocates
+// scratch for the duration of a call on that stream, from a memory pool of the
+// library's own that keeps up to kScratchKept bytes per device between calls
+// (the driver gives the rest back, and hands the pool's memory to any thread
+// or stream in order); commit() allocates a result with cudaMalloc. Freed with
+// the object unless released.
+constexpr uint64_t kScratchKept = 512ull << 20;
+class Arena {
+ public:
+  Arena() = default;
+  Arena(const Arena &) = delete;
+  Arena &operator=(const Arena &) = delete;
+  ~Arena();
+  template <typename T>
+  void take(T **p, uint64_t count) {
+    if (base_) *p = reinterpret_cast<T *>(base_ + used_);
+    used_ += (count * sizeof(T) + 255) & ~255ull;
+  }
+  cudaError_t commit();
+  cudaError_t commit(cudaStream_t stream);
+  void *release() {  // of a commit() without a stream
+    void *q = base_;
+    base_ = nullptr;
+    return q;
+  }
+
+ private:
+  char *base_ = nullptr;
+  uint64_t used_ = 0;
+  bool pooled_ = false;
+  cudaStream_t stream_ = nullptr;
+};
+
 // The logical BVH2 as the GPU builds it, left in device memory: the binary
 // radix tree over the nv valid triangles in Morton order. Interior node i in
 // [0, nv-2] has children left[i], right[i]; node ids >= nv-1 are radix
 // leaves (leaf k = node nv-1+k holds the sorted triangle ids[k]). An
 // interior node with whole[i] = 1 is a logical leaf over the sorted
 // triangles rlo[i]..rhi[i]; the logical tree is what is reachable from node
-// 0 without entering such a node. Boxes nlo/nhi: 3 floats per node (2nv-1
-// nodes). Node 0 is the root (a radix leaf when nv = 1). Owns its device
+// 0 without entering such a node. Boxes: one per node (2nv-1 nodes), 8-byte
+// aligned. Node 0 is the root (a radix leaf when nv = 1). Owns its device
 // memory; freed with the object.
 struct LbvhTree {
   uint32_t nv = 0;
   const uint32_t *ids = nullptr;
   const uint32_t *left = nullptr, *right = nullptr, *rlo = nullptr, *rhi = nullptr;
   const uint8_t *axis = nullptr, *whole = nullptr;
-  const float *nlo = nullptr, *nhi = nullptr;
+  const Box3 *box = nullptr;
   double gpu_ms = 0.0;  // device time of the build kernels
-  std::vector<void *> owned;
-  LbvhTree() = default;
-  LbvhTree(const LbvhTree &) = delete;
-  LbvhTree &operator=(const LbvhTree &) = delete;
-  ~LbvhTree();
+  Arena memory;
 };
 
 // Build from device vertex (float[n_verts][3]) and optional device index
-// (u32[n_tris][3]) arrays. Triangles with a non-finite vertex are left out.
+// (u32[n_tris][3]) arrays. Triangles with a non-finite vertex are left out. An
+// index out of range gives INVALID_ARG, found on the GPU before any kernel
+// reads through the indices.
 // Synchronises `stream` before returning.
 scion_status lbvh_build_tree(const float *d_verts, uint64_t n_verts, const uint32_t *d_indices, uint64_t n_tris,
                              uint32_t leaf_max, cudaStream_t stream, LbvhTree *out, std::string *err);
