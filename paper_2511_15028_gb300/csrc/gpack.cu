@@ -16,12 +16,14 @@
 // entry; the nodes are written with the codecs of codec_fast.h, a lane per child
 // of a wide node, and the leaf entries by a thread each.
 //
-// The bounds of the levels stay on the device: the two kernels per level are
-// issued for many levels at once, and the host reads the bounds back only to
-// learn whether there are more. Scratch is one allocation and the result
+// The bounds of the levels stay on the device: one CTA takes the small levels at
+// the top and at the bottom without a launch in between, the large ones take two
+// launches each, all issued at once, and the host reads the bounds back only to
+// learn whether there are more. Opening a node takes one load (LbvhTree::open);
+// a level is a chain of such loads. Scratch is one allocation and the result
 // another. Measured, scion_build_gpu and a frame traced after it: 1.4 M triangles,
-// 1080p, bvh4 f32 6.34 -> 1.77 ms (0.35 of it the trace); 40 K triangles 1.72 ->
-// 0.77 ms. A synchronisation and five launches per level, FP64 areas and pads and
+// 1080p, bvh4 f32 6.34 -> 1.61 ms (0.35 of it the trace); 40 K triangles 1.72 ->
+// 0.69 ms. A synchronisation and five launches per level, FP64 areas and pads and
 // some 30 allocations were three quarters of it.
 #include "gpack.h"
 
@@ -145,6 +147,7 @@ struct DTree {
   const uint32_t *ids, *left, *right, *rlo, *rhi;
   const uint8_t *axis, *whole;
   const Box3 *box;
+  const uint4 *open;
 };
 
 // a logical leaf: a radix leaf, or a subtree kept as one leaf
@@ -184,10 +187,19 @@ __device__ __forceinline__ double box_area_d(const Box3 &b) {
 // kfirst[i] = breadth-first index of the first of them (they are consecutive).
 // For depth-first positions: chain[i] = ancestors whose leaves start at the
 // same sorted triangle, starts[lo] = nodes whose leaves start at lo.
+// Logical nodes are kept with a mark where they are logical leaves.
+constexpr uint32_t kLeafMark = 0x80000000u;  // node numbers stay below 2^28
+__device__ __forceinline__ uint32_t marked(uint32_t c, float open) { return open < 0.0f ? c | kLeafMark : c; }
+__device__ __forceinline__ bool is_leaf(uint32_t y) { return (y & kLeafMark) != 0u; }
+__device__ __forceinline__ uint32_t plain(uint32_t y) { return y & ~kLeafMark; }
+
 constexpr uint32_t kMaxLevels = 512;  // a radix tree over 32-bit keys and positions is at most 64 deep
 constexpr int kLevelGrid = 152 * 4;
+constexpr int kSmallThreads = 1024;
+constexpr uint32_t kSmallLevel = 2 * kSmallThreads;  // a level one CTA takes
 struct Levels {
   uint32_t *lvl;  // level k = nodes [lvl[k], lvl[k + 1])
+  uint32_t *cur;  // the first level that is not done
   uint32_t *rad, *wchild, *nk, *kfirst, *chain, *starts, *tsum;
   uint32_t cap;   // nodes the arrays hold
   int *bad;
@@ -198,45 +210,32 @@ __device__ __forceinline__ uint32_t first_of(const DTree &t, uint32_t x) {
   return x + 1 >= t.nv ? x - (t.nv - 1) : t.rlo[x];
 }
 
-__global__ void first_level_kernel(Levels L) {
-  L.lvl[0] = 0;
-  L.lvl[1] = 1;
-  L.rad[0] = 0;  // the root is logical node 0
-  L.chain[0] = 0;
-  if (L.starts) L.starts[0] = 1;
-}
-
 __device__ __noinline__ double box_area_of(const DTree &t, uint32_t x) { return box_area_d(node_box(t, x)); }
 
-// The children of a wide node with root x: the greedy collapse. Areas are
-// compared in float (relative error at most 5 units of 2^-24: sums of
+// The children (marked) of a wide node with root x: the greedy collapse. Areas
+// are compared in float (relative error at most 5 units of 2^-24: sums of
 // non-negative products); children within 2e-6 of the largest, and areas out
 // of float's range, are compared in double, which is what the host packer
 // compares, so the choice is the same.
 template <int W>
-__device__ __forceinline__ uint32_t collapse(const DTree &t, uint32_t x, uint32_t (&ch)[W]) {
+__device__ __forceinline__ void collapse(const DTree &t, uint32_t x, uint32_t (&ch)[W]) {
   float ar[W];
-  auto area = [&](uint32_t c) {
-    if (lleaf(t, c)) return -1.0f;
-    const Box3 b = node_box(t, c);
-    const float e0 = b.hi[0] - b.lo[0], e1 = b.hi[1] - b.lo[1], e2 = b.hi[2] - b.lo[2];
-    return e0 * e1 + e1 * e2 + e2 * e0;
-  };
 #pragma unroll
   for (int k = 0; k < W; ++k) {
     ch[k] = kEmptyRef;
     ar[k] = -1.0f;
   }
-  if (lleaf(t, x)) {  // only a root can be a leaf: a one-child wide root
+  if (is_leaf(x)) {  // only a root can be a leaf: a one-child wide root
     ch[0] = x;
-    return 1;
+    return;
   }
-  ch[0] = t.left[x];
-  ch[1] = t.right[x];
-  ar[0] = area(ch[0]);
-  ar[1] = area(ch[1]);
-  uint32_t n = 2;
-  while (n < (uint32_t)W) {
+  uint4 o = __ldg(t.open + x);
+  ch[0] = o.x;
+  ch[1] = o.y;
+  ar[0] = __uint_as_float(o.z);
+  ar[1] = __uint_as_float(o.w);
+#pragma unroll
+  for (int n = 2; n < W; ++n) {
     int best = -1;
     float top = -1.0f;
 #pragma unroll
@@ -245,46 +244,136 @@ __device__ __forceinline__ uint32_t collapse(const DTree &t, uint32_t x, uint32_
         top = ar[k];
         best = k;
       }
-    if (best < 0) break;
-    const bool in_range = top > 1e-30f && top < 1e37f;
-    const float near = in_range ? top * (1.0f - 2e-6f) : 0.0f;
-    bool close = !in_range;
+    if (best >= 0) {
+      const bool in_range = top > 1e-30f && top < 1e37f;
+      const float near = in_range ? top * (1.0f - 2e-6f) : 0.0f;
+      bool close = !in_range;
 #pragma unroll
-    for (int k = 0; k < W; ++k) close |= k != best && ar[k] >= near;
-    if (close) {
-      double most = -1.0;
+      for (int k = 0; k < W; ++k) close |= k != best && ar[k] >= near;
+      if (close) {
+        double most = -1.0;
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+          if (ar[k] >= near) {
+            const double d = box_area_of(t, ch[k]);
+            if (d > most) {
+              most = d;
+              best = k;
+            }
+          }
+      }
+      uint32_t c = 0;
 #pragma unroll
       for (int k = 0; k < W; ++k)
-        if (ar[k] >= near) {
-          const double d = box_area_of(t, ch[k]);
-          if (d > most) {
-            most = d;
-            best = k;
-          }
+        if (k == best) c = ch[k];
+      o = __ldg(t.open + c);
+#pragma unroll
+      for (int k = W - 1; k >= 0; --k) {
+        if (k > best + 1) {
+          ch[k] = ch[k > 0 ? k - 1 : 0];
+          ar[k] = ar[k > 0 ? k - 1 : 0];
+        } else if (k == best + 1) {
+          ch[k] = o.y;
+          ar[k] = __uint_as_float(o.w);
+        } else if (k == best) {
+          ch[k] = o.x;
+          ar[k] = __uint_as_float(o.z);
         }
-    }
-    uint32_t c = 0;
-#pragma unroll
-    for (int k = 0; k < W; ++k)
-      if (k == best) c = ch[k];
-    const uint32_t l = t.left[c], r = t.right[c];
-    const float al = area(l), arr = area(r);
-#pragma unroll
-    for (int k = W - 1; k >= 0; --k) {
-      if (k > best + 1) {
-        ch[k] = ch[k > 0 ? k - 1 : 0];
-        ar[k] = ar[k > 0 ? k - 1 : 0];
-      } else if (k == best + 1) {
-        ch[k] = r;
-        ar[k] = arr;
-      } else if (k == best) {
-        ch[k] = l;
-        ar[k] = al;
       }
     }
-    ++n;
   }
-  return n;
+#pragma unroll
+  for (int k = 0; k < W; ++k)
+    if (ch[k] != kEmptyRef) ch[k] = marked(ch[k], ar[k]);
+}
+
+// The physical children of node x (marked logical nodes; W = 0: own-box) in
+// kid, their number returned.
+template <int W>
+__device__ __forceinline__ uint32_t find_children(const DTree &t, const Levels &L, uint32_t i, uint32_t x,
+                                                  uint32_t (&kid)[W == 0 ? 2 : W]) {
+  uint32_t nk = 0;
+  if constexpr (W == 0) {
+    if (!is_leaf(x)) {
+      const uint4 o = __ldg(t.open + x);
+      kid[0] = marked(o.x, __uint_as_float(o.z));
+      kid[1] = marked(o.y, __uint_as_float(o.w));
+      nk = 2;
+    }
+  } else {
+    collapse<W>(t, x, kid);
+#pragma unroll
+    for (int c = 0; c < W; ++c) {
+      L.wchild[(size_t)W * i + c] = kid[c];
+      if (kid[c] != kEmptyRef && !is_leaf(kid[c])) ++nk;
+    }
+  }
+  return nk;
+}
+
+// Node i's children take the indices from kf on.
+template <int W>
+__device__ __forceinline__ void place_children(const DTree &t, const Levels &L, uint32_t i, uint32_t x, uint32_t kf,
+                                               uint32_t nk, const uint32_t (&kid)[W == 0 ? 2 : W]) {
+  L.nk[i] = nk;
+  L.kfirst[i] = kf;
+  if (nk == 0) return;
+  if ((uint64_t)kf + nk > L.cap) {  // cannot be: the arrays hold every node a tree of nv leaves can have
+    atomicOr(L.bad, 8);
+    return;
+  }
+  const uint32_t lo = first_of(t, plain(x)), chain = L.chain[i];
+  uint32_t r = 0;
+#pragma unroll
+  for (int c = 0; c < (W == 0 ? 2 : W); ++c) {
+    const uint32_t y = kid[c];
+    if (W != 0 && (y == kEmptyRef || is_leaf(y))) continue;
+    L.rad[kf + r] = y;
+    const uint32_t cl = first_of(t, plain(y));
+    L.chain[kf + r] = cl == lo ? chain + 1 : 0u;
+    if (L.starts) atomicAdd(L.starts + cl, 1u);
+    ++r;
+  }
+}
+
+// Levels small enough for one CTA, one after the other without a launch in
+// between: from level *cur on while a level has at most `most` nodes. first:
+// sets up the root's level.
+template <int W>
+__global__ void __launch_bounds__(kSmallThreads) small_levels_kernel(DTree t, Levels L, uint32_t most, int first) {
+  __shared__ uint32_t ws[33];
+  if (first) {
+    if (threadIdx.x == 0) {
+      L.lvl[0] = 0;
+      L.lvl[1] = 1;
+      L.rad[0] = lleaf(t, 0) ? kLeafMark : 0u;  // the root is logical node 0
+      L.chain[0] = 0;
+      if (L.starts) L.starts[0] = 1;
+    }
+    __syncthreads();
+  }
+  uint32_t k = first ? 0u : *L.cur, b = L.lvl[k], e = L.lvl[k + 1];
+  while (e > b && e - b <= most && k + 2 < kMaxLevels) {
+    uint32_t next = e;
+    for (uint32_t j0 = b; j0 < e; j0 += kSmallThreads) {
+      const uint32_t i = j0 + threadIdx.x;
+      uint32_t kid[W == 0 ? 2 : W], nk = 0, x = 0;
+      if (i < e) {
+        x = L.rad[i];
+        nk = find_children<W>(t, L, i, x, kid);
+      }
+      uint32_t total;
+      const uint32_t at = block_scan(nk, ws, &total);
+      if (i < e) place_children<W>(t, L, i, x, next + at, nk, kid);
+      next += total;
+    }
+    __syncthreads();  // the next level's nodes are written
+    b = e;
+    e = next;
+    ++k;
+    if (threadIdx.x == 0) L.lvl[k + 1] = e;
+  }
+  if (threadIdx.x == 0) *L.cur = k;
 }
 
 // sum of the block's values, in every thread
@@ -294,28 +383,18 @@ __device__ __forceinline__ uint32_t block_sum(uint32_t x, uint32_t *ws) {
   return total;
 }
 
-// Children of level k's nodes; tsum[tile] = physical children of the tile's
-// nodes (a tile: kThreads nodes). W = 0: own-box nodes.
+// Children of the nodes of level *cur + slot; tsum[tile] = physical children of
+// the tile's nodes (a tile: kThreads nodes).
 template <int W>
-__global__ void __launch_bounds__(kThreads) expand_kernel(DTree t, Levels L, uint32_t k) {
+__global__ void __launch_bounds__(kThreads) expand_kernel(DTree t, Levels L, uint32_t slot) {
   __shared__ uint32_t ws[33];
-  const uint32_t b = L.lvl[k], m = L.lvl[k + 1] - b;
+  const uint32_t k = *L.cur + slot, b = L.lvl[k], m = L.lvl[k + 1] - b;
   for (uint32_t tile = blockIdx.x; tile * kThreads < m; tile += gridDim.x) {
     const uint32_t j = tile * kThreads + threadIdx.x, i = b + j;
     uint32_t nk = 0;
     if (j < m) {
-      const uint32_t x = L.rad[i];
-      if constexpr (W == 0) {
-        nk = lleaf(t, x) ? 0u : 2u;
-      } else {
-        uint32_t ch[W];
-        const uint32_t n = collapse<W>(t, x, ch);
-#pragma unroll
-        for (int c = 0; c < W; ++c) {
-          L.wchild[(size_t)W * i + c] = ch[c];
-          if ((uint32_t)c < n && !lleaf(t, ch[c])) ++nk;
-        }
-      }
+      uint32_t kid[W == 0 ? 2 : W];
+      nk = find_children<W>(t, L, i, L.rad[i], kid);
       L.nk[i] = nk;
     }
     const uint32_t sum = block_sum(nk, ws);
@@ -323,11 +402,11 @@ __global__ void __launch_bounds__(kThreads) expand_kernel(DTree t, Levels L, uin
   }
 }
 
-// Places level k + 1 and hands its nodes their logical nodes.
+// Places the next level and hands its nodes their logical nodes.
 template <int W>
-__global__ void __launch_bounds__(kThreads) emit_kernel(DTree t, Levels L, uint32_t k) {
+__global__ void __launch_bounds__(kThreads) emit_kernel(DTree t, Levels L, uint32_t slot) {
   __shared__ uint32_t ws[33];
-  const uint32_t b = L.lvl[k], e = L.lvl[k + 1], m = e - b;  // e: first index of the next level
+  const uint32_t k = *L.cur + slot, b = L.lvl[k], e = L.lvl[k + 1], m = e - b;
   if (m == 0 && blockIdx.x == 0 && threadIdx.x == 0) L.lvl[k + 2] = e;
   for (uint32_t tile = blockIdx.x; tile * kThreads < m; tile += gridDim.x) {
     uint32_t s = 0;
@@ -339,37 +418,24 @@ __global__ void __launch_bounds__(kThreads) emit_kernel(DTree t, Levels L, uint3
     const uint32_t kf = base + block_scan(nk, ws, &total);
     if ((tile + 1) * kThreads >= m && threadIdx.x == 0) L.lvl[k + 2] = base + total;
     if (j >= m) continue;
-    L.kfirst[i] = kf;
-    if (nk == 0) continue;
-    if ((uint64_t)kf + nk > L.cap) {  // cannot be: the arrays hold every node a tree of nv leaves can have
-      atomicOr(L.bad, 8);
-      continue;
-    }
-    const uint32_t x = L.rad[i], lo = first_of(t, x), chain = L.chain[i];
-    auto give = [&](uint32_t at, uint32_t c) {
-      L.rad[at] = c;
-      const uint32_t cl = first_of(t, c);
-      L.chain[at] = cl == lo ? chain + 1 : 0u;
-      if (L.starts) atomicAdd(L.starts + cl, 1u);
-    };
+    const uint32_t x = L.rad[i];
+    uint32_t kid[W == 0 ? 2 : W] = {};
     if constexpr (W == 0) {
-      give(kf, t.left[x]);
-      give(kf + 1, t.right[x]);
+      if (nk) find_children<0>(t, L, i, x, kid);
     } else {
-      uint32_t r = 0;
 #pragma unroll
-      for (int c = 0; c < W; ++c) {
-        const uint32_t y = L.wchild[(size_t)W * i + c];
-        if (y != kEmptyRef && !lleaf(t, y)) give(kf + r++, y);
-      }
+      for (int c = 0; c < W; ++c) kid[c] = L.wchild[(size_t)W * i + c];
     }
+    place_children<W>(t, L, i, x, kf, nk, kid);
   }
 }
+
+__global__ void advance_kernel(Levels L, uint32_t slots) { *L.cur += slots; }
 
 // depth-first (pre-order) positions: starts scanned
 __global__ void preorder_kernel(DTree t, Levels L, uint32_t *pos, uint32_t n) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    pos[i] = L.starts[first_of(t, L.rad[i])] + L.chain[i];
+    pos[i] = L.starts[first_of(t, plain(L.rad[i]))] + L.chain[i];
 }
 
 // subtree sizes of one level (its children's are known)
@@ -415,16 +481,16 @@ __global__ void leaf_count_kernel(DTree t, const Levels L, const uint32_t *pos, 
     uint32_t c = 0, first, count;
     if constexpr (W == 0) {
       const uint32_t x = L.rad[i];
-      if (lleaf(t, x)) {
-        leaf_range(t, x, first, count);
+      if (is_leaf(x)) {
+        leaf_range(t, plain(x), first, count);
         c = count;
       }
     } else {
 #pragma unroll
       for (int k = 0; k < W; ++k) {
         const uint32_t ch = L.wchild[(size_t)W * i + k];
-        if (ch != kEmptyRef && lleaf(t, ch)) {
-          leaf_range(t, ch, first, count);
+        if (ch != kEmptyRef && is_leaf(ch)) {
+          leaf_range(t, plain(ch), first, count);
           c += count;
         }
       }
@@ -472,8 +538,8 @@ __global__ void encode_own_kernel(DTree t, const Levels L, const uint32_t *pos, 
   const bool quant = prec_is_world_grid(oa.prec);
   int badl = 0;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const uint32_t x = L.rad[i], p = pos[i];
-    const bool leaf = lleaf(t, x);
+    const uint32_t x = plain(L.rad[i]), p = pos[i];
+    const bool leaf = is_leaf(L.rad[i]);
     uint32_t ref, meta, count = 0, first = 0;
     if (leaf) {
       leaf_range(t, x, first, count);
@@ -537,9 +603,9 @@ __global__ void __launch_bounds__(kEncodeThreads) encode_wide_kernel(DTree t, co
     for (uint32_t w = k; w < node_words; w += W) mine[j * kPitch + w] = 0;
     __syncwarp();
     const uint32_t c = in ? L.wchild[(size_t)W * i + k] : kEmptyRef;
-    const bool used = c != kEmptyRef, leaf = used && lleaf(t, c), interior = used && !leaf;
+    const bool used = c != kEmptyRef, leaf = used && is_leaf(c), interior = used && !leaf;
     uint32_t first = 0, count = 0;
-    if (leaf) leaf_range(t, c, first, count);
+    if (leaf) leaf_range(t, plain(c), first, count);
     // leaf entries of the slots before this one
     uint32_t before = count;
 #pragma unroll
@@ -557,7 +623,7 @@ __global__ void __launch_bounds__(kEncodeThreads) encode_wide_kernel(DTree t, co
     if (interior && cref == REF_INDIRECT && cp != first_interior + rank) badl |= 1;
     Box3 b;
     for (int a = 0; a < 3; ++a) b.lo[a] = INFINITY, b.hi[a] = -INFINITY;
-    if (used) b = node_box(t, c);
+    if (used) b = node_box(t, plain(c));
     for (uint32_t q = 0; q < count; ++q) src[at + q] = first + q;
     uint32_t *node = mine + j * kPitch;
     badl |= encode_wide_lane<W, PREC>(b, used && !box_is_empty(b), k, soa, reinterpret_cast<uint8_t *>(node));
@@ -650,6 +716,7 @@ scion_status gpu_pack(const LbvhTree &t, const float *d_verts, uint64_t n_verts,
   for (int pass = 0; pass < 2 && nv > 0; ++pass) {  // sizes, then addresses
     if (pass) SCION_GP(scratch.commit(s));
     scratch.take(&L.lvl, kMaxLevels + 4);
+    scratch.take(&L.cur, 1);
     scratch.take(&L.bad, 1);
     scratch.take(&total, 1);
     scratch.take(&L.rad, cap);
@@ -668,47 +735,67 @@ scion_status gpu_pack(const LbvhTree &t, const float *d_verts, uint64_t n_verts,
     }
     if (direct) scratch.take(&src, nv);
   }
-  const DTree dt{nv, t.ids, t.left, t.right, t.rlo, t.rhi, t.axis, t.whole, t.box};
+  const DTree dt{nv, t.ids, t.left, t.right, t.rlo, t.rhi, t.axis, t.whole, t.box, t.open};
   std::vector<uint32_t> lvl{0, 0};
   uint32_t nn = 0, levels = 0;
   if (nv > 0) {
     L.cap = (uint32_t)std::min<uint64_t>(cap, 0xFFFFFFFFull);
     SCION_GP(cudaMemsetAsync(L.bad, 0, sizeof(int), s));
     if (pre) SCION_GP(cudaMemsetAsync(L.starts, 0, nv * sizeof(uint32_t), s));
-    first_level_kernel<<<1, 1, 0, s>>>(L);
-    // a binary tree over n leaves is rarely deeper than 1.6 log2 n; W-wide ones
-    // have log2 W levels of it in one
-    uint32_t log2n = 1;
-    while (log2n < 31 && (1u << log2n) < nv) ++log2n;
-    uint32_t issue = (own_box || W == 2) ? log2n * 8 / 5 + 2 : (W == 4 ? log2n * 4 / 5 + 3 : log2n * 3 / 5 + 3);
-    for (uint32_t k = 0;;) {
-      for (uint32_t q = 0; q < issue; ++q, ++k) {
-        switch (own_box ? 0u : W) {
+    // small levels at the top in one CTA, then the large ones with two launches
+    // each, then the small ones at the bottom; again where that was too few.
+    // Levels grow by 1.8, 3 and 5.6 or more in trees 2, 4 and 8 wide until most
+    // nodes are placed, a few levels after one of nv / kSmallLevel times the size.
+    uint32_t ratio = 0;  // log2 of that, rounded up
+    while (ratio < 31 && ((uint64_t)kSmallLevel << ratio) < nv) ++ratio;
+    uint32_t large = ratio == 0 ? 0u : ((own_box || W == 2) ? ratio * 6 / 5 + 4 : (W == 4 ? ratio * 5 / 8 + 3 : ratio * 2 / 5 + 3));
+    const uint32_t family = own_box ? 0u : W;
+    auto small = [&](uint32_t most, int first) {
+      switch (family) {
+        case 0: small_levels_kernel<0><<<1, kSmallThreads, 0, s>>>(dt, L, most, first); break;
+        case 2: small_levels_kernel<2><<<1, kSmallThreads, 0, s>>>(dt, L, most, first); break;
+        case 4: small_levels_kernel<4><<<1, kSmallThreads, 0, s>>>(dt, L, most, first); break;
+        default: small_levels_kernel<8><<<1, kSmallThreads, 0, s>>>(dt, L, most, first); break;
+      }
+    };
+    for (int first = 1;; first = 0) {
+      if (first) small(kSmallLevel, 1);
+      for (uint32_t q = 0; q < large; ++q) {
+        switch (family) {
           case 0:
-            expand_kernel<0><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
-            emit_kernel<0><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            expand_kernel<0><<<kLevelGrid, kThreads, 0, s>>>(dt, L, q);
+            emit_kernel<0><<<kLevelGrid, kThreads, 0, s>>>(dt, L, q);
             break;
           case 2:
-            expand_kernel<2><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
-            emit_kernel<2><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            expand_kernel<2><<<kLevelGrid, kThreads, 0, s>>>(dt, L, q);
+            emit_kernel<2><<<kLevelGrid, kThreads, 0, s>>>(dt, L, q);
             break;
           case 4:
-            expand_kernel<4><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
-            emit_kernel<4><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            expand_kernel<4><<<kLevelGrid, kThreads, 0, s>>>(dt, L, q);
+            emit_kernel<4><<<kLevelGrid, kThreads, 0, s>>>(dt, L, q);
             break;
           default:
-            expand_kernel<8><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
-            emit_kernel<8><<<kLevelGrid, kThreads, 0, s>>>(dt, L, k);
+            expand_kernel<8><<<kLevelGrid, kThreads, 0, s>>>(dt, L, q);
+            emit_kernel<8><<<kLevelGrid, kThreads, 0, s>>>(dt, L, q);
             break;
         }
       }
+      if (large) {
+        advance_kernel<<<1, 1, 0, s>>>(L, large);
+        small(kSmallLevel, 0);
+      }
       SCION_GP(cudaGetLastError());
-      lvl.resize(k + 2);
-      SCION_GP(cudaMemcpyAsync(lvl.data(), L.lvl, (k + 2) * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+      uint32_t k = 0;
+      lvl.resize(kMaxLevels + 4);
+      SCION_GP(cudaMemcpyAsync(lvl.data(), L.lvl, lvl.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+      SCION_GP(cudaMemcpyAsync(&k, L.cur, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
       SCION_GP(cudaStreamSynchronize(s));
-      if (lvl[k + 1] == lvl[k]) break;  // the last level issued placed no further nodes
-      issue = 8;
-      if (k + issue + 2 > kMaxLevels) {
+      if (lvl[k + 1] == lvl[k]) {  // level k is empty
+        lvl.resize(k + 2);
+        break;
+      }
+      large = 6;
+      if (k + large + 4 > kMaxLevels) {
         *err = "GPU packer: the tree has too many levels";
         return SCION_ERR_CUDA;
       }

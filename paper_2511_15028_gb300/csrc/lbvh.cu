@@ -23,7 +23,7 @@
 //      double.
 // Measured for 1.4 M triangles (ncu, kernels alone): bounds 96 -> 14 us (seven
 // atomics per CTA instead of per warp), sort 283 -> 104, boxes and leaf choice
-// 274 + 832 -> 225 (the costs were in FP64 for every node, and both climbs went
+// 274 + 832 -> 192 (the costs were in FP64 for every node, and both climbs went
 // through L2 from the leaves up). The boxes' least traffic is 0.17 GB, 25 us; the
 // climb above the tiles is a chain of dependent L2 round trips.
 #include "lbvh.h"
@@ -244,6 +244,18 @@ __global__ void __launch_bounds__(kSortThreads) radix_scan_kernel(uint32_t *hist
   if (threadIdx.x == 0) totals[blockIdx.x] = carry;
 }
 
+// Place of a lane's key among its warp's keys of digit d so far, in lane order;
+// counts them.
+__device__ __forceinline__ uint32_t rank_in_warp(uint32_t *cnt, uint32_t d, uint32_t lane) {
+  const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
+  const uint32_t before = __popc(peers & ((1u << lane) - 1u));
+  const uint32_t seen = cnt[d];
+  __syncwarp();
+  if (before == 0) cnt[d] = seen + __popc(peers);
+  __syncwarp();
+  return seen + before;
+}
+
 // 3c. stable scatter of one tile. Warp w holds keys w*512 .. w*512+511, item i
 // of a lane being key i*32 + lane of them.
 __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(const uint32_t *__restrict__ kin,
@@ -269,16 +281,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(const uint3
     val[i] = vin[base + 32 * i];
   }
 #pragma unroll
-  for (int i = 0; i < kSortItems; ++i) {
-    const uint32_t d = (k[i] >> shift) & 255u;
-    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
-    const uint32_t before = __popc(peers & ((1u << lane) - 1u));
-    const uint32_t seen = cnt[warp][d];
-    __syncwarp();
-    if (before == 0) cnt[warp][d] = seen + __popc(peers);
-    __syncwarp();
-    place[i] = seen + before;
-  }
+  for (int i = 0; i < kSortItems; ++i) place[i] = rank_in_warp(cnt[warp], (k[i] >> shift) & 255u, lane);
   __syncthreads();
   // digit t (kSortThreads == kRadix): its warps in order, its place in the
   // tile and in the output
@@ -315,6 +318,59 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(const uint3
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < kSortItems; ++i) vout[out[i]] = buf[i * kSortThreads + t];
+}
+
+// All four passes of a single tile in one launch: twelve launches would be most
+// of the time of a small build.
+__global__ void __launch_bounds__(kSortThreads) radix_tile_sort_kernel(uint32_t *keys, uint32_t *vals) {
+  __shared__ uint32_t cnt[kSortWarps][kRadix];
+  __shared__ uint32_t start[kRadix];
+  __shared__ uint32_t buf[kSortTile];
+  __shared__ uint32_t warp_sums[33];
+  const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5, base = warp * (32 * kSortItems) + lane;
+  uint32_t k[kSortItems], val[kSortItems], place[kSortItems];
+#pragma unroll
+  for (int i = 0; i < kSortItems; ++i) {
+    k[i] = keys[base + 32 * i];
+    val[i] = vals[base + 32 * i];
+  }
+  for (int shift = 0; shift < 32; shift += 8) {
+    for (int i = t; i < kSortWarps * kRadix; i += kSortThreads) (&cnt[0][0])[i] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) place[i] = rank_in_warp(cnt[warp], (k[i] >> shift) & 255u, lane);
+    __syncthreads();
+    uint32_t run = 0, total;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) {
+      const uint32_t x = cnt[w][t];
+      cnt[w][t] = run;
+      run += x;
+    }
+    start[t] = block_exclusive_scan(run, warp_sums, &total);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+      const uint32_t d = (k[i] >> shift) & 255u;
+      place[i] += start[d] + cnt[warp][d];
+      buf[place[i]] = k[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) k[i] = buf[base + 32 * i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) buf[place[i]] = val[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) val[i] = buf[base + 32 * i];
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < kSortItems; ++i) {
+    keys[base + 32 * i] = k[i];
+    vals[base + 32 * i] = val[i];
+  }
 }
 
 // 4. radix tree (Karras 2012). Interior node i in [0, n-2]; leaf k is node
@@ -383,6 +439,7 @@ struct TreeArgs {
   uint32_t lmax;
   float *cost;
   uint8_t *whole;
+  uint4 *open;
   uint32_t *arrived;
 };
 
@@ -444,27 +501,43 @@ __device__ __noinline__ bool leaf_is_cheaper(const TreeArgs &T, const Box3 &b, u
 }
 
 // Box of node p from its children's, and where the subtree is small enough the
-// leaf choice; cl, cr: the children's costs (only read for such a subtree).
-// Returns the node's cost.
-__device__ __forceinline__ float make_node(const TreeArgs &T, uint32_t p, uint32_t l, uint32_t r, uint32_t cnt,
-                                           const Box3 &b0, const Box3 &b1, float cl, float cr, Box3 &b) {
+// leaf choice (the children's costs only count for such a subtree).
+__device__ __forceinline__ float half_area(const Box3 &b) {
+  const float ex = b.hi[0] - b.lo[0], ey = b.hi[1] - b.lo[1], ez = b.hi[2] - b.lo[2];
+  return ex * ey + ey * ez + ez * ex;
+}
+// What a climb carries of a node and keeps of it in shared memory.
+struct Made {
+  Box3 b;
+  float cost;
+  float open;  // half area, or -1: a logical leaf
+};
+__device__ __forceinline__ Made make_node(const TreeArgs &T, uint32_t p, uint32_t l, uint32_t r, uint32_t cnt,
+                                          const Made &ml, const Made &mr) {
+  const Box3 &b0 = ml.b, &b1 = mr.b;
+  Made m;
+  Box3 &b = m.b;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     b.lo[a] = fminf(b0.lo[a], b1.lo[a]);
     b.hi[a] = fmaxf(b0.hi[a], b1.hi[a]);
   }
   store_box(T.box + p, b);
-  if (cnt > T.lmax) return 0.0f;
-  const float a = area_float(b), leaf = a * (float)cnt, split = a + cl + cr;
+  T.open[p] = make_uint4(l, r, __float_as_uint(ml.open), __float_as_uint(mr.open));
+  m.cost = 0.0f;
+  m.open = half_area(b);
+  if (cnt > T.lmax) return m;
+  const float a = area_float(b), leaf = a * (float)cnt, split = a + ml.cost + mr.cost;
   bool w = leaf <= split;
   // the terms of a subtree of at most 16 triangles carry at most 5 + 16 units
   // of 2^-24 each way: 2^-18 leaves a margin of three
   const float near = 3.8147e-06f * split;
   if (!(fabsf(leaf - split) > near) || !(split < 1e37f) || !(a > 1e-30f)) w = leaf_is_cheaper(T, b, cnt, l, r);
   T.whole[p] = w ? 1 : 0;
-  const float c = w ? leaf : split;
-  T.cost[p] = c;
-  return c;
+  m.cost = w ? leaf : split;
+  T.cost[p] = m.cost;
+  if (w) m.open = -1.0f;
+  return m;
 }
 
 // A CTA takes kBoxTile consecutive leaves. A node whose leaves all lie in the
@@ -473,14 +546,14 @@ __device__ __forceinline__ float make_node(const TreeArgs &T, uint32_t p, uint32
 // memory; the rest climb through L2.
 constexpr int kBoxTile = 256;
 __global__ void __launch_bounds__(kBoxTile) boxes_kernel(TreeArgs T) {
-  __shared__ Box3 leaf_box[kBoxTile], node_box[kBoxTile];
-  __shared__ float node_cost[kBoxTile];
+  __shared__ Box3 leaf_box[kBoxTile];
+  __shared__ Made made[kBoxTile];
   __shared__ uint32_t s_left[kBoxTile], s_right[kBoxTile], s_parent[kBoxTile], s_lo[kBoxTile], s_hi[kBoxTile];
   __shared__ uint32_t s_arrived[kBoxTile];
   const uint32_t first_leaf = (uint32_t)(T.n - 1), t = threadIdx.x;
-  for (uint32_t t0 = blockIdx.x * kBoxTile; t0 < (uint32_t)T.n; t0 += gridDim.x * kBoxTile) {
+  const uint32_t t0 = blockIdx.x * kBoxTile;
+  {
     const uint32_t i = t0 + t, t1 = t0 + kBoxTile - 1;
-    __syncthreads();
     s_arrived[t] = 0;
     if (i < first_leaf) {
       s_left[t] = T.left[i];
@@ -490,18 +563,18 @@ __global__ void __launch_bounds__(kBoxTile) boxes_kernel(TreeArgs T) {
       s_hi[t] = T.rhi[i];
     }
     uint32_t p = kNone, node = first_leaf + i;
-    Box3 b{};
+    auto leaf_made = [](const Box3 &b) { return Made{b, area_float(b), -1.0f}; };
+    Made me{};
     if (i < (uint32_t)T.n) {
       const float2 *tb = reinterpret_cast<const float2 *>(T.tbox + T.ids[i]);
-      b = unpack_box(__ldg(tb), __ldg(tb + 1), __ldg(tb + 2));
-      leaf_box[t] = b;
-      store_box(T.box + node, b);
+      me = leaf_made(unpack_box(__ldg(tb), __ldg(tb + 1), __ldg(tb + 2)));
+      leaf_box[t] = me.b;
+      store_box(T.box + node, me.b);
       p = T.parent[node];
     }
-    float cost = area_float(b);
     __syncthreads();
     // at most one thread continues past each node: the second to arrive. It
-    // carries its own node's box and cost and fetches its sibling's.
+    // carries its own node and fetches its sibling.
     while (p != kNone && p - t0 < (uint32_t)kBoxTile && s_lo[p - t0] >= t0 && s_hi[p - t0] <= t1) {
       const uint32_t j = p - t0;
       __threadfence_block();
@@ -511,14 +584,11 @@ __global__ void __launch_bounds__(kBoxTile) boxes_kernel(TreeArgs T) {
       }
       __threadfence_block();
       const uint32_t l = s_left[j], r = s_right[j], cnt = s_hi[j] - s_lo[j] + 1u;
-      const uint32_t sib = l == node ? r : l;
-      const bool sib_leaf = sib >= first_leaf;
-      const Box3 bs = sib_leaf ? leaf_box[sib - first_leaf - t0] : node_box[sib - t0];
-      const float cs = sib_leaf ? area_float(bs) : node_cost[sib - t0];
       const bool left = l == node;
-      cost = make_node(T, p, l, r, cnt, b, bs, left ? cost : cs, left ? cs : cost, b);
-      node_cost[j] = cost;
-      node_box[j] = b;
+      const uint32_t sib = left ? r : l;
+      const Made other = sib >= first_leaf ? leaf_made(leaf_box[sib - first_leaf - t0]) : made[sib - t0];
+      me = make_node(T, p, l, r, cnt, left ? me : other, left ? other : me);
+      made[j] = me;
       node = p;
       p = s_parent[j];
     }
@@ -529,12 +599,18 @@ __global__ void __launch_bounds__(kBoxTile) boxes_kernel(TreeArgs T) {
       __threadfence();
       if (atomicAdd(T.arrived + p, 1u) == 0u) break;
       __threadfence();
-      const uint32_t sib = l == node ? r : l, cnt = hi - lo + 1u;
-      const Box3 bs = load_box_l2(T.box + sib);
-      float cs = 0.0f;
-      if (cnt <= T.lmax) cs = sib >= first_leaf ? area_float(bs) : __ldcg(T.cost + sib);
       const bool left = l == node;
-      cost = make_node(T, p, l, r, cnt, b, bs, left ? cost : cs, left ? cs : cost, b);
+      const uint32_t sib = left ? r : l, cnt = hi - lo + 1u;
+      Made other;
+      other.b = load_box_l2(T.box + sib);
+      if (sib >= first_leaf) {
+        other = leaf_made(other.b);
+      } else {
+        const bool w = __ldcg(T.whole + sib) != 0;
+        other.cost = cnt <= T.lmax ? __ldcg(T.cost + sib) : 0.0f;
+        other.open = w ? -1.0f : half_area(other.b);
+      }
+      me = make_node(T, p, l, r, cnt, left ? me : other, left ? other : me);
       node = p;
       p = up;
     }
@@ -628,6 +704,7 @@ scion_status lbvh_build_tree(const float *d_verts, uint64_t n_verts, const uint3
   uint32_t *keys[2], *vals[2], *hist, *totals, *cb, *nvalid, *left, *right, *parent, *arrived, *rlo, *rhi;
   uint8_t *axis, *whole;
   float *cost;
+  uint4 *open;
   cudaError_t e;
 #define SCION_LB(call)              \
   do {                              \
@@ -656,6 +733,7 @@ scion_status lbvh_build_tree(const float *d_verts, uint64_t n_verts, const uint3
     mem.take(&parent, nn_max);
     mem.take(&arrived, n);
     mem.take(&cost, n);
+    mem.take(&open, n);
   }
   nvalid = cb + 6;
   int *bad_index = reinterpret_cast<int *>(cb + 7);
@@ -684,7 +762,11 @@ scion_status lbvh_build_tree(const float *d_verts, uint64_t n_verts, const uint3
                                                bad_index);
   SCION_LB(cudaGetLastError());
   int cur = 0;
-  for (int shift = 0; shift < 32; shift += 8) {
+  if (tiles == 1) {
+    radix_tile_sort_kernel<<<1, kSortThreads, 0, s>>>(keys[0], vals[0]);
+    SCION_LB(cudaGetLastError());
+  }
+  for (int shift = 0; shift < 32 && tiles > 1; shift += 8) {
     radix_hist_kernel<<<tiles, kSortThreads, 0, s>>>(keys[cur], shift, hist, tiles);
     radix_scan_kernel<<<kRadix, kSortThreads, 0, s>>>(hist, tiles, totals);
     radix_scatter_kernel<<<tiles, kSortThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], shift,
@@ -716,8 +798,9 @@ scion_status lbvh_build_tree(const float *d_verts, uint64_t n_verts, const uint3
     SCION_LB(cudaGetLastError());
   }
   const TreeArgs T{(int)nv, vals[cur], left, right, parent, rlo, rhi, tbox, box, leaf_max ? leaf_max : 1u,
-                   cost,    whole,     arrived};
-  boxes_kernel<<<grid_for(nv, kBoxTile), kBoxTile, 0, s>>>(T);
+                   cost,    whole,     open, arrived};
+  // a CTA per tile: one that climbs through L2 must not hold up another tile
+  boxes_kernel<<<(nv + kBoxTile - 1) / kBoxTile, kBoxTile, 0, s>>>(T);
   SCION_LB(cudaGetLastError());
   SCION_LB(cudaEventRecord(ev1, s));
   SCION_LB(cudaStreamSynchronize(s));
@@ -733,6 +816,7 @@ scion_status lbvh_build_tree(const float *d_verts, uint64_t n_verts, const uint3
   out->axis = axis;
   out->whole = whole;
   out->box = box;
+  out->open = open;
   return SCION_OK;
 }
 

@@ -63,7 +63,9 @@ class Arena {
 // leaves (leaf k = node nv-1+k holds the sorted triangle ids[k]). An
 // interior node with whole[i] = 1 is a logical leaf over the sorted
 // triangles rlo[i]..rhi[i]; the logical tree is what is reachable from node
-// 0 without entering such a node. Boxes: one per node (2nv-1 nodes), 8-byte
+// 0 without entering such a node. open[i] of an interior node that is not a
+// leaf: its children and their half areas, -1 for a logical leaf: what opening
+// the node takes, in one load. Boxes: one per node (2nv-1 nodes), 8-byte
 // aligned. Node 0 is the root (a radix leaf when nv = 1). Owns its device
 // memory; freed with the object.
 struct LbvhTree {
@@ -72,6 +74,7 @@ struct LbvhTree {
   const uint32_t *left = nullptr, *right = nullptr, *rlo = nullptr, *rhi = nullptr;
   const uint8_t *axis = nullptr, *whole = nullptr;
   const Box3 *box = nullptr;
+  const uint4 *open = nullptr;
   double gpu_ms = 0.0;  // device time of the build kernels
   Arena memory;
 };
