@@ -1058,7 +1058,8 @@ struct scion_batch_s {
   uint32_t *d_counters = nullptr;   // u64 work counter + u32 exit counter
   uint32_t n_scenes = 0;            // scenes in the multi-family launch
   unsigned long long total = 0;     // padded global ray count
-  uint32_t threads = 256, smem_stack = 16, grid = 0;
+  uint32_t threads = 256, smem_stack = 16, grid = 0, chunk = 32;
+  BatchKernel kernel = nullptr;     // of the scenes' one family, or of several
   // scenes whose layout the batched kernel does not handle: plain launches
   std::vector<scion_bvh> rest_bvh;
   std::vector<const scion_ray *> rest_rays;
@@ -1077,6 +1078,9 @@ scion_status scion_batch_create(const scion_bvh *bvhs, const scion_ray *const *d
   if (!bt) return SCION_ERR_OOM;
   std::vector<BatchScene> table;
   unsigned long long total = 0;
+  int family = -1;
+  bool one_family = true;
+  scion_bvh first = nullptr;
   if (per_scene) {
     bt->threads = per_scene[0].threads_per_block ? per_scene[0].threads_per_block : 256;
     bt->smem_stack = per_scene[0].smem_stack ? per_scene[0].smem_stack : 16;
@@ -1134,6 +1138,9 @@ scion_status scion_batch_create(const scion_bvh *bvhs, const scion_ray *const *d
     a.status = b->d_scratch + 3;
     sc.begin = total;
     sc.family = (uint32_t)fam;
+    one_family = one_family && (table.empty() || fam == family);
+    family = fam;
+    if (!first) first = b;
     total += (n[i] + kBatchUnit - 1) / kBatchUnit * kBatchUnit;
     table.push_back(sc);
   }
@@ -1149,21 +1156,28 @@ scion_status scion_batch_create(const scion_bvh *bvhs, const scion_ray *const *d
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess && !table.empty()) {
+    bt->kernel = batched_kernel_for(one_family ? family : -1);
+    if (one_family) bt->smem_stack = stack_entries(first, bt->smem_stack);  // a ring as in the plain kernels
     const size_t smem = (size_t)bt->threads * bt->smem_stack * sizeof(uint2);
     int nb = 0;
     int dev = current_device();
-    const scion_status so = ensure_smem_optin(batched_kernel_ptr(), smem, dev);
+    const scion_status so = ensure_smem_optin((const void *)bt->kernel, smem, dev);
     if (so != SCION_OK) {
       if (bt->d_counters) cudaFree(bt->d_counters);
       if (bt->d_scenes) cudaFree(bt->d_scenes);
       delete bt;
       return so;
     }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batched_kernel_ptr(), (int)bt->threads, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void *)bt->kernel, (int)bt->threads, smem);
     // one unit per warp at a time: more CTAs than units would only idle
-    const uint64_t per_cta = (uint64_t)kBatchUnit * (bt->threads / 32);
-    const uint64_t want = ((uint64_t)total + per_cta - 1) / per_cta;
-    bt->grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)std::max(nb, 1) * device_sms(dev), want));
+    const uint64_t resident = (uint64_t)std::max(nb, 1) * device_sms(dev), warps = bt->threads / 32;
+    TraceArgs whole{};
+    whole.n_work = total;
+    if (one_family) small_launch(whole, resident * warps);
+    else whole.chunk = kBatchUnit;
+    bt->chunk = whole.chunk;
+    const uint64_t units = total / bt->chunk;
+    bt->grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(resident, (units + warps - 1) / warps));
   }
   if (e != cudaSuccess) {
     if (bt->d_counters) cudaFree(bt->d_counters);
@@ -1179,10 +1193,13 @@ scion_status scion_batch_create(const scion_bvh *bvhs, const scion_ray *const *d
 scion_status scion_batch_launch(scion_batch bt, scion_stream stream) {
   if (!bt) return SCION_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (bt->n_scenes > 0)
-    SCION_CUDA(launch_batched(bt->d_scenes, bt->n_scenes, bt->total,
-                              reinterpret_cast<unsigned long long *>(bt->d_counters), bt->d_counters + 2,
-                              bt->smem_stack, bt->threads, bt->grid, s));
+  if (bt->n_scenes > 0) {
+    BatchArgs ba{bt->d_scenes, bt->total, reinterpret_cast<unsigned long long *>(bt->d_counters), bt->d_counters + 2,
+                 bt->n_scenes, bt->chunk, bt->smem_stack};
+    void *args[] = {&ba};
+    SCION_CUDA(cudaLaunchKernel((const void *)bt->kernel, dim3(bt->grid), dim3(bt->threads), args,
+                                (size_t)bt->threads * bt->smem_stack * sizeof(uint2), s));
+  }
   for (size_t i = 0; i < bt->rest_bvh.size(); ++i) {
     scion_status st = launch_trace(bt->rest_bvh[i], bt->rest_rays[i], bt->rest_n[i], bt->rest_hits[i],
                                    &bt->rest_params[i], s, kQueryClosest);

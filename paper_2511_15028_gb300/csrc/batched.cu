@@ -1,15 +1,26 @@
 // Many scenes in one persistent launch (closest hit).
 //
 // Every scene keeps its own BVH and layout. Its rays occupy a range of a global
-// index space padded to multiples of 32, so each 32-ray unit a warp takes from
-// the global counter belongs to exactly one scene; the warp dispatches on that
-// scene's node family with a warp-uniform switch over the traversal template
-// instances and stays with the scene while the next units it takes belong to
-// it. The scene's fetch mode holds: warp batches (each lane traces its ray of
-// the unit to completion, then the warp takes the next unit) or warp refill
-// (idle lanes take the next rays as soon as at least rays_per_fetch of them
-// are idle, from a new unit when the current one is used up; a unit of
-// another scene ends the refill, the warp finishes its rays and moves on).
+// index space padded to multiples of 32, so each unit a warp takes from the
+// global counter belongs to exactly one scene; the warp stays with the scene
+// while the next units it takes belong to it. The scene's fetch mode holds:
+// warp batches (each lane traces its ray of the unit to completion, then the
+// warp takes the next unit) or warp refill (idle lanes take the next rays as
+// soon as at least rays_per_fetch of them are idle, from a new unit when the
+// current one is used up; a unit of another scene ends the refill, the warp
+// finishes its rays and moves on).
+//
+// Where all scenes have one node family, as an autotuned batch usually does, a
+// kernel of that family runs (batched_body in batched.cuh, instantiated beside
+// the family's other kernels): its loops are the plain launch's, with the
+// scene's arguments in shared memory. Scenes of several families run in the
+// kernel below, which dispatches with a warp-uniform switch over functions of
+// their own; those spill 200 to 300 bytes under the 64-register cap and read the
+// scene's arguments from global memory, which is why it is not used for both.
+// Measured, 48 scenes of one family (1.6 M rays): bvh4 u8 batches 839 -> 775 us,
+// refill 1,319 -> 847; bvh4 f32 refill 1,342 -> 854; bvh8 u8 1,131 -> 954; bvh2 q16
+// refill 2,511 -> 1,198; 5 small scenes 121 -> 68. One large scene runs within 4 %
+// of its plain launch (refill: twice as long before).
 // The launch allocates nothing and never synchronises the host, so it can be
 // captured in a CUDA graph and replayed; its counters reset themselves.
 #include <cuda_runtime.h>
@@ -154,8 +165,12 @@ __device__ __noinline__ unsigned long long run_scene(const BatchScene &S, unsign
 }
 
 __global__ void __launch_bounds__(kMaxThreadsPerBlock, kMinBlocksPerSm)
-    batched_kernel(const BatchScene *__restrict__ scenes, uint32_t n_scenes, unsigned long long total,
-                   unsigned long long *work, uint32_t *exit_count, uint32_t smem_stack) {
+    batched_kernel(BatchArgs ba) {
+  const BatchScene *__restrict__ scenes = ba.scenes;
+  const uint32_t n_scenes = ba.n_scenes, smem_stack = ba.smem_stack;
+  const unsigned long long total = ba.slots;
+  unsigned long long *const work = ba.work;
+  uint32_t *const exit_count = ba.exit_count;
   extern __shared__ uint2 smem[];
   // scene starts (padded global offsets) for the unit -> scene search
   __shared__ unsigned long long starts[kMaxSharedScenes];
@@ -218,14 +233,18 @@ int batched_family(uint32_t own_box, const scion_layout_desc &d) {
   return -1;
 }
 
-const void *batched_kernel_ptr() { return (const void *)batched_kernel; }
-
-cudaError_t launch_batched(const BatchScene *d_scenes, uint32_t n_scenes, unsigned long long total,
-                           unsigned long long *work, uint32_t *exit_count, uint32_t smem_stack,
-                           uint32_t threads, uint32_t grid, cudaStream_t s) {
-  const size_t smem = (size_t)threads * smem_stack * sizeof(uint2);
-  batched_kernel<<<grid, threads, smem, s>>>(d_scenes, n_scenes, total, work, exit_count, smem_stack);
-  return cudaGetLastError();
+BatchKernel batched_kernel_for(int family) {
+  switch (family) {
+    case kFamilyBin: return batched_own_p0(LAYOUT_AOS);
+    case kFamilyBinQ16: return batched_own_p3(LAYOUT_AOS);
+    case kFamilyW4F32: return batched_w4_p0(LAYOUT_SOA);
+    case kFamilyW4F16: return batched_w4_p1(LAYOUT_SOA);
+    case kFamilyW4U8: return batched_w4_p2(LAYOUT_SOA);
+    case kFamilyW8F16: return batched_w8_p1(LAYOUT_SOA);
+    case kFamilyW8U8: return batched_w8_p2(LAYOUT_AOS);
+    case kFamilyW8U8S: return batched_w8_p2(LAYOUT_SOA);
+    default: return batched_kernel;
+  }
 }
 
 }  // namespace scion

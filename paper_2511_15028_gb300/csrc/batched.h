@@ -36,9 +36,20 @@ struct alignas(16) BatchScene {
 
 // Family of a layout, or -1 if the batched kernel does not handle it.
 int batched_family(uint32_t own_box, const scion_layout_desc &d);
-const void *batched_kernel_ptr();
-cudaError_t launch_batched(const BatchScene *d_scenes, uint32_t n_scenes, unsigned long long total,
-                           unsigned long long *work, uint32_t *exit_count, uint32_t smem_stack,
-                           uint32_t threads, uint32_t grid, cudaStream_t s);
+
+// A batch's launch: `slots` = end of the padded global range, a multiple of 32;
+// chunk: slots a warp takes at a time (32, or a power of two below it in a
+// launch too small to fill the GPU; the kernel for several families takes 32).
+struct BatchArgs {
+  const BatchScene *scenes;
+  unsigned long long slots;
+  unsigned long long *work;
+  uint32_t *exit_count;
+  uint32_t n_scenes, chunk, smem_stack;
+};
+typedef void (*BatchKernel)(BatchArgs);
+
+// The kernel for scenes of one family, or of several (family < 0).
+BatchKernel batched_kernel_for(int family);
 
 }  // namespace scion

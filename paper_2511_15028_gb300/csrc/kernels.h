@@ -1,6 +1,7 @@
 // Kernel table: one persistent traversal kernel per (node codec, query).
 #pragma once
 
+#include "batched.h"
 #include "trace.cuh"
 
 namespace scion {
@@ -47,6 +48,15 @@ TraceKernel cpq_kernels_w8_p2(int soa, int cref, int stats);
 TraceKernel cpq_kernels_w2_p5(int soa, int cref, int stats);
 TraceKernel cpq_kernels_w4_p5(int soa, int cref, int stats);
 TraceKernel cpq_kernels_w8_p5(int soa, int cref, int stats);
+
+// multi-scene kernels of one family
+BatchKernel batched_own_p0(int soa);
+BatchKernel batched_own_p3(int soa);
+BatchKernel batched_w4_p0(int soa);
+BatchKernel batched_w4_p1(int soa);
+BatchKernel batched_w4_p2(int soa);
+BatchKernel batched_w8_p1(int soa);
+BatchKernel batched_w8_p2(int soa);
 
 constexpr int kMaxThreadsPerBlock = 256;
 constexpr uint32_t kMaxRegStack = 4;  // largest register tier of the traversal stack

@@ -2,6 +2,7 @@
 // times with -DSCION_OWN=1 -DSCION_PREC=<0|3|4|6> (own-box node with f32, q16
 // or eq10 boxes, or the shared-slab node), or -DSCION_W=<2|4|8> -DSCION_PREC=<0|1|2|5>, so the families
 // build in parallel.
+#include "batched.cuh"
 #include "cpq.cuh"
 #include "kernels.h"
 
@@ -11,21 +12,23 @@
 namespace scion {
 
 #if defined(SCION_OWN)
-#define SCION_FAMILY_OWN true
+#define SCION_FAMILY_OWN 1
 #define SCION_W 2
 #define SCION_GETTER SCION_CAT(kernels_own_p, SCION_PREC)
 #define SCION_CPQ_GETTER SCION_CAT(cpq_kernels_own_p, SCION_PREC)
+#define SCION_BATCH_GETTER SCION_CAT(batched_own_p, SCION_PREC)
 #else
-#define SCION_FAMILY_OWN false
+#define SCION_FAMILY_OWN 0
 #define SCION_GETTER SCION_CAT(SCION_CAT(SCION_CAT(kernels_w, SCION_W), _p), SCION_PREC)
 #define SCION_CPQ_GETTER SCION_CAT(SCION_CAT(SCION_CAT(cpq_kernels_w, SCION_W), _p), SCION_PREC)
+#define SCION_BATCH_GETTER SCION_CAT(SCION_CAT(SCION_CAT(batched_w, SCION_W), _p), SCION_PREC)
 #endif
 
 // The register tier of the stack spills under the 64-register cap of four
 // CTAs per SM; measured, that costs less than giving up a CTA per SM.
 template <int SOA, int CREF, bool ANY, bool STATS, int REG>
 __global__ void __launch_bounds__(kMaxThreadsPerBlock, kMinBlocksPerSm) trace_kernel(TraceArgs a) {
-  trace_kernel_body<SCION_FAMILY_OWN, SCION_W, SCION_PREC, SOA, CREF, ANY, STATS, REG>(a);
+  trace_kernel_body<SCION_FAMILY_OWN != 0, SCION_W, SCION_PREC, SOA, CREF, ANY, STATS, REG>(a);
 }
 
 // reg: register entries at the top of the stack, 0, 2 or 4 (the counting
@@ -62,7 +65,7 @@ TraceKernel SCION_CPQ_GETTER(int, int, int) { return nullptr; }
 #else
 template <int SOA, int CREF, bool STATS>
 __global__ void __launch_bounds__(kMaxThreadsPerBlock, kMinBlocksPerSm) cpq_kernel(TraceArgs a) {
-  cpq_kernel_body<SCION_FAMILY_OWN, SCION_W, SCION_PREC, SOA, CREF, STATS>(a);
+  cpq_kernel_body<SCION_FAMILY_OWN != 0, SCION_W, SCION_PREC, SOA, CREF, STATS>(a);
 }
 TraceKernel SCION_CPQ_GETTER(int soa, int cref, int stats) {
   static const TraceKernel table[2][2][2] = {
@@ -70,6 +73,25 @@ TraceKernel SCION_CPQ_GETTER(int soa, int cref, int stats) {
       {{cpq_kernel<1, 0, false>, cpq_kernel<1, 0, true>}, {cpq_kernel<1, 1, false>, cpq_kernel<1, 1, true>}}};
   return table[soa & 1][cref & 1][stats & 1];
 }
+#endif
+
+// Multi-scene kernels of the families a batch takes: own-box f32 and q16 (AoS),
+// 4-wide f32, f16 and u8 (SoA), 8-wide f16 (SoA) and u8 (both).
+#if (SCION_FAMILY_OWN && (SCION_PREC == 0 || SCION_PREC == 3)) || \
+    (!SCION_FAMILY_OWN && ((SCION_W == 4 && SCION_PREC <= 2) || (SCION_W == 8 && (SCION_PREC == 1 || SCION_PREC == 2))))
+template <int SOA>
+__global__ void __launch_bounds__(kMaxThreadsPerBlock, kMinBlocksPerSm) batched_kernel_one(BatchArgs ba) {
+  batched_body<SCION_FAMILY_OWN != 0, SCION_W, SCION_PREC, SOA>(ba);
+}
+#if SCION_FAMILY_OWN
+BatchKernel SCION_BATCH_GETTER(int) { return batched_kernel_one<LAYOUT_AOS>; }
+#elif SCION_W == 8 && SCION_PREC == 2
+BatchKernel SCION_BATCH_GETTER(int soa) {
+  return soa ? batched_kernel_one<LAYOUT_SOA> : batched_kernel_one<LAYOUT_AOS>;
+}
+#else
+BatchKernel SCION_BATCH_GETTER(int) { return batched_kernel_one<LAYOUT_SOA>; }
+#endif
 #endif
 
 }  // namespace scion

@@ -193,3 +193,35 @@ def test_batched_every_family_and_fetch_mode(mods, oracle_mod):
             assert scion.scion_get_status(bvhs[i]) == 0
     with pytest.raises(scion.ScionError):  # register stack tiers are for plain launches
         scion.Batch(bvhs[:1], rays[:1], params=[dict(reg_stack=4)])
+
+
+@pytest.mark.parametrize("scale,n_scenes", [(0.002, 3), (0.01, 9), (0.05, 12)])
+@pytest.mark.parametrize("kw", [dict(), dict(box_prec="q16"), dict(width=4, box_layout="soa"),
+                                dict(width=4, box_layout="soa", box_prec="f16"),
+                                dict(width=4, box_layout="soa", box_prec="u8", order="bfs"),
+                                dict(width=8, box_layout="soa", box_prec="f16"), dict(width=8, box_prec="u8"),
+                                dict(width=8, box_layout="soa", box_prec="u8")],
+                         ids=lambda kw: "-".join(str(v) for v in kw.values()) or "pbrt")
+def test_batched_one_family(mods, oracle_mod, kw, scale, n_scenes):
+    """Batches of a single node family (their own kernel), from a few rays (a
+    warp takes less than 32) to several units per warp, with scenes under both
+    fetch modes and a shallow shared stack: hits equal the oracle's, also
+    when launched again."""
+    scion, _ = mods
+    wl = scenes.config4_workload(seed=80, n_scenes=n_scenes, scale=scale)
+    modes = [{}, dict(rays_per_fetch=4), dict(rays_per_fetch=31, ordered_children=2), dict(ordered_children=3)]
+    bvhs = [scion.scion_build(sc.verts, scion.layout(prim_ref="direct" if i % 2 else "indirect", **kw), sc.indices)
+            for i, (sc, _) in enumerate(wl)]
+    rays = [torch.from_numpy(r).cuda() for _, r in wl]
+    for stack in (16, 1):
+        params = [dict(modes[i % 4], smem_stack=stack) for i in range(n_scenes)]
+        batch = scion.Batch(bvhs, rays, params=params)
+        for _ in range(2):
+            for h in batch.hits:
+                h.fill_(-1)
+            hits = batch.launch()
+            torch.cuda.synchronize()
+            for i, (sc, r) in enumerate(wl):
+                exp = oracle_mod.BVH2(sc.triangles()).closest(r)
+                assert scion.split_hits(hits[i]).tobytes() == exp.tobytes(), (i, params[i])
+                assert scion.scion_get_status(bvhs[i]) == 0
