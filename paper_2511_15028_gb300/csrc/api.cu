@@ -273,6 +273,35 @@ TraceKernel pick_cpq_kernel(const scion_bvh b, int stats) {
   return nullptr;
 }
 
+TraceKernel pick_coop_kernel(const scion_bvh b, int query) {
+  const scion_layout_desc &d = b->desc;
+  const int soa = (int)d.box_layout, cref = (int)d.child_ref;
+  if (b->own_box) {
+    switch (d.box_prec) {
+      case PREC_F32: return coop_own_p0(soa, cref, query);
+      case PREC_Q16: return coop_own_p3(soa, cref, query);
+      case PREC_EQ10: return coop_own_p4(soa, cref, query);
+      case PREC_SLAB: return coop_own_p6(soa, cref, query);
+    }
+    return nullptr;
+  }
+  switch (d.width * 10 + d.box_prec) {
+    case 20: return coop_w2_p0(soa, cref, query);
+    case 21: return coop_w2_p1(soa, cref, query);
+    case 22: return coop_w2_p2(soa, cref, query);
+    case 25: return coop_w2_p5(soa, cref, query);
+    case 40: return coop_w4_p0(soa, cref, query);
+    case 41: return coop_w4_p1(soa, cref, query);
+    case 42: return coop_w4_p2(soa, cref, query);
+    case 45: return coop_w4_p5(soa, cref, query);
+    case 80: return coop_w8_p0(soa, cref, query);
+    case 81: return coop_w8_p1(soa, cref, query);
+    case 82: return coop_w8_p2(soa, cref, query);
+    case 85: return coop_w8_p5(soa, cref, query);
+  }
+  return nullptr;
+}
+
 TraceKernel pick_kernel(const scion_bvh b, int query, int stats, uint32_t reg) {
   const scion_layout_desc &d = b->desc;
   const int soa = (int)d.box_layout, cref = (int)d.child_ref;
@@ -476,7 +505,46 @@ struct TraceLaunch {
   uint64_t grid = 0;
   uint32_t ctas_param = 0;  // scion_trace_params.ctas_per_sm (0: from occupancy)
   uint32_t reg_stack = 0;   // register entries at the top of the stack
+  bool coop = false;        // one query per warp
 };
+
+// One query per warp (coop.cuh) instead of one per lane, for launches too small to
+// fill the GPU with lanes. Where the line lies, in queries per resident warp
+// (4,864 on this part), from both kernels measured on trees of 2 K to 1.4 M
+// triangles:
+//  - rays: 4, for 8-wide nodes 6. At 16,000 camera rays 70 -> 37 us (bvh4 f32), 89
+//    -> 55 (bvh2 f32); at 20,000 random rays 46 -> 32 (bvh4, closest), 60 -> 48
+//    (bvh2 q16), 50 -> 26 (bvh8 u8, any hit); even at 20,000 short any-hit rays
+//    in bvh2 q16 (67, 69), 40,000 random ones in bvh4 (50, 50) and 48,000 camera
+//    rays (81, 86).
+//  - points: (log2 of the triangles - 6)^2 / 5, for own-box nodes / 6, 8-wide
+//    nodes / 4: a point in a large tree is long work. 1,000 points in 50 K
+//    triangles 170 -> 42 us, 20,000 in 1.4 M 647 -> 212; even at 30,000 in 2 K
+//    (105, 107), past it at 100,000 in 30 K (425, 487) and at 200,000 in 1.4 M
+//    (1,542, 1,511; bvh8 f16 2,144, 1,645).
+// Only with the default launch shape, stack and step limit, which are parameters of
+// the per-lane kernels, and only for trees that cannot overflow those kernels'
+// stack, so that what they report as an error stays one.
+void use_coop(const scion_bvh b, const scion_trace_params &p, int query, TraceLaunch *L) {
+  if (p.threads_per_block || p.ctas_per_sm || p.max_steps || p.smem_stack || p.reg_stack) return;
+  constexpr uint32_t kEntries = 16, kLaneStack = 64;  // per lane; a warp's stack is 32 times that
+  if (b->stack_need > kLaneStack) return;
+  const uint64_t warps = (uint64_t)device_sms(b->device) * 32;
+  const bool eight = !b->own_box && b->desc.width == 8;
+  uint64_t most = warps * (eight ? 6 : 4);
+  if (query == kQueryPoint) {
+    uint64_t l = 6;
+    while (l < 31 && (1ull << l) < b->n_leaf_entries) ++l;
+    most = std::max<uint64_t>(warps, warps * (l - 6) * (l - 6) / (eight ? 4 : (b->own_box ? 6 : 5)));
+  }
+  if (L->a.n > most) return;
+  const TraceKernel k = pick_coop_kernel(b, query);
+  if (!k) return;
+  L->k = k;
+  L->coop = true;
+  L->a.smem_stack = kEntries;
+  L->smem = (size_t)L->tpb * kEntries * sizeof(uint2);
+}
 
 // Checks and set-up shared by every entry point that launches a traversal or
 // closest point kernel (scion_trace_closest/_any/_stats,
@@ -563,8 +631,10 @@ scion_status prepare_trace(scion_bvh b, const scion_ray *rays, uint64_t n, void 
   a.stats = nullptr;
   a.work = nullptr;
   a.exit_count = nullptr;
+  a.stack_need = b->stack_need;
   L->ctas_param = p.ctas_per_sm;
   L->reg_stack = p.reg_stack;
+  use_coop(b, p, query, L);
   return SCION_OK;
 }
 
@@ -580,7 +650,8 @@ scion_status issue_trace(TraceLaunch &L, cudaStream_t stream, TraceKernel k) {
     if (st != SCION_OK) return st;
   }
   const uint64_t resident = (uint64_t)ctas * device_sms(dev), warps = L.tpb / 32;
-  small_launch(L.a, resident * warps);
+  if (L.coop) L.a.chunk = 1;
+  else small_launch(L.a, resident * warps);
   const uint64_t blocks = (L.a.n_work + L.a.chunk - 1) / L.a.chunk;
   L.grid = std::min<uint64_t>(resident, (blocks + warps - 1) / warps);
   void *args[] = {&L.a};
@@ -598,6 +669,9 @@ scion_status launch_trace(scion_bvh b, const scion_ray *rays, uint64_t n, void *
   if (st != SCION_OK) return st;
   TraceKernel k = L.k;
   if (stats) {
+    L.coop = false;
+    L.a.smem_stack = stack_entries(b, params && params->smem_stack ? params->smem_stack : 16);
+    L.smem = (size_t)L.tpb * L.a.smem_stack * stack_entry_bytes(b, query);
     k = pick_kernel(b, query, 1, 0);
     if (!k) return SCION_ERR_UNSUPPORTED_LAYOUT;
   }

@@ -133,7 +133,16 @@ __device__ __forceinline__ float box_lower(const CpLane &L, float lox, float loy
 }
 
 // what a box bound is compared with (see the file comment)
-__device__ __forceinline__ float cp_limit(const CpLane &L) { return fmaf(L.b.d2, 1.0f + 3.814697265625e-06f, 1e-42f); }
+__device__ __forceinline__ float cp_limit(float d2) { return fmaf(d2, 1.0f + 3.814697265625e-06f, 1e-42f); }
+
+// all nine coordinates finite: x * 0 is 0, for infinities and NaN it is NaN
+__device__ __forceinline__ bool finite_triangle(float4 p0, float4 p1, float4 p2) {
+  float z = p0.x * 0.0f;
+  z = fmaf(p0.y, 0.0f, z); z = fmaf(p0.z, 0.0f, z);
+  z = fmaf(p1.x, 0.0f, z); z = fmaf(p1.y, 0.0f, z); z = fmaf(p1.z, 0.0f, z);
+  z = fmaf(p2.x, 0.0f, z); z = fmaf(p2.y, 0.0f, z); z = fmaf(p2.z, 0.0f, z);
+  return z == 0.0f;
+}
 
 // triangles [first, first + count): keep the lexicographic minimum of (d2, id)
 template <bool STATS>
@@ -164,12 +173,7 @@ __device__ __forceinline__ void cp_leaf(const TraceArgs &a, CpLane &L, uint32_t 
       p2 = ldg4f(q + 2);
       id = __float_as_uint(p0.w);
     }
-    // all nine coordinates finite: x * 0 is 0, for infinities and NaN it is NaN
-    float z = p0.x * 0.0f;
-    z = fmaf(p0.y, 0.0f, z); z = fmaf(p0.z, 0.0f, z);
-    z = fmaf(p1.x, 0.0f, z); z = fmaf(p1.y, 0.0f, z); z = fmaf(p1.z, 0.0f, z);
-    z = fmaf(p2.x, 0.0f, z); z = fmaf(p2.y, 0.0f, z); z = fmaf(p2.z, 0.0f, z);
-    if (z != 0.0f) continue;
+    if (!finite_triangle(p0, p1, p2)) continue;
     float u, v;
     const float d2 = cp_triangle(L.px, L.py, L.pz, p0, p1, p2, u, v);
     if (d2 < L.b.d2 || (d2 == L.b.d2 && id < L.b.id)) L.b = CpBest{d2, u, v, id};
@@ -179,7 +183,7 @@ __device__ __forceinline__ void cp_leaf(const TraceArgs &a, CpLane &L, uint32_t 
 // next stacked entry whose bound can still hold a closer point
 template <class S>
 __device__ __forceinline__ uint32_t cp_pop(const CpLane &L, S &st) {
-  const float lim = cp_limit(L);
+  const float lim = cp_limit(L.b.d2);
   while (!st.empty()) {
     const uint2 e = st.pop();
     if (__uint_as_float(e.y) <= lim) return e.x;
@@ -212,7 +216,7 @@ __device__ __forceinline__ void cp_step_wide(const TraceArgs &a, CpLane &L, S &s
     sy = __uint_as_float(((q[0].w >> 8) & 0xFFu) << 23);
     sz = __uint_as_float(((q[0].w >> 16) & 0xFFu) << 23);
   }
-  const float lim = cp_limit(L);
+  const float lim = cp_limit(L.b.d2);
   uint32_t cref[W];
   float clb[W];
   uint32_t base_node = 0, base_prim = 0, leaf_acc = 0;
@@ -305,7 +309,7 @@ __device__ __forceinline__ void cp_step_bin(const TraceArgs &a, CpLane &L, S &st
   uint32_t lc, lf, rc, rf;
   own_node<PREC, SOA>(a, l, llo, lhi, lc, lf);
   own_node<PREC, SOA>(a, r, rlo, rhi, rc, rf);
-  const float lim = cp_limit(L);
+  const float lim = cp_limit(L.b.d2);
   const float bl = box_lower(L, llo[0], llo[1], llo[2], lhi[0], lhi[1], lhi[2]);
   const float br = box_lower(L, rlo[0], rlo[1], rlo[2], rhi[0], rhi[1], rhi[2]);
   const bool inl = bl <= lim, inr = br <= lim;

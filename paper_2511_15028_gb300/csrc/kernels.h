@@ -49,6 +49,23 @@ TraceKernel cpq_kernels_w2_p5(int soa, int cref, int stats);
 TraceKernel cpq_kernels_w4_p5(int soa, int cref, int stats);
 TraceKernel cpq_kernels_w8_p5(int soa, int cref, int stats);
 
+// one query per warp (query: 0 closest hit, 1 any hit, 2 closest point)
+TraceKernel coop_own_p0(int soa, int cref, int query);
+TraceKernel coop_own_p3(int soa, int cref, int query);
+TraceKernel coop_own_p4(int soa, int cref, int query);
+TraceKernel coop_own_p6(int soa, int cref, int query);  // null: not supported
+TraceKernel coop_w2_p0(int soa, int cref, int query);
+TraceKernel coop_w2_p1(int soa, int cref, int query);
+TraceKernel coop_w2_p2(int soa, int cref, int query);
+TraceKernel coop_w2_p5(int soa, int cref, int query);
+TraceKernel coop_w4_p0(int soa, int cref, int query);
+TraceKernel coop_w4_p1(int soa, int cref, int query);
+TraceKernel coop_w4_p2(int soa, int cref, int query);
+TraceKernel coop_w4_p5(int soa, int cref, int query);
+TraceKernel coop_w8_p0(int soa, int cref, int query);
+TraceKernel coop_w8_p1(int soa, int cref, int query);
+TraceKernel coop_w8_p2(int soa, int cref, int query);
+TraceKernel coop_w8_p5(int soa, int cref, int query);
 // multi-scene kernels of one family
 BatchKernel batched_own_p0(int soa);
 BatchKernel batched_own_p3(int soa);

@@ -48,6 +48,7 @@ struct TraceArgs {
   uint32_t max_steps;
   uint32_t ordered;         // 0 slot order, 1 sorted by entry distance, 2 nearest first
   uint32_t smem_stack;      // shared-memory stack entries per thread
+  uint32_t stack_need;      // entries that the tree can need (one query per warp)
   uint32_t refill_min;      // a warp takes new rays once this many of its lanes are idle (32: all)
   uint32_t raster_w;        // 0, or rays form a row-major image this wide: slots run through 8x4 tiles
   uint32_t chunk;           // slots a warp takes at a time: 32, or a power of two below for a small launch

@@ -3,6 +3,7 @@
 // or eq10 boxes, or the shared-slab node), or -DSCION_W=<2|4|8> -DSCION_PREC=<0|1|2|5>, so the families
 // build in parallel.
 #include "batched.cuh"
+#include "coop.cuh"
 #include "cpq.cuh"
 #include "kernels.h"
 
@@ -17,11 +18,13 @@ namespace scion {
 #define SCION_GETTER SCION_CAT(kernels_own_p, SCION_PREC)
 #define SCION_CPQ_GETTER SCION_CAT(cpq_kernels_own_p, SCION_PREC)
 #define SCION_BATCH_GETTER SCION_CAT(batched_own_p, SCION_PREC)
+#define SCION_COOP_GETTER SCION_CAT(coop_own_p, SCION_PREC)
 #else
 #define SCION_FAMILY_OWN 0
 #define SCION_GETTER SCION_CAT(SCION_CAT(SCION_CAT(kernels_w, SCION_W), _p), SCION_PREC)
 #define SCION_CPQ_GETTER SCION_CAT(SCION_CAT(SCION_CAT(cpq_kernels_w, SCION_W), _p), SCION_PREC)
 #define SCION_BATCH_GETTER SCION_CAT(SCION_CAT(SCION_CAT(batched_w, SCION_W), _p), SCION_PREC)
+#define SCION_COOP_GETTER SCION_CAT(SCION_CAT(SCION_CAT(coop_w, SCION_W), _p), SCION_PREC)
 #endif
 
 // The register tier of the stack spills under the 64-register cap of four
@@ -72,6 +75,26 @@ TraceKernel SCION_CPQ_GETTER(int soa, int cref, int stats) {
       {{cpq_kernel<0, 0, false>, cpq_kernel<0, 0, true>}, {cpq_kernel<0, 1, false>, cpq_kernel<0, 1, true>}},
       {{cpq_kernel<1, 0, false>, cpq_kernel<1, 0, true>}, {cpq_kernel<1, 1, false>, cpq_kernel<1, 1, true>}}};
   return table[soa & 1][cref & 1][stats & 1];
+}
+#endif
+
+// One query per warp; query 0 closest hit, 1 any hit, 2 closest point. The
+// shared-slab node carries intervals, not boxes: not offered.
+#if SCION_FAMILY_OWN && SCION_PREC == 6
+TraceKernel SCION_COOP_GETTER(int, int, int) { return nullptr; }
+#else
+template <int SOA, int CREF, int QUERY>
+__global__ void __launch_bounds__(kMaxThreadsPerBlock, kMinBlocksPerSm) coop_kernel(TraceArgs a) {
+  if constexpr (QUERY == 2) coop_body<SCION_FAMILY_OWN != 0, SCION_W, SCION_PREC, SOA, CREF, false, CoopPoint>(a);
+  else coop_body<SCION_FAMILY_OWN != 0, SCION_W, SCION_PREC, SOA, CREF, QUERY == 1, CoopRay<QUERY == 1>>(a);
+}
+TraceKernel SCION_COOP_GETTER(int soa, int cref, int query) {
+  static const TraceKernel table[2][2][3] = {
+      {{coop_kernel<0, 0, 0>, coop_kernel<0, 0, 1>, coop_kernel<0, 0, 2>},
+       {coop_kernel<0, 1, 0>, coop_kernel<0, 1, 1>, coop_kernel<0, 1, 2>}},
+      {{coop_kernel<1, 0, 0>, coop_kernel<1, 0, 1>, coop_kernel<1, 0, 2>},
+       {coop_kernel<1, 1, 0>, coop_kernel<1, 1, 1>, coop_kernel<1, 1, 2>}}};
+  return table[soa & 1][cref & 1][query];
 }
 #endif
 

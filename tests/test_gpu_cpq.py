@@ -62,6 +62,18 @@ def test_config1_every_layout(sc_mod, config1_points, kw):
     assert sc_mod.scion_get_status(bvh) == 0
 
 
+@pytest.mark.parametrize("kw", ALL, ids=lambda kw: "-".join(str(v) for v in kw.values()))
+def test_config1_every_layout_per_lane(sc_mod, config1_points, kw):
+    """The same points eight times over, which is past the launches that answer
+    one point per warp: the kernels with a point per lane."""
+    sc, pts, exp = config1_points
+    bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
+    many, exp = np.tile(pts, (8, 1)), np.tile(exp, 8)
+    same(query(sc_mod, bvh, many), exp, str(kw))
+    same(query(sc_mod, bvh, many, dict(smem_stack=1)), exp, str(kw) + " shallow shared stack")
+    assert sc_mod.scion_get_status(bvh) == 0
+
+
 def test_radius_surface_far_and_nonfinite_points(sc_mod, oracle_mod):
     sc = scenes.config1_scene()
     tris = sc.triangles()
@@ -83,6 +95,8 @@ def test_radius_surface_far_and_nonfinite_points(sc_mod, oracle_mod):
                dict(width=8, box_prec="f16", box_layout="soa"), dict(box_prec="q16"), dict(box_prec="eq10")):
         bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
         same(query(sc_mod, bvh, pts), exp, str(kw))
+        # a point per lane instead of one per warp
+        same(query(sc_mod, bvh, pts, dict(threads_per_block=128)), exp, str(kw) + " per lane")
 
 
 def test_soup_gpu_built_refit_and_counting(sc_mod, oracle_mod):

@@ -106,6 +106,20 @@ def test_small_launches(sc_mod, config1, n):
         assert sc_mod.scion_get_status(bvh) == 0
 
 
+@pytest.mark.parametrize("kw", ALL, ids=lambda kw: "-".join(str(v) for v in kw.values()))
+def test_config1_every_layout_per_lane(sc_mod, config1, kw):
+    """The same rays four times over, which is past the launches that trace one
+    ray per warp: the kernels with a ray per lane, in each fetch mode."""
+    sc, rays, exp, occ = config1
+    bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
+    many, exp, occ = np.tile(rays, (4, 1)), np.tile(exp, 4), np.tile(occ, 4)
+    for p in (None, dict(rays_per_fetch=1), dict(rays_per_fetch=13, ordered_children=2), dict(ordered_children=3),
+              dict(raster_width=128)):
+        assert_same_hits(gpu_closest(sc_mod, bvh, many, params=p), exp, f"{kw} {p}")
+        assert np.array_equal(gpu_any(sc_mod, bvh, many, params=p), occ), f"{kw} {p}"
+    assert sc_mod.scion_get_status(bvh) == 0
+
+
 def test_closed_form_scenes_on_gpu(sc_mod, oracle_mod):
     tri = np.array([[0, 0, 0], [1, 0, 0], [0, 1, 0]], np.float32)
     quad = np.array([[0, 0, 0], [1, 0, 0], [1, 1, 0], [0, 0, 0], [1, 1, 0], [0, 1, 0]], np.float32)
@@ -167,9 +181,15 @@ def test_edge_cases(sc_mod, oracle_mod):
     bad[9, 3] = -10.0
     bad[9, 4:7] = [0, 0, 1]
     exp = oracle_mod.closest_brute(sc.triangles(), bad)
+    occ = oracle_mod.any_brute(sc.triangles(), bad)
     for kw in ALL[::3]:
         b = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
         assert_same_hits(gpu_closest(sc_mod, b, bad), exp, str(kw))
+        assert np.array_equal(gpu_any(sc_mod, b, bad), occ), str(kw)
+        # a ray per lane instead of one per warp
+        for p in (dict(threads_per_block=128), dict(threads_per_block=128, rays_per_fetch=4)):
+            assert_same_hits(gpu_closest(sc_mod, b, bad, params=p), exp, f"{kw} {p}")
+            assert np.array_equal(gpu_any(sc_mod, b, bad, params=p), occ), f"{kw} {p}"
     # scenes with no hittable triangle, and a scene with non-finite triangles
     none = np.full((9, 3), np.nan, np.float32)
     for kw in ({}, dict(width=8, box_prec="u8")):
