@@ -305,6 +305,20 @@ scion_status scion_trace_backward(scion_bvh bvh, const scion_ray *d_rays, const 
                                   const float *d_grad_tuv, uint64_t n, float *d_grad_verts,
                                   scion_ray *d_grad_rays, scion_stream stream);
 
+/* scion_trace_backward for gradients that lie in arrays of their own: dL/dt of
+ * ray i is d_grad_t[i * stride_t] (stride 0: one value for every ray), or 0 for
+ * every ray where d_grad_t is NULL; u and v likewise. */
+scion_status scion_trace_backward_split(scion_bvh bvh, const scion_ray *d_rays, const scion_hit *d_hits,
+                                        const float *d_grad_t, int64_t stride_t, const float *d_grad_u,
+                                        int64_t stride_u, const float *d_grad_v, int64_t stride_v, uint64_t n,
+                                        float *d_grad_verts, scion_ray *d_grad_rays, scion_stream stream);
+
+/* The fields of d_hits (n of them) as arrays of their own: float d_t[n], d_u[n],
+ * d_v[n] and uint32 d_prim[n], all device memory (else
+ * SCION_ERR_INVALID_ARG), in one launch. */
+scion_status scion_split_hits(const scion_hit *d_hits, uint64_t n, float *d_t, float *d_u, float *d_v,
+                              uint32_t *d_prim, scion_stream stream);
+
 /* Closest point on the scene for each query point (App. G "Closest Point
  * Query", on any layout of the BVH): the lexicographic minimum of (d2, id)
  * over the triangles with d2 <= r2max, d2 the squared distance to the closest

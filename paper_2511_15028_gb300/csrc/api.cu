@@ -1095,34 +1095,67 @@ scion_status scion_trace_stats(scion_bvh b, const scion_ray *d_rays, uint64_t n,
 scion_status scion_trace_backward(scion_bvh b, const scion_ray *d_rays, const scion_hit *d_hits,
                                   const float *d_grad_tuv, uint64_t n, float *d_grad_verts,
                                   scion_ray *d_grad_rays, scion_stream stream) {
-  if (!b || (n > 0 && (!d_rays || !d_hits || !d_grad_tuv || !d_grad_verts))) return SCION_ERR_INVALID_ARG;
+  if (n > 0 && !d_grad_tuv) return SCION_ERR_INVALID_ARG;
+  return scion_trace_backward_split(b, d_rays, d_hits, d_grad_tuv, 3, d_grad_tuv + 1, 3, d_grad_tuv + 2, 3, n,
+                                    d_grad_verts, d_grad_rays, stream);
+}
+
+scion_status scion_trace_backward_split(scion_bvh b, const scion_ray *d_rays, const scion_hit *d_hits,
+                                        const float *d_grad_t, int64_t stride_t, const float *d_grad_u,
+                                        int64_t stride_u, const float *d_grad_v, int64_t stride_v, uint64_t n,
+                                        float *d_grad_verts, scion_ray *d_grad_rays, scion_stream stream) {
+  if (!b || (n > 0 && (!d_rays || !d_hits || !d_grad_verts))) return SCION_ERR_INVALID_ARG;
   if (n == 0) return SCION_OK;
+  const float *grad[3] = {d_grad_t, d_grad_u, d_grad_v};
+  const int64_t stride[3] = {stride_t, stride_u, stride_v};
+  bool aligned = true, device = true;
+  for (int k = 0; k < 3; ++k) {
+    if (!grad[k]) continue;
+    aligned = aligned && (reinterpret_cast<uintptr_t>(grad[k]) & 3u) == 0;
+    // one buffer for all three is looked up once
+    if (k == 0 || stride[k] != 3 || grad[k] != grad[0] + k) device = device && is_device_ptr(grad[k]);
+  }
   if ((reinterpret_cast<uintptr_t>(d_rays) & 15u) || (reinterpret_cast<uintptr_t>(d_hits) & 15u) ||
-      (reinterpret_cast<uintptr_t>(d_grad_rays) & 15u) || (reinterpret_cast<uintptr_t>(d_grad_tuv) & 3u) ||
-      (reinterpret_cast<uintptr_t>(d_grad_verts) & 3u)) {
+      (reinterpret_cast<uintptr_t>(d_grad_rays) & 15u) || !aligned || (reinterpret_cast<uintptr_t>(d_grad_verts) & 3u)) {
     g_last_error = "scion_trace_backward: misaligned buffer";
     return SCION_ERR_INVALID_ARG;
   }
   if (!on_bvh_device(b)) return SCION_ERR_INVALID_ARG;
   // the kernel scatters into the gradients with device atomics: device memory only
-  if (!is_device_ptr(d_rays) || !is_device_ptr(d_hits) || !is_device_ptr(d_grad_tuv) ||
-      !is_device_ptr(d_grad_verts) || (d_grad_rays && !is_device_ptr(d_grad_rays))) {
+  if (!is_device_ptr(d_rays) || !is_device_ptr(d_hits) || !device || !is_device_ptr(d_grad_verts) ||
+      (d_grad_rays && !is_device_ptr(d_grad_rays))) {
     g_last_error = "scion_trace_backward takes device buffers";
     return SCION_ERR_INVALID_ARG;
   }
   BackwardArgs a;
   a.rays = reinterpret_cast<const float *>(d_rays);
   a.hits = reinterpret_cast<const uint32_t *>(d_hits);
-  a.grad_tuv = d_grad_tuv;
+  for (int k = 0; k < 3; ++k) {
+    a.grad[k] = grad[k];
+    a.stride[k] = stride[k];
+  }
   a.verts = static_cast<const float4 *>(b->d_verts);
   a.tri_idx = static_cast<const uint32_t *>(b->d_idx);
   a.grad_verts = d_grad_verts;
   a.grad_rays = reinterpret_cast<float *>(d_grad_rays);
   a.n = n;
   a.n_tris = b->n_tris;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  SCION_CUDA(launch_backward(a, device_sms(dev), reinterpret_cast<cudaStream_t>(stream)));
+  SCION_CUDA(launch_backward(a, device_sms(b->device), reinterpret_cast<cudaStream_t>(stream)));
+  return SCION_OK;
+}
+
+scion_status scion_split_hits(const scion_hit *d_hits, uint64_t n, float *d_t, float *d_u, float *d_v,
+                              uint32_t *d_prim, scion_stream stream) {
+  if (n == 0) return SCION_OK;
+  const void *out[4] = {d_t, d_u, d_v, d_prim};
+  bool ok = d_hits && (reinterpret_cast<uintptr_t>(d_hits) & 15u) == 0 && is_device_ptr(d_hits);
+  for (const void *p : out) ok = ok && p && (reinterpret_cast<uintptr_t>(p) & 3u) == 0 && is_device_ptr(p);
+  if (!ok) {
+    g_last_error = "scion_split_hits takes device buffers, hits 16-byte and results 4-byte aligned";
+    return SCION_ERR_INVALID_ARG;
+  }
+  SCION_CUDA(launch_split_hits(reinterpret_cast<const uint32_t *>(d_hits), n, d_t, d_u, d_v, d_prim,
+                               device_sms(current_device()), reinterpret_cast<cudaStream_t>(stream)));
   return SCION_OK;
 }
 

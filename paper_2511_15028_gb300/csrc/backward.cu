@@ -128,7 +128,8 @@ __device__ __forceinline__ void add_vertex(float *grad_verts, uint32_t vid, floa
   atomicAdd(g + (odd ? 0 : 2), odd ? x : z);
 }
 
-template <bool PAIRED>
+// PACKED: the three gradients of a ray lie together (strides of 3 from grad[0]).
+template <bool PAIRED, bool PACKED>
 __global__ void __launch_bounds__(256) backward_kernel(BackwardArgs a) {
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
   const uint32_t lane = threadIdx.x & 31u;
@@ -156,7 +157,13 @@ __global__ void __launch_bounds__(256) backward_kernel(BackwardArgs a) {
       const Pair c0[3] = {{rd.x, 0.f}, {rd.y, 0.f}, {rd.z, 0.f}};
       const Pair c1[3] = {two_diff(p0.x, p1.x), two_diff(p0.y, p1.y), two_diff(p0.z, p1.z)};
       const Pair c2[3] = {two_diff(p0.x, p2.x), two_diff(p0.y, p2.y), two_diff(p0.z, p2.z)};
-      const float gt = a.grad_tuv[3 * i], gu = a.grad_tuv[3 * i + 1], gv = a.grad_tuv[3 * i + 2];
+      float g[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        if (PACKED) g[k] = __ldg(a.grad[0] + 3 * i + k);
+        else g[k] = a.grad[k] ? __ldg(a.grad[k] + (long long)i * a.stride[k]) : 0.0f;
+      }
+      const float gt = g[0], gu = g[1], gv = g[2];
       if (!solve_refined(c0, c1, c2, gt, gu, gv, lf)) {
         // the columns in double: differences of two floats
         const double e0[3] = {rd.x, rd.y, rd.z};
@@ -207,14 +214,40 @@ __global__ void __launch_bounds__(256) backward_kernel(BackwardArgs a) {
   }
 }
 
+__global__ void __launch_bounds__(256) split_hits_kernel(const uint4 *__restrict__ hits, unsigned long long n, float *t,
+                                                         float *u, float *v, uint32_t *prim) {
+  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const uint4 h = __ldg(hits + i);
+    t[i] = __uint_as_float(h.x);
+    u[i] = __uint_as_float(h.y);
+    v[i] = __uint_as_float(h.z);
+    prim[i] = h.w;
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_split_hits(const uint32_t *hits, unsigned long long n, float *t, float *u, float *v, uint32_t *prim,
+                              int sms, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  const unsigned long long blocks = (n + 255) / 256, most = (unsigned long long)sms * 16;
+  split_hits_kernel<<<(unsigned)(blocks < most ? blocks : most), 256, 0, s>>>(reinterpret_cast<const uint4 *>(hits), n, t, u,
+                                                                             v, prim);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_backward(const BackwardArgs &a, int sms, cudaStream_t s) {
   if (a.n == 0) return cudaSuccess;
   const unsigned long long blocks = (a.n + 255) / 256;
   const unsigned grid = (unsigned)(blocks < (unsigned long long)sms * 8 ? blocks : (unsigned long long)sms * 8);
-  if ((reinterpret_cast<uintptr_t>(a.grad_verts) & 7u) == 0) backward_kernel<true><<<grid, 256, 0, s>>>(a);
-  else backward_kernel<false><<<grid, 256, 0, s>>>(a);
+  const bool paired = (reinterpret_cast<uintptr_t>(a.grad_verts) & 7u) == 0;
+  const bool packed = a.grad[0] && a.grad[1] == a.grad[0] + 1 && a.grad[2] == a.grad[0] + 2 && a.stride[0] == 3 &&
+                      a.stride[1] == 3 && a.stride[2] == 3;
+  if (paired && packed) backward_kernel<true, true><<<grid, 256, 0, s>>>(a);
+  else if (paired) backward_kernel<true, false><<<grid, 256, 0, s>>>(a);
+  else if (packed) backward_kernel<false, true><<<grid, 256, 0, s>>>(a);
+  else backward_kernel<false, false><<<grid, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 

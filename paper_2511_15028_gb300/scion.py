@@ -142,6 +142,9 @@ def lib():
         L.scion_get_status.argtypes = [P, P, P]
         L.scion_trace_stats.argtypes = [P, P, U64, U32, P, ctypes.POINTER(TraceParams), P, P]
         L.scion_trace_backward.argtypes = [P, P, P, P, U64, P, P, P]
+        I64 = ctypes.c_int64
+        L.scion_trace_backward_split.argtypes = [P, P, P, P, I64, P, I64, P, I64, U64, P, P, P]
+        L.scion_split_hits.argtypes = [P, U64, P, P, P, P, P]
         L.scion_batch_create.argtypes = [P, P, P, P, U32, P, P, ctypes.POINTER(P)]
         L.scion_batch_launch.argtypes = [P, P]
         L.scion_batch_info.argtypes = [P, P, P]
@@ -175,7 +178,8 @@ def lib():
         for name in ("scion_build", "scion_build_gpu", "scion_bvh_build_times", "scion_refit",
                      "scion_query_closest_point",
                      "scion_build_many", "scion_bvh_info", "scion_trace_closest", "scion_trace_any",
-                     "scion_trace_stats", "scion_trace_backward", "scion_batch_create",
+                     "scion_trace_stats", "scion_trace_backward", "scion_trace_backward_split",
+                     "scion_split_hits", "scion_batch_create",
                      "scion_batch_launch", "scion_batch_info", "scion_trace_batched",
                      "scion_get_status", "scion_debug_build_host", "scion_debug_host_stats",
                      "scion_debug_host_decode", "scion_debug_host_raw"):
@@ -460,24 +464,33 @@ def _trace_fn():
 
         @staticmethod
         def forward(ctx, verts, rays, bvh):
-            hits = scion_trace_closest(bvh, rays.detach().contiguous())
+            r = rays.detach().contiguous()
+            hits = scion_trace_closest(bvh, r)
             ctx.save_for_backward(rays, hits)
             ctx.bvh = bvh
-            f = hits.view(torch.float32)
-            prim = hits[:, 3]
+            ctx.set_materialize_grads(False)  # a missing gradient is zero to the kernel
+            n = hits.shape[0]
+            t, u, v = (torch.empty(n, dtype=torch.float32, device=hits.device) for _ in range(3))
+            prim = torch.empty(n, dtype=torch.int32, device=hits.device)
+            _check(lib().scion_split_hits(hits.data_ptr(), n, t.data_ptr(), u.data_ptr(), v.data_ptr(),
+                                          prim.data_ptr(), _stream_ptr(None)), "scion_split_hits")
             ctx.mark_non_differentiable(prim)
-            return f[:, 0].clone(), f[:, 1].clone(), f[:, 2].clone(), prim.clone()
+            return t, u, v, prim
 
         @staticmethod
         def backward(ctx, gt, gu, gv, _gp):
             rays, hits = ctx.saved_tensors
-            n = rays.shape[0]
-            z = lambda x: x if x is not None else torch.zeros(n, device=rays.device)  # noqa: E731
-            g = torch.stack([z(gt), z(gu), z(gv)], -1).contiguous()
-            gverts, grays = scion_trace_backward(ctx.bvh, rays.detach().contiguous(), hits, g,
-                                                 want_ray_grads=ctx.needs_input_grad[1])
-            return (gverts if ctx.needs_input_grad[0] else None,
-                    grays if ctx.needs_input_grad[1] else None, None)
+            bvh, n = ctx.bvh, rays.shape[0]
+            r = rays.detach().contiguous()
+            # as they come, strides and all (a sum's gradient has stride 0)
+            g = [None if x is None else x.float() for x in (gt, gu, gv)]
+            args = [a for x in g for a in ((None, 0) if x is None else (x.data_ptr(), x.stride(0) if n > 1 else 0))]
+            gverts = torch.zeros((bvh.n_verts, 3), dtype=torch.float32, device=r.device)
+            grays = torch.empty((n, 8), dtype=torch.float32, device=r.device) if ctx.needs_input_grad[1] else None
+            _check(lib().scion_trace_backward_split(bvh.handle, r.data_ptr(), hits.data_ptr(), *args, n,
+                                                    gverts.data_ptr(), None if grays is None else grays.data_ptr(),
+                                                    _stream_ptr(None)), "scion_trace_backward")
+            return (gverts if ctx.needs_input_grad[0] else None, grays, None)
 
     return TraceFn
 

@@ -129,6 +129,39 @@ def test_autograd_function_and_accumulation(setup):
     assert np.all(np.abs(gv2.cpu().numpy() - 2 * gvv) <= 2e-5 * S + 2e-6)
 
 
+def test_autograd_missing_and_strided_gradients(setup):
+    """Gradients of one output only (the others missing), of a plain sum (one
+    value with stride 0) and of a strided view, against the same gradients
+    written out; outputs are tensors of their own that may be changed in
+    place."""
+    scion, sc, rays, tris, g, hits, gv64, gr64 = setup
+    bvh = scion.scion_build(sc.verts, scion.layout(width=4, box_layout="soa"), sc.indices)
+    verts = torch.from_numpy(sc.verts).cuda().requires_grad_(True)
+    r = torch.from_numpy(rays).cuda().requires_grad_(True)
+    w = torch.from_numpy(g).cuda()
+    n = r.shape[0]
+    out = scion.trace_fn().apply(verts, r, bvh)
+    h = scion.split_hits(scion.scion_trace_closest(bvh, r.detach()))
+    for x, name in zip(out, ("t", "u", "v", "prim")):
+        assert x.is_contiguous() and np.array_equal(x.detach().cpu().numpy().view(np.uint32), h[name].view(np.uint32))
+    t, u, v, prim = out
+    assert not prim.requires_grad
+    for loss, full in (((u * w[:, 1]).sum(), torch.stack([0 * w[:, 0], w[:, 1], 0 * w[:, 0]], 1)),
+                       (u.sum() + v.sum(), torch.tensor([0.0, 1.0, 1.0], device="cuda").expand(n, 3)),
+                       ((u * w.t()[2]).sum(), torch.stack([0 * w[:, 0], w[:, 2], 0 * w[:, 0]], 1))):
+        got = torch.autograd.grad(loss, [verts, r], retain_graph=True)
+        ref = scion.scion_trace_backward(bvh, r.detach(), scion.scion_trace_closest(bvh, r.detach()), full.contiguous())
+        assert torch.equal(got[1], ref[1])
+        # the vertices' sums come in another order: FP32 summation error of the reference test
+        S = _abs_scale(sc, rays, hits, full.cpu().numpy().astype(np.float32), tris)
+        assert np.all(np.abs((got[0] - ref[0]).cpu().numpy()) <= 1e-5 * S + 1e-6)
+    t2, u2, _, _ = scion.trace_fn().apply(verts, r, bvh)
+    u2.mul_(2.0)
+    two = torch.autograd.grad((u2 * w[:, 1]).sum(), [r])[0]
+    one = torch.autograd.grad((u * w[:, 1]).sum(), [r])[0]
+    assert torch.equal(two, 2 * one)
+
+
 def test_backward_and_counters_take_device_buffers_only(setup):
     """Gradients and visit counters are added with device atomics: host
     buffers are rejected before any launch."""
