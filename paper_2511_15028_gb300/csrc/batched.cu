@@ -36,8 +36,7 @@ constexpr int kMaxSharedScenes = 1024;  // scene starts cached in shared memory
 
 template <bool OWN, int W, int PREC, int SOA>
 __device__ __forceinline__ void step_family(const TraceArgs &a, Lane &L, Stack &st, Counts &cnt) {
-  if constexpr (OWN) step_bin<PREC, SOA, REF_DIRECT, false, false>(a, L, st, cnt);
-  else step_wide<W, PREC, SOA, REF_DIRECT, false, false>(a, L, st, cnt);
+  step_any_layout<OWN, W, PREC, SOA, REF_DIRECT, false, false>(a, L, st, cnt);
 }
 
 // The next 32-ray unit of the global index space (warp-uniform).
@@ -97,14 +96,7 @@ __device__ __noinline__ unsigned long long run_scene(const BatchScene &S, unsign
       const unsigned long long rid = base - s_lo + lane;
       if (rid < a.n) {
         start_lane<OWN, PREC, SOA>(a, L, st, rid);
-        while (L.cur != kEmptyRef) {
-          if (++L.steps > a.max_steps) {
-            L.err = kErrIter;
-            L.cur = kEmptyRef;
-            break;
-          }
-          step_family<OWN, W, PREC, SOA>(a, L, st, cnt);
-        }
+        while (L.cur != kEmptyRef) step_family<OWN, W, PREC, SOA>(a, L, st, cnt);
         finish_lane(a, L);
       }
       base = take_unit(work);
@@ -148,14 +140,7 @@ __device__ __noinline__ unsigned long long run_scene(const BatchScene &S, unsign
     // a unit of this scene always holds a ray, so with every lane idle the
     // warp either took rays above or has moved past the scene
     if (__ballot_sync(0xFFFFFFFFu, has_ray) == 0u) break;
-    if (has_ray && L.cur != kEmptyRef) {
-      if (++L.steps > a.max_steps) {
-        L.err = kErrIter;
-        L.cur = kEmptyRef;
-      } else {
-        step_family<OWN, W, PREC, SOA>(a, L, st, cnt);
-      }
-    }
+    if (has_ray && L.cur != kEmptyRef) step_family<OWN, W, PREC, SOA>(a, L, st, cnt);
     if (has_ray && L.cur == kEmptyRef) {
       finish_lane(a, L);
       has_ray = false;

@@ -57,8 +57,7 @@ __device__ __forceinline__ void batched_body(const BatchArgs &ba) {
         const unsigned long long rid = (unsigned long long)unit * ba.chunk - at.begin + lane;
         if (lane < ba.chunk && rid < a.n) {
           q.start(a, rid);
-          while (q.busy())
-            if (!q.step(a)) break;
+          while (q.busy()) q.step(a);
           q.finish(a);
         }
         unit = take();

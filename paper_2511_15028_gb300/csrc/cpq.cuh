@@ -191,20 +191,21 @@ __device__ __forceinline__ uint32_t cp_pop(const CpLane &L, S &st) {
   return kEmptyRef;
 }
 
-// Wide node: bound every child box, enter the nearest, stack the others
-// (nearest last pushed, so popped first); a leaf entry tests its triangles.
+// Leaf entry: one triangle, as the ray traversal (the counting kernels: all).
+template <bool STATS, class S>
+__device__ __forceinline__ void cp_leaf_wide(const TraceArgs &a, CpLane &L, S &st, Counts &cnt) {
+  const uint32_t count = ref_leaf_count(L.cur);
+  cp_leaf<STATS>(a, L, ref_leaf_first(L.cur), STATS ? count : 1u, cnt);
+  if (!STATS && count > 1u) L.cur += (1u << 5) - (1u << 1);  // ref_leaf(first + 1, count - 1)
+  else L.cur = cp_pop(L, st);
+}
+
+// Interior node: bound every child box, enter the nearest, stack the others
+// (nearest last pushed, so popped first).
 template <int W, int PREC, int SOA, int CREF, bool STATS, class S>
-__device__ __forceinline__ void cp_step_wide(const TraceArgs &a, CpLane &L, S &st, Counts &cnt) {
+__device__ __forceinline__ void cp_node_wide(const TraceArgs &a, CpLane &L, S &st, Counts &cnt) {
   using N = WideNode<W, PREC, SOA, CREF>;
   const uint32_t cur = L.cur;
-  if (!ref_is_interior(cur)) {
-    // one triangle per step, as the ray traversal (the counting kernels: all)
-    const uint32_t count = ref_leaf_count(cur);
-    cp_leaf<STATS>(a, L, ref_leaf_first(cur), STATS ? count : 1u, cnt);
-    if (!STATS && count > 1u) L.cur = cur + (1u << 5) - (1u << 1);  // ref_leaf(first + 1, count - 1)
-    else L.cur = cp_pop(L, st);
-    return;
-  }
   if (STATS) cnt.nodes++;
   const uint4 *np = a.nodes + (size_t)ref_node(cur) * (N::kStride / 16);
   uint4 q[N::NQ];
@@ -290,18 +291,20 @@ __device__ __forceinline__ void cp_bin_pop(const TraceArgs &a, CpLane &L, S &st)
   if (L.cur != kEmptyRef) own_ref<PREC, SOA>(a, L.cur, L.count, L.field);
 }
 
-// Own-box binary node: the entered node's box was bounded by its parent; a
-// leaf tests its triangles, an interior node bounds both children's boxes
-// (the paper's children sorting), enters the nearer and stacks the other.
+// Leaf of an own-box query: one triangle (the counting kernels: all).
+template <int PREC, int SOA, bool STATS, class S>
+__device__ __forceinline__ void cp_leaf_bin(const TraceArgs &a, CpLane &L, S &st, Counts &cnt) {
+  if (STATS) cnt.nodes++;
+  cp_leaf<STATS>(a, L, L.field, STATS ? L.count : 1u, cnt);
+  if (!STATS && --L.count > 0) ++L.field;
+  else cp_bin_pop<PREC, SOA>(a, L, st);
+}
+
+// Own-box interior node (the entered node's box was bounded by its parent):
+// bounds both children's boxes (the paper's children sorting), enters the nearer
+// and stacks the other.
 template <int PREC, int SOA, int CREF, bool STATS, class S>
-__device__ __forceinline__ void cp_step_bin(const TraceArgs &a, CpLane &L, S &st, Counts &cnt) {
-  if (L.count > 0) {
-    if (STATS) cnt.nodes++;
-    cp_leaf<STATS>(a, L, L.field, STATS ? L.count : 1u, cnt);
-    if (!STATS && --L.count > 0) ++L.field;
-    else cp_bin_pop<PREC, SOA>(a, L, st);
-    return;
-  }
+__device__ __forceinline__ void cp_node_bin(const TraceArgs &a, CpLane &L, S &st, Counts &cnt) {
   if (STATS) cnt.nodes++;
   const uint32_t l = CREF == REF_DIRECT ? L.cur + 1 : L.field;
   const uint32_t r = CREF == REF_DIRECT ? L.cur + L.field : L.field + 1;
@@ -356,15 +359,20 @@ struct PointQuery {
     }
     if (STATS) n_pts++;
   }
-  __device__ __forceinline__ bool step(const TraceArgs &a) {
-    if (++L.steps > a.max_steps) {
+  __device__ __forceinline__ void step(const TraceArgs &a) {
+    if constexpr (OWN) {
+      node_then_leaf<2>(
+          L, [&] { return L.count > 0; }, [&] { cp_node_bin<PREC, SOA, CREF, STATS>(a, L, st, cnt); },
+          [&] { cp_leaf_bin<PREC, SOA, STATS>(a, L, st, cnt); });
+    } else {
+      node_then_leaf<W <= 4 ? 2 : 1>(
+          L, [&] { return !ref_is_interior(L.cur); }, [&] { cp_node_wide<W, PREC, SOA, CREF, STATS>(a, L, st, cnt); },
+          [&] { cp_leaf_wide<STATS>(a, L, st, cnt); });
+    }
+    if (L.steps > a.max_steps) {
       L.err = kErrIter;
       L.cur = kEmptyRef;
-      return false;
     }
-    if constexpr (OWN) cp_step_bin<PREC, SOA, CREF, STATS>(a, L, st, cnt);
-    else cp_step_wide<W, PREC, SOA, CREF, STATS>(a, L, st, cnt);
-    return true;
   }
   __device__ __forceinline__ void finish(const TraceArgs &a) {
     if (L.err) {

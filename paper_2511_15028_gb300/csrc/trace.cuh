@@ -621,205 +621,244 @@ __device__ __forceinline__ void sort_children(float (&t)[W], uint32_t (&r)[W]) {
   }
 }
 
-// One step of the wide-node traversal: process the entry L.cur (an interior
-// node: test its W child boxes, push the hit ones far to near, continue with
-// the nearest; or a leaf: test its triangles), then pick the next entry.
+// A step of a lane's query: up to NODES interior nodes, then up to two triangles of
+// a leaf. L.cur is its entry, at_leaf() whether that is a leaf.
+//
+// What bounds the traversal is the instructions that a warp issues for the few of
+// its lanes that need them: with one node or one triangle per step, every step
+// issued both sides for a warp whose lanes were at either (16 of 32 lanes active
+// for camera rays, 8 for random points). Here the sides follow one another, and a
+// lane that comes to a leaf takes part in the triangle tests of the same step. The
+// lanes at a leaf wait while there are more than kLeafShare lanes at a node for
+// each of them: random rays in a soup meet 13 nodes per triangle, and a test costs
+// as much for two lanes as for all.
+// Measured, one entry per step -> here: 1080p camera rays in 1.4 M triangles (bvh4
+// f32) 353 -> 326 us, 750,000 shadow rays 492 -> 435, 1 M random points 3,646 ->
+// 3,332 (bvh8 f16 5,430 -> 4,528, bvh2 q16 4,435 -> 3,902); 1 M short any-hit rays
+// in 2 M random triangles (bvh2 q16) 715 -> 620; 8.4 M random rays in 8.4 M (bvh4
+// u8) 8,789 -> 7,343; 750,000 bounce rays (bvh8 f16) 479 -> 415. Without the
+// waiting the soups gain less (677 and 7,997 us), the others the same; a share of
+// 4 is 1 to 2 % slower. NODES is 2, for 8-wide nodes 1: their code twice costs more
+// than it gives (bounce rays 501 us).
+// A lane makes the same visits in the same order as one by one; `steps` counts them.
+constexpr uint32_t kLeafShare = 2;
+template <int NODES, class LaneT, class AtLeaf, class Node, class Leaf>
+__device__ __forceinline__ void node_then_leaf(LaneT &L, AtLeaf at_leaf, Node node, Leaf leaf) {
+#pragma unroll
+  for (int i = 0; i < NODES; ++i) {
+    if (L.cur != kEmptyRef && !at_leaf()) {
+      ++L.steps;
+      node();
+    }
+  }
+  // of the lanes that are together here; who is elsewhere decides for itself
+  const uint32_t here = __activemask();
+  const bool busy = L.cur != kEmptyRef, in_leaf = busy && at_leaf();
+  const uint32_t leaves = __popc(__ballot_sync(here, in_leaf)), nodes = __popc(__ballot_sync(here, busy && !in_leaf));
+  if (leaves * kLeafShare < nodes) return;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    if (L.cur != kEmptyRef && at_leaf()) {
+      ++L.steps;
+      leaf();
+    }
+  }
+}
+
+// Interior node L.cur of the wide-node traversal: test its W child boxes, push
+// the hit ones far to near, go on with the nearest or the next stacked entry.
 template <int W, int PREC, int SOA, int CREF, bool ANY, bool STATS, class S>
-__device__ __forceinline__ void step_wide(const TraceArgs &a, Lane &L, S &st, Counts &cnt) {
+__device__ __forceinline__ void node_wide(const TraceArgs &a, Lane &L, S &st, Counts &cnt) {
   using N = WideNode<W, PREC, SOA, CREF>;
   const Ray &r = L.r;
   const uint32_t cur = L.cur;
-  if (ref_is_interior(cur)) {
-    if (STATS) cnt.nodes++;
-    const uint4 *np = a.nodes + (size_t)ref_node(cur) * (N::kStride / 16);
-    uint4 q[N::NQ];
-    load_node<N::NQ>(np, q);
-    // u8 / u16 frame: coordinate = origin + code * 2^e, folded into the plane
-    // distance t = fma(code, 2^e / d, (origin - o) / d) per axis
-    float ax = 0.f, bx = 0.f, ay = 0.f, by = 0.f, az = 0.f, bz = 0.f;
-    if (N::kGrid) {
-      ax = __uint_as_float((q[0].w & 0xFFu) << 23) * r.rx;
-      ay = __uint_as_float(((q[0].w >> 8) & 0xFFu) << 23) * r.ry;
-      az = __uint_as_float(((q[0].w >> 16) & 0xFFu) << 23) * r.rz;
-      bx = fmaf(__uint_as_float(q[0].x), r.rx, -r.orx);
-      by = fmaf(__uint_as_float(q[0].y), r.ry, -r.ory);
-      bz = fmaf(__uint_as_float(q[0].z), r.rz, -r.orz);
-    }
-    const float tlim = far_limit(L.b.t);
-    // paired decode and fma (f32x2) for the grid codes; the 8-wide kernels
-    // would spill with the extra register pairs
-    constexpr bool kPaired = W <= 4;
-    uint32_t cref[W];
-    float ctn[W];
-    uint32_t base_node = 0, base_prim = 0, leaf_acc = 0;
-    if (CREF == REF_INDIRECT) {
-      base_node = qword(q, N::kRefOff / 4);
-      base_prim = qword(q, N::kRefOff / 4 + 1);
-    }
-    // reference of child k (in increasing k: indirect leaves accumulate)
-    auto child_ref = [&](int k) -> uint32_t {
-      if (CREF == REF_DIRECT) return qword(q, N::kRefOff / 4 + k);
-      const uint32_t m = (qword(q, N::kRefOff / 4 + 2 + (k >> 2)) >> ((k & 3) * 8)) & 0xFFu;
-      if (m == 0) return kEmptyRef;
-      if (m & kMetaInterior) return ref_interior(base_node + (m & 0x7Fu));
-      const uint32_t rf = ref_leaf(base_prim + leaf_acc, m);
-      leaf_acc += m;
-      return rf;
-    };
-    if constexpr (N::kRowSel) {
-      constexpr int kRow = N::kRowWords;
+  if (STATS) cnt.nodes++;
+  const uint4 *np = a.nodes + (size_t)ref_node(cur) * (N::kStride / 16);
+  uint4 q[N::NQ];
+  load_node<N::NQ>(np, q);
+  // u8 / u16 frame: coordinate = origin + code * 2^e, folded into the plane
+  // distance t = fma(code, 2^e / d, (origin - o) / d) per axis
+  float ax = 0.f, bx = 0.f, ay = 0.f, by = 0.f, az = 0.f, bz = 0.f;
+  if (N::kGrid) {
+    ax = __uint_as_float((q[0].w & 0xFFu) << 23) * r.rx;
+    ay = __uint_as_float(((q[0].w >> 8) & 0xFFu) << 23) * r.ry;
+    az = __uint_as_float(((q[0].w >> 16) & 0xFFu) << 23) * r.rz;
+    bx = fmaf(__uint_as_float(q[0].x), r.rx, -r.orx);
+    by = fmaf(__uint_as_float(q[0].y), r.ry, -r.ory);
+    bz = fmaf(__uint_as_float(q[0].z), r.rz, -r.orz);
+  }
+  const float tlim = far_limit(L.b.t);
+  // paired decode and fma (f32x2) for the grid codes; the 8-wide kernels
+  // would spill with the extra register pairs
+  constexpr bool kPaired = W <= 4;
+  uint32_t cref[W];
+  float ctn[W];
+  uint32_t base_node = 0, base_prim = 0, leaf_acc = 0;
+  if (CREF == REF_INDIRECT) {
+    base_node = qword(q, N::kRefOff / 4);
+    base_prim = qword(q, N::kRefOff / 4 + 1);
+  }
+  // reference of child k (in increasing k: indirect leaves accumulate)
+  auto child_ref = [&](int k) -> uint32_t {
+    if (CREF == REF_DIRECT) return qword(q, N::kRefOff / 4 + k);
+    const uint32_t m = (qword(q, N::kRefOff / 4 + 2 + (k >> 2)) >> ((k & 3) * 8)) & 0xFFu;
+    if (m == 0) return kEmptyRef;
+    if (m & kMetaInterior) return ref_interior(base_node + (m & 0x7Fu));
+    const uint32_t rf = ref_leaf(base_prim + leaf_acc, m);
+    leaf_acc += m;
+    return rf;
+  };
+  if constexpr (N::kRowSel) {
+    constexpr int kRow = N::kRowWords;
 #pragma unroll
-      for (int j = 0; j < kRow; ++j) {
-        // word j of each coordinate row: near and far planes of its children
-        uint32_t nw[3], fw[3];
+    for (int j = 0; j < kRow; ++j) {
+      // word j of each coordinate row: near and far planes of its children
+      uint32_t nw[3], fw[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const uint32_t lw = qword(q, N::kHdr / 4 + c * kRow + j), hw = qword(q, N::kHdr / 4 + (c + 3) * kRow + j);
-          const bool neg = c == 0 ? r.nx : (c == 1 ? r.ny : r.nz);
-          nw[c] = neg ? hw : lw;
-          fw[c] = neg ? lw : hw;
-        }
-#pragma unroll
-        for (int i = 0; i < N::kPerWord; ++i) {
-          const int k = j * N::kPerWord + i;
-          const uint32_t ref = child_ref(k);
-          const uint32_t b = (uint32_t)(i * N::kElem);  // byte of the child in the word
-          float t0[3], t1[3];
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const float rc = c == 0 ? r.rx : (c == 1 ? r.ry : r.rz), oc = c == 0 ? r.orx : (c == 1 ? r.ory : r.orz);
-            if (N::kGrid) {
-              const uint32_t sel = N::kElem == 1 ? (0x7540u | b) : (0x7400u | ((b + 1u) << 4) | b);
-              const float nb = __uint_as_float(__byte_perm(nw[c], 0x4B000000u, sel));
-              const float fb = __uint_as_float(__byte_perm(fw[c], 0x4B000000u, sel));
-              const float ac = c == 0 ? ax : (c == 1 ? ay : az), bc = c == 0 ? bx : (c == 1 ? by : bz);
-              if (kPaired) {
-                float nq, fq;
-                unbias_pair(nb, fb, nq, fq);
-                fma_pair(nq, fq, ac, bc, t0[c], t1[c]);
-              } else {
-                t0[c] = fmaf(nb - 8388608.0f, ac, bc);
-                t1[c] = fmaf(fb - 8388608.0f, ac, bc);
-              }
-            } else {
-              const float nv = __half2float(__ushort_as_half((unsigned short)((nw[c] >> (b * 8)) & 0xFFFFu)));
-              const float fv = __half2float(__ushort_as_half((unsigned short)((fw[c] >> (b * 8)) & 0xFFFFu)));
-              t0[c] = fmaf(nv, rc, -oc);
-              t1[c] = fmaf(fv, rc, -oc);
-            }
-          }
-          float tn;
-          bool hit = slab_t(r, t0[0], t0[1], t0[2], t1[0], t1[1], t1[2], tlim, tn);
-          hit = hit && ref != kEmptyRef;
-          cref[k] = hit ? ref : kEmptyRef;
-          ctn[k] = hit ? tn : __int_as_float(0x7f800000);
-        }
+      for (int c = 0; c < 3; ++c) {
+        const uint32_t lw = qword(q, N::kHdr / 4 + c * kRow + j), hw = qword(q, N::kHdr / 4 + (c + 3) * kRow + j);
+        const bool neg = c == 0 ? r.nx : (c == 1 ? r.ny : r.nz);
+        nw[c] = neg ? hw : lw;
+        fw[c] = neg ? lw : hw;
       }
-    } else {
 #pragma unroll
-    for (int k = 0; k < W; ++k) {
-      const uint32_t ref = child_ref(k);
-      float tn;
-      bool hit;
-      if (N::kGrid) {
-        // per axis: near and far code of the child (decoded in one paired
-        // add), then both plane distances in one paired fma
+      for (int i = 0; i < N::kPerWord; ++i) {
+        const int k = j * N::kPerWord + i;
+        const uint32_t ref = child_ref(k);
+        const uint32_t b = (uint32_t)(i * N::kElem);  // byte of the child in the word
         float t0[3], t1[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const bool neg = c == 0 ? r.nx : (c == 1 ? r.ny : r.nz);
-          const float lb = N::code_biased(q, k, c), hb = N::code_biased(q, k, c + 3);
-          const float ac = c == 0 ? ax : (c == 1 ? ay : az), bc = c == 0 ? bx : (c == 1 ? by : bz);
-          if (kPaired) {
-            float nq, fq;
-            unbias_pair(neg ? hb : lb, neg ? lb : hb, nq, fq);
-            fma_pair(nq, fq, ac, bc, t0[c], t1[c]);
+          const float rc = c == 0 ? r.rx : (c == 1 ? r.ry : r.rz), oc = c == 0 ? r.orx : (c == 1 ? r.ory : r.orz);
+          if (N::kGrid) {
+            const uint32_t sel = N::kElem == 1 ? (0x7540u | b) : (0x7400u | ((b + 1u) << 4) | b);
+            const float nb = __uint_as_float(__byte_perm(nw[c], 0x4B000000u, sel));
+            const float fb = __uint_as_float(__byte_perm(fw[c], 0x4B000000u, sel));
+            const float ac = c == 0 ? ax : (c == 1 ? ay : az), bc = c == 0 ? bx : (c == 1 ? by : bz);
+            if (kPaired) {
+              float nq, fq;
+              unbias_pair(nb, fb, nq, fq);
+              fma_pair(nq, fq, ac, bc, t0[c], t1[c]);
+            } else {
+              t0[c] = fmaf(nb - 8388608.0f, ac, bc);
+              t1[c] = fmaf(fb - 8388608.0f, ac, bc);
+            }
           } else {
-            t0[c] = fmaf((neg ? hb : lb) - 8388608.0f, ac, bc);
-            t1[c] = fmaf((neg ? lb : hb) - 8388608.0f, ac, bc);
+            const float nv = __half2float(__ushort_as_half((unsigned short)((nw[c] >> (b * 8)) & 0xFFFFu)));
+            const float fv = __half2float(__ushort_as_half((unsigned short)((fw[c] >> (b * 8)) & 0xFFFFu)));
+            t0[c] = fmaf(nv, rc, -oc);
+            t1[c] = fmaf(fv, rc, -oc);
           }
         }
-        hit = slab_t(r, t0[0], t0[1], t0[2], t1[0], t1[1], t1[2], tlim, tn);
-      } else {
-        float lo[3], hi[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const uint32_t ql = N::raw(q, k, c), qh = N::raw(q, k, c + 3);
-          if (PREC == PREC_F32) {
-            lo[c] = __uint_as_float(ql);
-            hi[c] = __uint_as_float(qh);
-          } else {
-            lo[c] = __half2float(__ushort_as_half((unsigned short)ql));
-            hi[c] = __half2float(__ushort_as_half((unsigned short)qh));
-          }
-        }
-        hit = slab<false>(r, lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], tlim, tn);
+        float tn;
+        bool hit = slab_t(r, t0[0], t0[1], t0[2], t1[0], t1[1], t1[2], tlim, tn);
+        hit = hit && ref != kEmptyRef;
+        cref[k] = hit ? ref : kEmptyRef;
+        ctn[k] = hit ? tn : __int_as_float(0x7f800000);
       }
-      hit = hit && ref != kEmptyRef;
-      cref[k] = hit ? ref : kEmptyRef;
-      ctn[k] = hit ? tn : __int_as_float(0x7f800000);
     }
-    }
-    if (!ANY && a.ordered == 1) {
-      sort_children<W>(ctn, cref);
-    } else if (!ANY && a.ordered == 2) {
-      // nearest first, the rest in slot order: move the nearest hit child
-      // into slot 0 (one pass of compare-exchanges toward the front)
+  } else {
 #pragma unroll
-      for (int k = W - 1; k > 0; --k) cmpx(ctn, cref, k - 1, k);
-    }
-    // push every hit child but the first, last one first; go on with the first
-    uint32_t next = kEmptyRef;
-    float next_tn = 0.f;
-    if (S::kRegs == 0 && st.sp - st.base + W <= st.cap_sh) {
-      // room in shared memory for any node: predicated stores, one check
-      int sp = st.sp;
-      if (!ANY && a.ordered) {
-        // the nearest child is in slot 0 (a child entered at +inf may not be:
-        // it is then stacked with the others and popped below)
+  for (int k = 0; k < W; ++k) {
+    const uint32_t ref = child_ref(k);
+    float tn;
+    bool hit;
+    if (N::kGrid) {
+      // per axis: near and far code of the child (decoded in one paired
+      // add), then both plane distances in one paired fma
+      float t0[3], t1[3];
 #pragma unroll
-        for (int k = W - 1; k > 0; --k)
-          if (cref[k] != kEmptyRef) st.sh_put(st.slot(sp++), make_uint2(cref[k], __float_as_uint(ctn[k])));
-        next = cref[0];
-      } else {
-#pragma unroll
-        for (int k = W - 1; k >= 0; --k) {
-          const bool h = cref[k] != kEmptyRef;
-          if (h && next != kEmptyRef) st.sh_put(st.slot(sp++), make_uint2(next, __float_as_uint(next_tn)));
-          next = h ? cref[k] : next;
-          next_tn = h ? ctn[k] : next_tn;
+      for (int c = 0; c < 3; ++c) {
+        const bool neg = c == 0 ? r.nx : (c == 1 ? r.ny : r.nz);
+        const float lb = N::code_biased(q, k, c), hb = N::code_biased(q, k, c + 3);
+        const float ac = c == 0 ? ax : (c == 1 ? ay : az), bc = c == 0 ? bx : (c == 1 ? by : bz);
+        if (kPaired) {
+          float nq, fq;
+          unbias_pair(neg ? hb : lb, neg ? lb : hb, nq, fq);
+          fma_pair(nq, fq, ac, bc, t0[c], t1[c]);
+        } else {
+          t0[c] = fmaf((neg ? hb : lb) - 8388608.0f, ac, bc);
+          t1[c] = fmaf((neg ? lb : hb) - 8388608.0f, ac, bc);
         }
       }
-      st.sp = sp;
+      hit = slab_t(r, t0[0], t0[1], t0[2], t1[0], t1[1], t1[2], tlim, tn);
+    } else {
+      float lo[3], hi[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const uint32_t ql = N::raw(q, k, c), qh = N::raw(q, k, c + 3);
+        if (PREC == PREC_F32) {
+          lo[c] = __uint_as_float(ql);
+          hi[c] = __uint_as_float(qh);
+        } else {
+          lo[c] = __half2float(__ushort_as_half((unsigned short)ql));
+          hi[c] = __half2float(__ushort_as_half((unsigned short)qh));
+        }
+      }
+      hit = slab<false>(r, lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], tlim, tn);
+    }
+    hit = hit && ref != kEmptyRef;
+    cref[k] = hit ? ref : kEmptyRef;
+    ctn[k] = hit ? tn : __int_as_float(0x7f800000);
+  }
+  }
+  if (!ANY && a.ordered == 1) {
+    sort_children<W>(ctn, cref);
+  } else if (!ANY && a.ordered == 2) {
+    // nearest first, the rest in slot order: move the nearest hit child
+    // into slot 0 (one pass of compare-exchanges toward the front)
+#pragma unroll
+    for (int k = W - 1; k > 0; --k) cmpx(ctn, cref, k - 1, k);
+  }
+  // push every hit child but the first, last one first; go on with the first
+  uint32_t next = kEmptyRef;
+  float next_tn = 0.f;
+  if (S::kRegs == 0 && st.sp - st.base + W <= st.cap_sh) {
+    // room in shared memory for any node: predicated stores, one check
+    int sp = st.sp;
+    if (!ANY && a.ordered) {
+      // the nearest child is in slot 0 (a child entered at +inf may not be:
+      // it is then stacked with the others and popped below)
+#pragma unroll
+      for (int k = W - 1; k > 0; --k)
+        if (cref[k] != kEmptyRef) st.sh_put(st.slot(sp++), make_uint2(cref[k], __float_as_uint(ctn[k])));
+      next = cref[0];
     } else {
 #pragma unroll
       for (int k = W - 1; k >= 0; --k) {
-        if (cref[k] == kEmptyRef) continue;
-        if (next != kEmptyRef && !st.push(next, next_tn)) { L.err = kErrStack; L.cur = kEmptyRef; return; }
-        next = cref[k];
-        next_tn = ctn[k];
+        const bool h = cref[k] != kEmptyRef;
+        if (h && next != kEmptyRef) st.sh_put(st.slot(sp++), make_uint2(next, __float_as_uint(next_tn)));
+        next = h ? cref[k] : next;
+        next_tn = h ? ctn[k] : next_tn;
       }
     }
-    L.cur = next != kEmptyRef ? next : pop_next<ANY>(st, L.b.t);
+    st.sp = sp;
   } else {
-    // One triangle per step: the entry then names the leaf's remaining
-    // triangles (first + 1, count - 1), so a lane in a leaf holds its warp for
-    // one triangle test per step rather than for the whole leaf while the
-    // other lanes wait. The counting kernels test the whole leaf at once (the
-    // same triangles, so the same counts).
-    const uint32_t count = ref_leaf_count(cur);
-    constexpr bool kWhole = STATS;
-    if (visit_leaf<ANY, STATS>(a, r, ref_leaf_first(cur), kWhole ? count : 1u, L.b, cnt)) {
-      L.found = true;
-      L.cur = kEmptyRef;
-      return;
+#pragma unroll
+    for (int k = W - 1; k >= 0; --k) {
+      if (cref[k] == kEmptyRef) continue;
+      if (next != kEmptyRef && !st.push(next, next_tn)) { L.err = kErrStack; L.cur = kEmptyRef; return; }
+      next = cref[k];
+      next_tn = ctn[k];
     }
-    if (!kWhole && count > 1u) {
-      L.cur = cur + (1u << 5) - (1u << 1);  // ref_leaf(first + 1, count - 1)
-      return;
-    }
-    L.cur = pop_next<ANY>(st, L.b.t);
   }
+  L.cur = next != kEmptyRef ? next : pop_next<ANY>(st, L.b.t);
+}
+
+// Leaf entry L.cur: one triangle, after which the entry names the leaf's other
+// triangles (first + 1, count - 1), so that a long leaf does not hold the warp.
+// The counting kernels test the whole leaf at once (the same triangles, so the
+// same counts).
+template <bool ANY, bool STATS, class S>
+__device__ __forceinline__ void leaf_wide(const TraceArgs &a, Lane &L, S &st, Counts &cnt) {
+  const uint32_t count = ref_leaf_count(L.cur);
+  if (visit_leaf<ANY, STATS>(a, L.r, ref_leaf_first(L.cur), STATS ? count : 1u, L.b, cnt)) {
+    L.found = true;
+    L.cur = kEmptyRef;
+    return;
+  }
+  if (!STATS && count > 1u) L.cur += (1u << 5) - (1u << 1);  // ref_leaf(first + 1, count - 1)
+  else L.cur = pop_next<ANY>(st, L.b.t);
 }
 
 // Exact small-integer to float conversions with full-rate integer ops: the
@@ -932,22 +971,8 @@ __device__ __forceinline__ void bin_pop(const TraceArgs &a, Lane &L, S &st) {
 // rays 0.586 -> 0.430 ms, bounce rays 0.846 -> 0.570 ms; q16 nodes, 1 M short
 // any-hit rays in 2 M random triangles: 0.841 -> 0.718 ms.
 template <int PREC, int SOA, int CREF, bool ANY, bool STATS, class S>
-__device__ __forceinline__ void step_bin(const TraceArgs &a, Lane &L, S &st, Counts &cnt) {
+__device__ __forceinline__ void node_bin(const TraceArgs &a, Lane &L, S &st, Counts &cnt) {
   const Ray &r = L.r;
-  if (L.count > 0) {
-    // one triangle per step, as the wide nodes (the counting kernels: all)
-    if (visit_leaf<ANY, STATS>(a, r, L.field, STATS ? L.count : 1u, L.b, cnt)) {
-      L.found = true;
-      L.cur = kEmptyRef;
-      return;
-    }
-    if (!STATS && --L.count > 0) {
-      ++L.field;
-      return;
-    }
-    bin_pop<PREC, SOA, ANY>(a, L, st);
-    return;
-  }
   if (STATS) cnt.nodes += 2;
   const uint32_t l = CREF == REF_DIRECT ? L.cur + 1 : L.field;
   const uint32_t rr = CREF == REF_DIRECT ? L.cur + L.field : L.field + 1;
@@ -967,6 +992,19 @@ __device__ __forceinline__ void step_bin(const TraceArgs &a, Lane &L, S &st, Cou
   L.cur = right ? rr : l;
   L.count = right ? rc : lc;
   L.field = right ? rf : lf;
+}
+
+// Leaf of an own-box query: one triangle, as the wide nodes (the counting
+// kernels: all).
+template <int PREC, int SOA, bool ANY, bool STATS, class S>
+__device__ __forceinline__ void leaf_bin(const TraceArgs &a, Lane &L, S &st, Counts &cnt) {
+  if (visit_leaf<ANY, STATS>(a, L.r, L.field, STATS ? L.count : 1u, L.b, cnt)) {
+    L.found = true;
+    L.cur = kEmptyRef;
+    return;
+  }
+  if (!STATS && --L.count > 0) ++L.field;
+  else bin_pop<PREC, SOA, ANY>(a, L, st);
 }
 
 // Shared-slab binary node (Section 8.3): the node's box is not stored; the
@@ -1070,12 +1108,26 @@ using StackFor = StackT<OWN && PREC == PREC_SLAB, (OWN && PREC != PREC_SLAB) || 
                         (OWN && PREC == PREC_SLAB) || !ANY>;
 
 // ------------------------------------------------------------------ kernel body
-// Trace one ray to completion with the layout's step function.
+// A step of the layout's traversal. A ray of more than max_steps visits ends with
+// an error.
 template <bool OWN, int W, int PREC, int SOA, int CREF, bool ANY, bool STATS, class S>
 __device__ __forceinline__ void step_any_layout(const TraceArgs &a, Lane &L, S &st, Counts &cnt) {
-  if constexpr (OWN && PREC == PREC_SLAB) step_slab<CREF, ANY, STATS>(a, L, st, cnt);
-  else if constexpr (OWN) step_bin<PREC, SOA, CREF, ANY, STATS>(a, L, st, cnt);
-  else step_wide<W, PREC, SOA, CREF, ANY, STATS>(a, L, st, cnt);
+  if constexpr (OWN && PREC == PREC_SLAB) {
+    ++L.steps;
+    step_slab<CREF, ANY, STATS>(a, L, st, cnt);
+  } else if constexpr (OWN) {
+    node_then_leaf<2>(
+        L, [&] { return L.count > 0; }, [&] { node_bin<PREC, SOA, CREF, ANY, STATS>(a, L, st, cnt); },
+        [&] { leaf_bin<PREC, SOA, ANY, STATS>(a, L, st, cnt); });
+  } else {
+    node_then_leaf<W <= 4 ? 2 : 1>(
+        L, [&] { return !ref_is_interior(L.cur); }, [&] { node_wide<W, PREC, SOA, CREF, ANY, STATS>(a, L, st, cnt); },
+        [&] { leaf_wide<ANY, STATS>(a, L, st, cnt); });
+  }
+  if (L.steps > a.max_steps) {
+    L.err = kErrIter;
+    L.cur = kEmptyRef;
+  }
 }
 
 // ------------------------------------------------------------------ work
@@ -1135,8 +1187,7 @@ __device__ __forceinline__ void batch_loop(const TraceArgs &a, Q &q) {
     const unsigned long long rid = slot_ray(a, slot);
     if (rid >= a.n) continue;
     q.start(a, rid);
-    while (q.busy())
-      if (!q.step(a)) break;
+    while (q.busy()) q.step(a);
     q.finish(a);
   }
   release_blocks(a);
@@ -1145,9 +1196,9 @@ __device__ __forceinline__ void batch_loop(const TraceArgs &a, Q &q) {
 // refill_loop: once at least refill_min lanes of the warp are idle they take
 // the next rays of the warp's block (then of the next block) while the others
 // are mid-ray. Every lane steps kFreeSteps times between two checks: the vote
-// brings the whole warp together, and measured (8.4 M random rays in 8.4 M
-// triangles, 4-wide u8 nodes) 1, 2, 4 and 8 steps take 9.20, 8.97, 8.87 and
-// 9.1 ms. A finished lane keeps its result until the refill, so results leave
+// brings the whole warp together, and measured (750,000 shadow rays in 1.4 M
+// triangles, bvh4 f32, 4 idle lanes) 1, 2 and 4 steps take 470, 465 and 448 us;
+// 8.4 M random rays in 8.4 M triangles (bvh4 u8) 7.36, 7.43 and 7.34 ms. A finished lane keeps its result until the refill, so results leave
 // and rays enter with many lanes at a time.
 constexpr int kFreeSteps = 4;
 template <class Q>
@@ -1222,15 +1273,8 @@ struct TraceQuery {
       if (OWN && PREC != PREC_SLAB && a.n_nodes > 0) cnt.nodes++;  // the root
     }
   }
-  // false: the step limit ended the ray
-  __device__ __forceinline__ bool step(const TraceArgs &a) {
-    if (++L.steps > a.max_steps) {
-      L.err = kErrIter;
-      L.cur = kEmptyRef;
-      return false;
-    }
+  __device__ __forceinline__ void step(const TraceArgs &a) {
     step_any_layout<OWN, W, PREC, SOA, CREF, ANY, STATS>(a, L, st, cnt);
-    return true;
   }
   __device__ __forceinline__ void finish(const TraceArgs &a) {
     if (L.err) atomicCAS(a.status, 0u, L.err);

@@ -204,6 +204,35 @@ def test_edge_cases(sc_mod, oracle_mod):
     assert_same_hits(gpu_closest(sc_mod, b, rays), oracle_mod.closest_brute(v.reshape(-1, 9), rays), "nonfinite")
 
 
+@pytest.mark.parametrize("fetch", [0, 4])
+@pytest.mark.parametrize("kw", [dict(box_prec="f32"), dict(box_prec="q16"), dict(box_prec="slab"),
+                                dict(width=4, box_layout="soa"), dict(width=8, box_prec="u8")], ids=str)
+def test_step_limit_counts_single_visits(sc_mod, kw, fetch):
+    """max_steps is a limit on a ray's visits (nodes and triangles; the shared slab's leaf is one), whatever a
+    kernel does per step: a ray that makes just as many finishes, with one fewer it is an error."""
+    sc = scenes.config1_scene()
+    rays = scenes.config1_rays()[::len(scenes.config1_rays()) // 40]
+    bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
+    own = kw.get("width", 2) == 2
+    visits = []
+    for r in rays:
+        nodes, _, prims, _ = sc_mod.scion_trace_stats(bvh, torch.from_numpy(r[None].copy()).cuda(), 0)[1].tolist()
+        if kw.get("box_prec") == "slab":
+            visits.append(nodes)
+        elif own:  # the counters' nodes are the boxes tested: the root's and two per interior node
+            visits.append((nodes - 1) // 2 + prims)
+        else:
+            visits.append(nodes + prims)
+    visits = np.array(visits)
+    want = gpu_closest(sc_mod, bvh, rays)
+    for limit in sorted(set(visits[visits > 0]) | set(v - 1 for v in visits if v > 1)):
+        got = gpu_closest(sc_mod, bvh, rays, params=dict(max_steps=int(limit), rays_per_fetch=fetch))
+        over = visits > limit
+        assert np.array_equal(got["prim"] == 0xFFFFFFFE, over)
+        assert_same_hits(got[~over], want[~over], "within the limit")
+        assert sc_mod.scion_get_status(bvh) == (6 if over.any() else 0)
+
+
 def test_device_errors_are_reported_not_faulted(sc_mod):
     """A tiny step limit and a stack deeper than the traversal stack end the
     affected rays with prim = ERROR and a status code; nothing faults."""
