@@ -151,12 +151,13 @@ typedef struct {
  *                      child first and the others in slot order.
  *  rays_per_fetch    : 0 (or 32) = each warp takes 32 consecutive rays and
  *                      traces them to completion; k in 1..31 = a warp
- *                      refills its idle lanes as soon as at least k of them
- *                      are idle (32-ray blocks are dealt to the CTAs
- *                      round-robin, rays handed out from a shared-memory
- *                      counter; k = 1 refills a lane at the next step).
- *                      Results are identical; which is faster depends on the
- *                      layout and the rays. Above 32: SCION_ERR_INVALID_ARG.
+ *                      refills its idle lanes from its block of rays, and
+ *                      then the next block, once at least k of them are idle
+ *                      (looked at every few steps). Launches with too few
+ *                      rays to give every warp 32 take smaller blocks, or
+ *                      one ray per warp, whatever k. Results are identical;
+ *                      which is faster depends on the layout and the rays.
+ *                      Above 32: SCION_ERR_INVALID_ARG.
  *  max_steps         : per-ray node+leaf visit limit (0 = derived from size).
  *  raster_width      : 0, or the rays are a row-major image this many rays
  *                      wide (ray i is pixel (i mod w, i / w); the last row
@@ -221,14 +222,15 @@ scion_status scion_build_many(const float *verts, uint64_t n_verts, const uint32
  * Karras (2012) and boxes bottom-up; a subtree of at most leaf_max triangles
  * becomes one leaf where the surface area heuristic prefers it to splitting
  * (sah_bins is not used). The tree is then packed
- * into `desc` by the same host packers as scion_build.
+ * into `desc` on the GPU, into the bytes that the host packers give for it
+ * (treelet order and the shared-slab node: by the host packers).
  *  d_verts   : float [n_verts][3], DEVICE memory (read, not retained).
  *  d_indices : uint32 [n_tris][3] in DEVICE memory, or NULL for a soup.
  *  stream    : stream for the build kernels and copies; the call returns
  *              after they complete.
- * Device scratch of about 180 bytes per triangle is allocated for the
- * duration of the call. Errors as scion_build; host pointers give
- * INVALID_ARG. */
+ * Device scratch of about 180 bytes per triangle is taken for the duration of
+ * the call from a memory pool of the library, which keeps up to 512 MB of it
+ * for the next call. Errors as scion_build; host pointers give INVALID_ARG. */
 scion_status scion_build_gpu(const float *d_verts, uint64_t n_verts, const uint32_t *d_indices,
                              uint64_t n_tris, const scion_layout_desc *desc, scion_stream stream,
                              scion_bvh *out);
@@ -256,7 +258,7 @@ scion_status scion_refit(scion_bvh bvh, const float *d_verts, uint64_t n_verts, 
 
 /* Build timings of a BVH in milliseconds: logical_ms = construction of the
  * logical BVH2 (host wall time of the binned-SAH builder, or device time of
- * scion_build_gpu's kernels); pack_ms = host packing into the layout. Either
+ * scion_build_gpu's kernels); pack_ms = packing into the layout. Either
  * pointer may be NULL. */
 scion_status scion_bvh_build_times(scion_bvh bvh, double *logical_ms, double *pack_ms);
 
@@ -298,8 +300,9 @@ scion_status scion_trace_any(scion_bvh bvh, const scion_ray *d_rays, uint64_t n,
  *  d_grad_rays    : device scion_ray-shaped float[n][8] receiving dL/d(o, d)
  *                   (tmin and tmax entries are 0), or NULL.
  * Missed rays (prim = SCION_PRIM_MISS) and errored rays contribute nothing.
- * The per-ray 3x3 solve is done in double precision. Every buffer must be
- * device memory (the gradients are scattered with device atomics), else
+ * The per-ray 3x3 solve is done in single precision and refined once with a
+ * residual of about twice that; where that is singular or out of range, in
+ * double precision. Every buffer must be device memory (the gradients are scattered with device atomics), else
  * SCION_ERR_INVALID_ARG. */
 scion_status scion_trace_backward(scion_bvh bvh, const scion_ray *d_rays, const scion_hit *d_hits,
                                   const float *d_grad_tuv, uint64_t n, float *d_grad_verts,

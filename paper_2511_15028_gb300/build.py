@@ -22,6 +22,9 @@ LIB = os.path.join(BUILD, "libscion.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "--fmad=false", "-prec-div=true", "-prec-sqrt=true", "-ftz=false",
+              # nvcc compresses device code above a size that the kernel families are at; a family's first launch
+              # in a process then unpacks it (9.0 ms instead of 2.3)
+              "--no-compress",
               "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off", "-I", INCLUDE]
 CXX_FLAGS = ["-O2", "-std=c++17", "-fPIC", "-fopenmp", "-ffp-contract=off", "-fno-fast-math",
              "-Wall", "-I", INCLUDE]

@@ -229,10 +229,16 @@ void set_raster(TraceArgs &a, uint32_t raster_w) {
 // against this rule: 1,000 rays 43.6 -> 31.1 us, 4,000 53.9 -> 43.4, 16,000
 // 68.2 -> 55.8, 40,000 68.2 -> 59.9; at 80,000 blocks of 16 are slower (70 ->
 // 79 us), and there the rule leaves 32.
-void small_launch(TraceArgs &a, uint64_t resident_warps) {
+// Closest points refill, and with one to two blocks a warp some take one block and
+// some two of work that varies from point to point: they get blocks of 16. Around
+// 1.4 M triangles, 32 against 16: 220,000 points 1,426 -> 1,315 us (bvh4 f32),
+// 300,000 1,534 -> 1,507 (bvh2 q16 2,070 -> 1,964); no gain at 600,000 (2,278,
+// 2,302), nor for rays (bounce rays at 200,000 189 -> 197).
+void small_launch(TraceArgs &a, uint64_t resident_warps, bool points) {
   a.chunk = 32;
   while (a.chunk > 1 && a.n_work / a.chunk < resident_warps / 2) a.chunk >>= 1;
   if (a.chunk < 32) a.refill_min = 32;
+  else if (points && a.n_work / 32 >= resident_warps && a.n_work / 32 < 2 * resident_warps) a.chunk = 16;
 }
 
 // Shared-memory stack bytes per entry, as StackFor (trace.cuh) chooses them:
@@ -506,22 +512,24 @@ struct TraceLaunch {
   uint32_t ctas_param = 0;  // scion_trace_params.ctas_per_sm (0: from occupancy)
   uint32_t reg_stack = 0;   // register entries at the top of the stack
   bool coop = false;        // one query per warp
+  bool points = false;      // closest points
 };
 
 // One query per warp (coop.cuh) instead of one per lane, for launches too small to
 // fill the GPU with lanes. Where the line lies, in queries per resident warp
 // (4,864 on this part), from both kernels measured on trees of 2 K to 1.4 M
 // triangles:
-//  - rays: 4, for 8-wide nodes 6. At 16,000 camera rays 70 -> 37 us (bvh4 f32), 89
-//    -> 55 (bvh2 f32); at 20,000 random rays 46 -> 32 (bvh4, closest), 60 -> 48
-//    (bvh2 q16), 50 -> 26 (bvh8 u8, any hit); even at 20,000 short any-hit rays
-//    in bvh2 q16 (67, 69), 40,000 random ones in bvh4 (50, 50) and 48,000 camera
-//    rays (81, 86).
-//  - points: (log2 of the triangles - 6)^2 / 5, for own-box nodes / 6, 8-wide
-//    nodes / 4: a point in a large tree is long work. 1,000 points in 50 K
-//    triangles 170 -> 42 us, 20,000 in 1.4 M 647 -> 212; even at 30,000 in 2 K
-//    (105, 107), past it at 100,000 in 30 K (425, 487) and at 200,000 in 1.4 M
-//    (1,542, 1,511; bvh8 f16 2,144, 1,645).
+//  - rays: 4, for 8-wide nodes 6. At 19,000 camera rays in 1.4 M triangles 66 -> 37
+//    us (bvh4 f32), 76 -> 48 (bvh2 f32); at 19,000 random rays 188 -> 100 (bvh4,
+//    closest, 2 M triangles), 119 -> 92 (bvh2 q16, 30 K), 177 -> 57 (bvh8 u8, any
+//    hit, 2 M), 82 -> 66 (short any-hit rays, bvh2 q16); of these the last is the
+//    first to turn, at 28,000 (74, 92).
+//  - points: (log2 of the triangles - 4)^2 / 10, for own-box nodes / 12, 8-wide
+//    nodes / 8: a point in a large tree is long work. bvh4 f32: 20,000 points in
+//    30 K triangles 232 -> 123 us, 60,000 in 1.4 M 851 -> 492; even at 27,000 in
+//    2 K, 58,000 in 30 K and 185,000 in 1.4 M (1,301, 1,213 at 160,000; 1,441,
+//    1,572 at 210,000). bvh2 q16: even at 19,000, 47,000 and 120,000; bvh8 f16:
+//    34,000 in 2 K and 75,000 in 30 K.
 // Only with the default launch shape, stack and step limit, which are parameters of
 // the per-lane kernels, and only for trees that cannot overflow those kernels'
 // stack, so that what they report as an error stays one.
@@ -533,9 +541,9 @@ void use_coop(const scion_bvh b, const scion_trace_params &p, int query, TraceLa
   const bool eight = !b->own_box && b->desc.width == 8;
   uint64_t most = warps * (eight ? 6 : 4);
   if (query == kQueryPoint) {
-    uint64_t l = 6;
+    uint64_t l = 4;
     while (l < 31 && (1ull << l) < b->n_leaf_entries) ++l;
-    most = std::max<uint64_t>(warps, warps * (l - 6) * (l - 6) / (eight ? 4 : (b->own_box ? 6 : 5)));
+    most = std::max<uint64_t>(warps, warps * (l - 4) * (l - 4) / (eight ? 8 : (b->own_box ? 12 : 10)));
   }
   if (L->a.n > most) return;
   const TraceKernel k = pick_coop_kernel(b, query);
@@ -634,6 +642,7 @@ scion_status prepare_trace(scion_bvh b, const scion_ray *rays, uint64_t n, void 
   a.stack_need = b->stack_need;
   L->ctas_param = p.ctas_per_sm;
   L->reg_stack = p.reg_stack;
+  L->points = query == kQueryPoint;
   use_coop(b, p, query, L);
   return SCION_OK;
 }
@@ -651,7 +660,7 @@ scion_status issue_trace(TraceLaunch &L, cudaStream_t stream, TraceKernel k) {
   }
   const uint64_t resident = (uint64_t)ctas * device_sms(dev), warps = L.tpb / 32;
   if (L.coop) L.a.chunk = 1;
-  else small_launch(L.a, resident * warps);
+  else small_launch(L.a, resident * warps, L.points);
   const uint64_t blocks = (L.a.n_work + L.a.chunk - 1) / L.a.chunk;
   L.grid = std::min<uint64_t>(resident, (blocks + warps - 1) / warps);
   void *args[] = {&L.a};
@@ -1280,7 +1289,7 @@ scion_status scion_batch_create(const scion_bvh *bvhs, const scion_ray *const *d
     const uint64_t resident = (uint64_t)std::max(nb, 1) * device_sms(dev), warps = bt->threads / 32;
     TraceArgs whole{};
     whole.n_work = total;
-    if (one_family) small_launch(whole, resident * warps);
+    if (one_family) small_launch(whole, resident * warps, false);
     else whole.chunk = kBatchUnit;
     bt->chunk = whole.chunk;
     const uint64_t units = total / bt->chunk;

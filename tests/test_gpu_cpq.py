@@ -74,6 +74,18 @@ def test_config1_every_layout_per_lane(sc_mod, config1_points, kw):
     assert sc_mod.scion_get_status(bvh) == 0
 
 
+@pytest.mark.parametrize("n", [155_648, 200_001, 311_295])
+def test_one_to_two_blocks_per_warp(sc_mod, config1_points, n):
+    """Between one and two blocks of 32 points for each of 4,864 warps the blocks are halved: every point once."""
+    sc, pts, exp = config1_points
+    many, exp = np.tile(pts, (39, 1))[:n], np.tile(exp, 39)[:n]
+    for kw in (dict(box_prec="q16"), dict(width=4, box_layout="soa"), dict(width=8, box_prec="u8")):
+        bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
+        for _ in range(2):  # the counters are ready for the next launch
+            same(query(sc_mod, bvh, many), exp, f"{kw} {n}")
+        assert sc_mod.scion_get_status(bvh) == 0
+
+
 def test_radius_surface_far_and_nonfinite_points(sc_mod, oracle_mod):
     sc = scenes.config1_scene()
     tris = sc.triangles()
