@@ -35,6 +35,9 @@ CANDIDATE_PARAMS = {"ordered": {}, "slot_order": {"ordered_children": 2},
                     "nearest_first_refill8": {"ordered_children": 3, "rays_per_fetch": 8}}
 
 
+FILL = 1 << 18  # rays of a timed launch at least
+
+
 @dataclass
 class Choice:
     name: str
@@ -92,6 +95,9 @@ class Autotuner:
         n = rays.shape[0]
         step = max(1, n // self.sample)
         sample = rays[::step][: self.sample].contiguous()
+        # as many times over as fill the GPU: a launch of few rays is split differently (smaller blocks, or a
+        # ray per warp) and would favour the layouts with the shortest chain of loads, not the fastest ones
+        sample = sample.repeat(max(1, -(-FILL // max(1, sample.shape[0]))), 1)
         out = torch.empty((sample.shape[0], 4), dtype=torch.int32, device=rays.device)
         times = {}
         for name, bvh in zip(names, bvhs):

@@ -185,8 +185,8 @@ void bvh_args(const scion_bvh b, TraceArgs &a) {
 constexpr size_t kSmemOptIn = 32 * 1024;
 
 // Closest point queries are refilled once this many lanes of a warp are idle
-// (1 M random points around 1.4 M triangles, bvh4 f32: 3.65 ms at 4 lanes, 3.68
-// at 8; 5.90 ms in whole batches of 32).
+// (1 M random points around 1.4 M triangles, bvh4 f32: 3.33 ms at 4 lanes, 3.37
+// at 1, 3.34 at 8; whole batches of 32 took 5.90 when a step was one visit).
 constexpr uint32_t kCpRefill = 4;
 
 // Query kinds of launch_trace.

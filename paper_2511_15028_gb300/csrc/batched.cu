@@ -19,7 +19,8 @@
 // scene's arguments from global memory, which is why it is not used for both.
 // Measured, 48 scenes of one family (1.6 M rays): bvh4 u8 batches 839 -> 775 us,
 // refill 1,319 -> 847; bvh4 f32 refill 1,342 -> 854; bvh8 u8 1,131 -> 954; bvh2 q16
-// refill 2,511 -> 1,198; 5 small scenes 121 -> 68. One large scene runs within 4 %
+// refill 2,511 -> 1,198; 5 small scenes 121 -> 68 (48 scenes, bvh4 u8, with the
+// steps of node_then_leaf: 707). One large scene runs within 4 %
 // of its plain launch (refill: twice as long before).
 // The launch allocates nothing and never synchronises the host, so it can be
 // captured in a CUDA graph and replayed; its counters reset themselves.
@@ -34,9 +35,21 @@ namespace {
 
 constexpr int kMaxSharedScenes = 1024;  // scene starts cached in shared memory
 
+// One visit per step: the steps of node_then_leaf spill 30 to 60 % more here
+// (64 scenes of three families, 7.2 M rays: 4.39 -> 3.79 to 4.16 ms).
 template <bool OWN, int W, int PREC, int SOA>
 __device__ __forceinline__ void step_family(const TraceArgs &a, Lane &L, Stack &st, Counts &cnt) {
-  step_any_layout<OWN, W, PREC, SOA, REF_DIRECT, false, false>(a, L, st, cnt);
+  if constexpr (OWN) {
+    if (L.count > 0) leaf_bin<PREC, SOA, false, false>(a, L, st, cnt);
+    else node_bin<PREC, SOA, REF_DIRECT, false, false>(a, L, st, cnt);
+  } else {
+    if (ref_is_interior(L.cur)) node_wide<W, PREC, SOA, REF_DIRECT, false, false>(a, L, st, cnt);
+    else leaf_wide<false, false>(a, L, st, cnt);
+  }
+  if (++L.steps > a.max_steps) {
+    L.err = kErrIter;
+    L.cur = kEmptyRef;
+  }
 }
 
 // The next 32-ray unit of the global index space (warp-uniform).

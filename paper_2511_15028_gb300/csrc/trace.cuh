@@ -18,6 +18,8 @@
 // part, conflict-free) and whose tail spills to local memory, or, where a
 // kernel has the register for it, whose shared part is a ring of the most
 // recent entries (StackT). The current entry is always in registers.
+// A step of a lane is a few nodes, then a few triangles (node_then_leaf). Launches
+// of few rays give each a whole warp instead (coop.cuh).
 //
 // Arithmetic: the box test only has to be conservative; the triangle test is
 // pinned bit for bit (see tri_test). Translation units are compiled with
@@ -961,15 +963,15 @@ __device__ __forceinline__ void bin_pop(const TraceArgs &a, Lane &L, S &st) {
   if (L.cur != kEmptyRef) own_ref<PREC, SOA>(a, L.cur, L.count, L.field);
 }
 
-// One step of the own-box binary traversal. The lane is at a node whose box
-// it has entered and whose reference it holds: a leaf tests its triangles; an
-// interior node loads both children at once, tests their boxes, enters the
-// nearer of those hit (any hit and slot order: the left) and stacks the other
-// with its entry distance. Testing a node only when it is reached, as the
+// Interior node of the own-box binary traversal. The lane is at a node whose box
+// it has entered and whose reference it holds: it loads both children at once,
+// tests their boxes, enters the nearer of those hit (any hit and slot order: the
+// left) and stacks the other with its entry distance. Testing a node only when it is reached, as the
 // node's own box suggests, costs a dependent load, a push and a pop for every
-// second child, hit or not. Measured (1.4 M triangles, f32 nodes, 1080p): camera
-// rays 0.586 -> 0.430 ms, bounce rays 0.846 -> 0.570 ms; q16 nodes, 1 M short
-// any-hit rays in 2 M random triangles: 0.841 -> 0.718 ms.
+// second child, hit or not. Measured, with a node or a triangle per step on both
+// sides (1.4 M triangles, f32 nodes, 1080p): camera rays 0.586 -> 0.430 ms, bounce
+// rays 0.846 -> 0.570 ms; q16 nodes, 1 M short any-hit rays in 2 M random
+// triangles: 0.841 -> 0.718 ms.
 template <int PREC, int SOA, int CREF, bool ANY, bool STATS, class S>
 __device__ __forceinline__ void node_bin(const TraceArgs &a, Lane &L, S &st, Counts &cnt) {
   const Ray &r = L.r;
