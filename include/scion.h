@@ -389,13 +389,14 @@ scion_status scion_trace_closest_noalloc(scion_bvh bvh, const scion_ray *d_rays,
  * defaults) into a device table (it allocates and uploads; synchronous on
  * `stream`). threads_per_block and smem_stack are taken from per_scene[0];
  * each scene's ordered_children, rays_per_fetch (warp batches or warp
- * refill, applied within the 256-ray chunks a warp takes) and max_steps are
+ * refill, applied within the blocks of rays a warp takes) and max_steps are
  * its own. raster_width and reg_stack are plain-launch parameters: non-zero
  * values give SCION_ERR_INVALID_ARG.
  * Scenes whose layout is one of the batched node families (width-2 own-box
  * AoS with f32 or q16 boxes, width-4 SoA with f32, f16 or u8 boxes, width-8
  * SoA f16, width-8 u8 AoS or SoA, each with direct child references;
- * triangles direct or indirect) run in one persistent kernel; any other scene
+ * triangles direct or indirect) run in one persistent kernel, or, where the
+ * batch has many rays and several of the families, in one per family; any other scene
  * gets its own plain launch from scion_batch_launch.
  * The pointers are captured: the buffers must stay valid until the batch is
  * destroyed.

@@ -35,7 +35,7 @@ CANDIDATE_PARAMS = {"ordered": {}, "slot_order": {"ordered_children": 2},
                     "nearest_first_refill8": {"ordered_children": 3, "rays_per_fetch": 8}}
 
 
-FILL = 1 << 18  # rays of a timed launch at least
+FILL = 1 << 17  # rays of a timed launch at least
 
 
 @dataclass
@@ -52,7 +52,7 @@ class Autotuner:
     one scene and its ray sample), so the choice is what the batched launch
     will run; `plain=True` times plain launches instead."""
 
-    def __init__(self, prim_refs=("direct",), params=None, sample: int = 8192, reps: int = 3,
+    def __init__(self, prim_refs=("direct",), params=None, sample: int = 1 << 17, reps: int = 3,
                  layouts=None, plain: bool = False):
         self.descs = {}
         for name, kw in (layouts or CANDIDATE_LAYOUTS).items():

@@ -13,8 +13,9 @@
 // Where all scenes have one node family, as an autotuned batch usually does, a
 // kernel of that family runs (batched_body in batched.cuh, instantiated beside
 // the family's other kernels): its loops are the plain launch's, with the
-// scene's arguments in shared memory. Scenes of several families run in the
-// kernel below, which dispatches with a warp-uniform switch over functions of
+// scene's arguments in shared memory. A batch of several families with enough
+// rays is launched a family at a time (split_batch in api.cu); a smaller one runs in
+// the kernel below, which dispatches with a warp-uniform switch over functions of
 // their own; those spill 200 to 300 bytes under the 64-register cap and read the
 // scene's arguments from global memory, which is why it is not used for both.
 // Measured, 48 scenes of one family (1.6 M rays): bvh4 u8 batches 839 -> 775 us,

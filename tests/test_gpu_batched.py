@@ -225,3 +225,26 @@ def test_batched_one_family(mods, oracle_mod, kw, scale, n_scenes):
                 exp = oracle_mod.BVH2(sc.triangles()).closest(r)
                 assert scion.split_hits(hits[i]).tobytes() == exp.tobytes(), (i, params[i])
                 assert scion.scion_get_status(bvhs[i]) == 0
+
+
+@pytest.mark.parametrize("n", [100_000, 116_736 + 33, 233_477])
+def test_batched_split_by_family(mods, oracle_mod, n):
+    """Batches of two families around the size from which each family has a launch of its own (4 scenes, 467,000
+    rays in all on 152 SMs), scenes of the families in turn: hits equal the oracle's, also when launched again."""
+    scion, _ = mods
+    sc = scenes.config1_scene()
+    r = scenes.config1_rays()
+    many, exp = np.tile(r, (15, 1)), np.tile(oracle_mod.BVH2(sc.triangles()).closest(r), 15)
+    kws = [dict(width=4, box_layout="soa"), dict(box_prec="q16")] * 2
+    bvhs = [scion.scion_build(sc.verts, scion.layout(**kw), sc.indices) for kw in kws]
+    rays = [torch.from_numpy(many[i:i + n]).cuda() for i in range(4)]
+    batch = scion.Batch(bvhs, rays, params=[{}, dict(rays_per_fetch=4), dict(rays_per_fetch=8), {}])
+    for _ in range(2):
+        for h in batch.hits:
+            h.fill_(-1)
+        hits = batch.launch()
+        torch.cuda.synchronize()
+        for i in range(4):
+            assert scion.split_hits(hits[i]).tobytes() == exp[i:i + n].tobytes(), i
+            assert scion.scion_get_status(bvhs[i]) == 0
+    assert batch.info() == dict(batched_scenes=4, plain_scenes=0)
