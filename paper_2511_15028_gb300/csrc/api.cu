@@ -46,8 +46,8 @@ struct scion_bvh_s {
   cudaStream_t slot_stream[kStreamSlotCount] = {};
   double build_ms = 0.0, logical_ms = 0.0, pack_ms = 0.0;
   int device = 0;
-  // refit scratch, allocated by the first scion_refit; refit_linked: it holds
-  // the nodes' parents and counters
+  // refit scratch, allocated by the first scion_refit; refit_linked: a launch
+  // that writes the nodes' parents and counters into it has been issued
   bool refit_linked = false;
   uint32_t *d_refit_parent = nullptr, *d_refit_pending = nullptr;
   void *d_refit_boxes = nullptr;
@@ -1016,7 +1016,12 @@ scion_status scion_refit(scion_bvh bvh, const float *d_verts, uint64_t n_verts, 
   rb.frame = b->d_refit_frame;
   rb.status = b->d_scratch + 3;
   SCION_CUDA(refit_launch(rb, d_verts, s));
-  b->refit_linked = true;
+  // A launch that is only recorded into a graph computes no links until the graph
+  // runs, if it ever does: they are kept from the first launch that is issued. (An
+  // error here is a capture on another stream; it says nothing of this one.)
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
+  else if (capture == cudaStreamCaptureStatusNone) b->refit_linked = true;
   if (prec_has_frame(b->desc.box_prec) && b->n_nodes > 0) {
     // the traversal takes the grid as a launch argument: read it back
     SCION_CUDA(cudaMemcpyAsync(b->frame, b->d_refit_frame, 9 * sizeof(float), cudaMemcpyDeviceToHost, s));

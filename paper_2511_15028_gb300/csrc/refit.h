@@ -19,9 +19,9 @@ struct RefitBuffers {
   uint64_t n_verts;
   bool own_box;
   scion_layout_desc desc;
-  // refit scratch (device): n_nodes parents and counters (written by the
-  // BVH's first refit and kept), n_nodes boxes of 24 bytes, 18 floats of world
-  // grid (q16/eq10)
+  // refit scratch (device): n_nodes parents and counters, n_nodes boxes of 24
+  // bytes, 18 floats of world grid (q16/eq10). first: the parents and counters
+  // are still to be written; later refits find them as this one leaves them.
   bool first;
   uint32_t *parent, *pending;
   void *boxes;

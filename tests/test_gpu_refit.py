@@ -91,6 +91,33 @@ def test_refit_back_and_soup_and_gpu_built(sc_mod, oracle_mod):
         check(sc_mod, oracle_mod, bvh, v, None, r, f"gpu-built soup refit {k}")
 
 
+@pytest.mark.parametrize("kw", [dict(), dict(width=2, box_prec="f16"), dict(width=4, box_layout="soa", child_ref="indirect"),
+                                dict(width=8, box_prec="u8")], ids=str)
+def test_first_refit_captured_into_a_graph(sc_mod, oracle_mod, kw):
+    """A BVH's first refit recorded into a CUDA graph has not run: refits issued before the first replay, after it
+    and once the graph is gone find the nodes' links for themselves."""
+    sc = scenes.config1_scene()
+    bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
+    rays = scenes.config1_rays()
+    v = [moved(sc.verts, amp) for amp in (0.1, 0.2, 0.3, 0.15)]
+    d = [torch.from_numpy(x).cuda() for x in v]
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s, capture_error_mode="relaxed"):  # the first refit allocates
+        sc_mod.scion_refit(bvh, d[0], stream=s)
+    torch.cuda.synchronize()
+    sc_mod.scion_refit(bvh, d[1])
+    check(sc_mod, oracle_mod, bvh, v[1], sc.indices, rays, f"{kw} issued before the replay")
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    check(sc_mod, oracle_mod, bvh, v[0], sc.indices, rays, f"{kw} replayed")
+    sc_mod.scion_refit(bvh, d[2])
+    check(sc_mod, oracle_mod, bvh, v[2], sc.indices, rays, f"{kw} issued after the replay")
+    del g
+    sc_mod.scion_refit(bvh, d[3])
+    check(sc_mod, oracle_mod, bvh, v[3], sc.indices, rays, f"{kw} the graph gone")
+
+
 def test_refit_nonfinite_and_arguments(sc_mod, oracle_mod):
     sc = scenes.config1_scene()
     rays = scenes.config1_rays()
