@@ -217,17 +217,25 @@ __device__ __forceinline__ int own_box_words(uint32_t prec) { return prec == PRE
 // ------------------------------------------------------------ u8 / u16 frames
 // Smallest e >= -126 with qmax 2^e >= span, span = fhi - origin > 0 (the loop of
 // encode_wide_boxes ends there too).
+SCION_SLOW int frame_exponent_slow(float fhi, float origin, uint32_t qmax) {
+  const double span = (double)fhi - (double)origin;
+  int e = -126;
+  while (e < 127 && ldexp((double)qmax, e) < span) ++e;
+  return e;
+}
 SCION_HD int frame_exponent(float fhi, float origin, uint32_t qmax) {
   const FPair s = two_sum(fhi, -origin);
   if (!(s.hi > 0.0f)) return -126;
+  // below, every qmax 2^e up to the one that is returned is a finite float
+  if (!(s.hi < 1e33f)) return frame_exponent_slow(fhi, origin, qmax);
   const int es = (int)((float_bits(s.hi) >> 23) & 255u) - 127;  // 2^es <= s.hi < 2^(es + 1)
   int e = es - (qmax == 255u ? 8 : 16);
   if (e < -126) e = -126;
-  while (e < 127) {
-    // qmax 2^e is a float while it does not overflow; its equality with the
-    // leading part is left to the trailing part (rounded away in double only
-    // where it is below 2^-52 of the span)
-    const float reach = e <= 127 - 16 ? (float)qmax * pow2f(e) : INFINITY;
+  while (true) {
+    // qmax 2^e is a float; its equality with the leading part is left to the
+    // trailing part (rounded away in double only where it is below 2^-52 of the
+    // span)
+    const float reach = (float)qmax * pow2f(e);
     if (reach > s.hi || (reach == s.hi && s.lo <= s.hi * 1.1102230246251565e-16f)) break;
     ++e;
   }

@@ -1,6 +1,7 @@
 """The FP32 box codecs of the device encoders (codec_fast.h) give the bytes of
 the double-precision codecs (codec.h): both compiled for the host and compared
-on random and degenerate boxes (flat, dyadic, at zero, huge and tiny scales)."""
+on random and degenerate boxes (flat, dyadic, at zero, scales from denormal
+numbers to the largest floats)."""
 import os
 import subprocess
 
@@ -64,8 +65,12 @@ static long differs(const Box3 *v, int n, uint32_t soa) {
 int main() {
   long pad = 0, grid = 0, wide = 0;
   for (int it = 0; it < 60000; ++it) {
-    const int mode = rng() % 9, n = 1 + rng() % 8;
-    const double sc = mode == 1 ? std::pow(10, U(-30, 30)) : (mode == 2 ? 1e-3 : (mode == 3 ? 1e4 : 1));
+    const int mode = rng() % 12, n = 1 + rng() % 8;
+    double sc = mode == 2 ? 1e-3 : (mode == 3 ? 1e4 : 1);
+    if (mode == 1) sc = std::pow(10, U(-30, 30));
+    if (mode == 9) sc = std::pow(2, U(98, 127.99));  // extents to twice the largest float
+    if (mode == 10) sc = std::pow(2, U(-149, -100));
+    if (mode == 11) sc = std::ldexp(1.0, 100 + (int)(rng() % 28));
     Box3 v[8];
     double c[3];
     for (double &x : c) x = mode == 4 ? 0 : U(-1, 1) * sc;
@@ -78,8 +83,8 @@ int main() {
         if (mode == 6) l = std::floor(U(-64, 64)) / 32;
         if (mode == 7) l = std::floor(U(-8, 8));
         if (mode == 8 && rng() % 3 == 0) l = 0;
-        v[k].lo[a] = (float)l;
-        v[k].hi[a] = fmaxf((float)(l + w), v[k].lo[a]);
+        v[k].lo[a] = fminf(fmaxf((float)l, -3.4028235e38f), 3.4028235e38f);
+        v[k].hi[a] = fminf(fmaxf((float)(l + w), v[k].lo[a]), 3.4028235e38f);
       }
       if (rng() % 40 == 0) v[k].lo[0] = INFINITY, v[k].hi[0] = -INFINITY;
       if (box_is_empty(v[k])) continue;

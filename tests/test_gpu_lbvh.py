@@ -179,6 +179,27 @@ def test_gpu_packer_bytes_equal_host_packer(sc_mod):
                 _same_bytes(scion, got, ref, f"{kw} leaf_max={leaf_max} indexed={ix is not None}")
 
 
+@pytest.mark.parametrize("exp", [-100, 100, 118, 121, 124, 125])
+def test_build_and_refit_of_tiny_and_huge_scenes(sc_mod, exp):
+    """Scenes scaled by powers of two, which change no sorting key and no leaf choice: the GPU packer's bytes, and
+    those of the unscaled scene's tree refit to the scaled vertices, equal the host packer's (the codecs of codec.h),
+    and no code fails to enclose its box."""
+    scion = sc_mod
+    sc = scenes.config1_scene()
+    ix = torch.from_numpy(sc.indices.astype(np.int32)).cuda()
+    scaled = torch.from_numpy(np.ldexp(sc.verts, exp)).cuda()
+    for kw in (dict(width=8, box_prec="u8"), dict(width=4, box_layout="soa", box_prec="u8", order="bfs"),
+               dict(width=2, box_prec="u16"), dict(width=8, box_prec="u16", box_layout="soa"), dict(box_prec="q16"),
+               dict(width=4, box_layout="soa"), dict()):
+        desc = scion.layout(prim_ref="direct", **kw)
+        ref = scion.scion_build_gpu(scaled, desc, ix, host_pack=True)
+        _same_bytes(scion, scion.scion_build_gpu(scaled, desc, ix), ref, f"{kw} built")
+        moved = scion.scion_build_gpu(torch.from_numpy(sc.verts).cuda(), desc, ix)
+        scion.scion_refit(moved, scaled)
+        _same_bytes(scion, moved, ref, f"{kw} refit")
+        assert scion.scion_get_status(moved) == 0
+
+
 def test_gpu_packer_full_size(sc_mod, oracle_mod):
     """2^23 random triangles: the GPU packer's bytes equal the host packer's
     for the layouts the benchmark sweeps in both orders and one of each
