@@ -158,7 +158,12 @@ typedef struct {
  *                      one ray per warp, whatever k. Results are identical;
  *                      which is faster depends on the layout and the rays.
  *                      Above 32: SCION_ERR_INVALID_ARG.
- *  max_steps         : per-ray node+leaf visit limit (0 = derived from size).
+ *  max_steps         : per-ray limit on visits (0 = derived from size): of nodes
+ *                      and leaf triangles (closest points and the counting
+ *                      kernels: leaves) in wide trees; of nodes in own-box and
+ *                      shared-slab trees, a trace's visit of an own-box node
+ *                      being the test of its box (the root's, and both
+ *                      children's of every interior node entered).
  *  raster_width      : 0, or the rays are a row-major image this many rays
  *                      wide (ray i is pixel (i mod w, i / w); the last row
  *                      may be partial): each warp then traces an 8 x 4 pixel

@@ -47,7 +47,7 @@ __device__ __forceinline__ void step_family(const TraceArgs &a, Lane &L, Stack &
     if (ref_is_interior(L.cur)) node_wide<W, PREC, SOA, REF_DIRECT, false, false>(a, L, st, cnt);
     else leaf_wide<false, false>(a, L, st, cnt);
   }
-  if (++L.steps > a.max_steps) {
+  if (L.steps > a.max_steps) {
     L.err = kErrIter;
     L.cur = kEmptyRef;
   }

@@ -191,13 +191,18 @@ __device__ __forceinline__ uint32_t cp_pop(const CpLane &L, S &st) {
   return kEmptyRef;
 }
 
-// Leaf entry: one triangle, as the ray traversal (the counting kernels: all).
+// Leaf entry: one triangle, as the ray traversal (the counting kernels: all). A
+// leaf is one visit, counted with its last triangle.
 template <bool STATS, class S>
 __device__ __forceinline__ void cp_leaf_wide(const TraceArgs &a, CpLane &L, S &st, Counts &cnt) {
   const uint32_t count = ref_leaf_count(L.cur);
   cp_leaf<STATS>(a, L, ref_leaf_first(L.cur), STATS ? count : 1u, cnt);
-  if (!STATS && count > 1u) L.cur += (1u << 5) - (1u << 1);  // ref_leaf(first + 1, count - 1)
-  else L.cur = cp_pop(L, st);
+  if (!STATS && count > 1u) {
+    L.cur += (1u << 5) - (1u << 1);  // ref_leaf(first + 1, count - 1)
+    return;
+  }
+  ++L.steps;
+  L.cur = cp_pop(L, st);
 }
 
 // Interior node: bound every child box, enter the nearest, stack the others
@@ -206,6 +211,7 @@ template <int W, int PREC, int SOA, int CREF, bool STATS, class S>
 __device__ __forceinline__ void cp_node_wide(const TraceArgs &a, CpLane &L, S &st, Counts &cnt) {
   using N = WideNode<W, PREC, SOA, CREF>;
   const uint32_t cur = L.cur;
+  ++L.steps;
   if (STATS) cnt.nodes++;
   const uint4 *np = a.nodes + (size_t)ref_node(cur) * (N::kStride / 16);
   uint4 q[N::NQ];
@@ -296,8 +302,12 @@ template <int PREC, int SOA, bool STATS, class S>
 __device__ __forceinline__ void cp_leaf_bin(const TraceArgs &a, CpLane &L, S &st, Counts &cnt) {
   if (STATS) cnt.nodes++;
   cp_leaf<STATS>(a, L, L.field, STATS ? L.count : 1u, cnt);
-  if (!STATS && --L.count > 0) ++L.field;
-  else cp_bin_pop<PREC, SOA>(a, L, st);
+  if (!STATS && --L.count > 0) {
+    ++L.field;
+    return;
+  }
+  ++L.steps;
+  cp_bin_pop<PREC, SOA>(a, L, st);
 }
 
 // Own-box interior node (the entered node's box was bounded by its parent):
@@ -305,6 +315,7 @@ __device__ __forceinline__ void cp_leaf_bin(const TraceArgs &a, CpLane &L, S &st
 // and stacks the other.
 template <int PREC, int SOA, int CREF, bool STATS, class S>
 __device__ __forceinline__ void cp_node_bin(const TraceArgs &a, CpLane &L, S &st, Counts &cnt) {
+  ++L.steps;
   if (STATS) cnt.nodes++;
   const uint32_t l = CREF == REF_DIRECT ? L.cur + 1 : L.field;
   const uint32_t r = CREF == REF_DIRECT ? L.cur + L.field : L.field + 1;

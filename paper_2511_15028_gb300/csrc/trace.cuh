@@ -642,14 +642,14 @@ __device__ __forceinline__ void sort_children(float (&t)[W], uint32_t (&r)[W]) {
 // waiting the soups gain less (677 and 7,997 us), the others the same; a share of
 // 4 is 1 to 2 % slower. NODES is 2, for 8-wide nodes 1: their code twice costs more
 // than it gives (bounce rays 501 us).
-// A lane makes the same visits in the same order as one by one; `steps` counts them.
+// A lane makes the same visits in the same order as one by one; node() and leaf()
+// count them in `steps`, in the units of max_steps (scion.h).
 constexpr uint32_t kLeafShare = 2;
 template <int NODES, class LaneT, class AtLeaf, class Node, class Leaf>
 __device__ __forceinline__ void node_then_leaf(LaneT &L, AtLeaf at_leaf, Node node, Leaf leaf) {
 #pragma unroll
   for (int i = 0; i < NODES; ++i) {
     if (L.cur != kEmptyRef && !at_leaf()) {
-      ++L.steps;
       node();
     }
   }
@@ -661,7 +661,6 @@ __device__ __forceinline__ void node_then_leaf(LaneT &L, AtLeaf at_leaf, Node no
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     if (L.cur != kEmptyRef && at_leaf()) {
-      ++L.steps;
       leaf();
     }
   }
@@ -674,6 +673,7 @@ __device__ __forceinline__ void node_wide(const TraceArgs &a, Lane &L, S &st, Co
   using N = WideNode<W, PREC, SOA, CREF>;
   const Ray &r = L.r;
   const uint32_t cur = L.cur;
+  ++L.steps;
   if (STATS) cnt.nodes++;
   const uint4 *np = a.nodes + (size_t)ref_node(cur) * (N::kStride / 16);
   uint4 q[N::NQ];
@@ -854,6 +854,7 @@ __device__ __forceinline__ void node_wide(const TraceArgs &a, Lane &L, S &st, Co
 template <bool ANY, bool STATS, class S>
 __device__ __forceinline__ void leaf_wide(const TraceArgs &a, Lane &L, S &st, Counts &cnt) {
   const uint32_t count = ref_leaf_count(L.cur);
+  ++L.steps;
   if (visit_leaf<ANY, STATS>(a, L.r, ref_leaf_first(L.cur), STATS ? count : 1u, L.b, cnt)) {
     L.found = true;
     L.cur = kEmptyRef;
@@ -975,6 +976,7 @@ __device__ __forceinline__ void bin_pop(const TraceArgs &a, Lane &L, S &st) {
 template <int PREC, int SOA, int CREF, bool ANY, bool STATS, class S>
 __device__ __forceinline__ void node_bin(const TraceArgs &a, Lane &L, S &st, Counts &cnt) {
   const Ray &r = L.r;
+  L.steps += 2;  // both children's boxes
   if (STATS) cnt.nodes += 2;
   const uint32_t l = CREF == REF_DIRECT ? L.cur + 1 : L.field;
   const uint32_t rr = CREF == REF_DIRECT ? L.cur + L.field : L.field + 1;
@@ -997,7 +999,7 @@ __device__ __forceinline__ void node_bin(const TraceArgs &a, Lane &L, S &st, Cou
 }
 
 // Leaf of an own-box query: one triangle, as the wide nodes (the counting
-// kernels: all).
+// kernels: all). No further visit: the leaf's box was counted at its parent.
 template <int PREC, int SOA, bool ANY, bool STATS, class S>
 __device__ __forceinline__ void leaf_bin(const TraceArgs &a, Lane &L, S &st, Counts &cnt) {
   if (visit_leaf<ANY, STATS>(a, L.r, L.field, STATS ? L.count : 1u, L.b, cnt)) {
@@ -1092,6 +1094,7 @@ __device__ __forceinline__ void start_ray(const TraceArgs &a, Lane &L) {
     L.ctf = tf;
   } else if constexpr (OWN) {
     L.cur = kEmptyRef;
+    L.steps = 1;  // the root's box
     if (a.n_nodes > 0) {
       float lo[3], hi[3], tn;
       own_node<PREC, SOA>(a, 0u, lo, hi, L.count, L.field);

@@ -136,6 +136,29 @@ def test_soup_gpu_built_refit_and_counting(sc_mod, oracle_mod):
     assert e.value.status == 2  # unsupported layout
 
 
+@pytest.mark.parametrize("kw", [dict(), dict(box_prec="q16"), dict(width=4, box_layout="soa"), dict(width=8, box_prec="u8")],
+                         ids=str)
+def test_step_limit_counts_nodes_and_leaves(sc_mod, config1_points, kw):
+    """max_steps limits a point's visits of nodes (own-box trees, whose leaves are nodes) or of nodes and leaves
+    (wide trees), however many triangles a leaf has: a point with just as many finishes, with one fewer it is an
+    error."""
+    sc, pts, exp = config1_points
+    pts, exp = pts[::len(pts) // 40], exp[::len(pts) // 40]
+    bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(leaf_max=8, **kw), sc.indices)
+    visits = []
+    for p in pts:
+        nodes, leaves, _, _ = sc_mod.scion_trace_stats(bvh, torch.from_numpy(p[None].copy()).cuda(), 2)[1].tolist()
+        visits.append(nodes + (leaves if "width" in kw else 0))
+    visits = np.array(visits)
+    for limit in sorted(set(visits[visits > 0]) | set(v - 1 for v in visits if v > 1)):
+        got = sc_mod.split_hits(sc_mod.scion_query_closest_point(bvh, torch.from_numpy(pts).cuda(),
+                                                                 params=dict(max_steps=int(limit))))
+        over = visits > limit
+        assert np.array_equal(got["prim"] == 0xFFFFFFFE, over)
+        same(got[~over].view(np.uint32).reshape(-1, 4), exp[~over], "within the limit")
+        assert sc_mod.scion_get_status(bvh) == (6 if over.any() else 0)
+
+
 def test_points_in_pinned_host_memory(sc_mod, config1_points):
     """Query points and results in pinned host memory, read and written by the
     kernel in place: the same records as from device buffers."""

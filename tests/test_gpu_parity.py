@@ -208,8 +208,9 @@ def test_edge_cases(sc_mod, oracle_mod):
 @pytest.mark.parametrize("kw", [dict(box_prec="f32"), dict(box_prec="q16"), dict(box_prec="slab"),
                                 dict(width=4, box_layout="soa"), dict(width=8, box_prec="u8")], ids=str)
 def test_step_limit_counts_single_visits(sc_mod, kw, fetch):
-    """max_steps is a limit on a ray's visits (nodes and triangles; the shared slab's leaf is one), whatever a
-    kernel does per step: a ray that makes just as many finishes, with one fewer it is an error."""
+    """max_steps is a limit on a ray's visits (wide trees: nodes and leaf triangles; own-box trees: boxes tested, the
+    root's and two per interior node; the shared slab: nodes), whatever a kernel does per step: a ray that makes just
+    as many finishes, with one fewer it is an error."""
     sc = scenes.config1_scene()
     rays = scenes.config1_rays()[::len(scenes.config1_rays()) // 40]
     bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
@@ -217,12 +218,7 @@ def test_step_limit_counts_single_visits(sc_mod, kw, fetch):
     visits = []
     for r in rays:
         nodes, _, prims, _ = sc_mod.scion_trace_stats(bvh, torch.from_numpy(r[None].copy()).cuda(), 0)[1].tolist()
-        if kw.get("box_prec") == "slab":
-            visits.append(nodes)
-        elif own:  # the counters' nodes are the boxes tested: the root's and two per interior node
-            visits.append((nodes - 1) // 2 + prims)
-        else:
-            visits.append(nodes + prims)
+        visits.append(nodes if own else nodes + prims)
     visits = np.array(visits)
     want = gpu_closest(sc_mod, bvh, rays)
     for limit in sorted(set(visits[visits > 0]) | set(v - 1 for v in visits if v > 1)):
