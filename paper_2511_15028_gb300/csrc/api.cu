@@ -524,12 +524,16 @@ struct TraceLaunch {
 //    closest, 2 M triangles), 119 -> 92 (bvh2 q16, 30 K), 177 -> 57 (bvh8 u8, any
 //    hit, 2 M), 82 -> 66 (short any-hit rays, bvh2 q16); of these the last is the
 //    first to turn, at 28,000 (74, 92).
-//  - points: (log2 of the triangles - 4)^2 / 10, for own-box nodes / 12, 8-wide
-//    nodes / 8: a point in a large tree is long work. bvh4 f32: 20,000 points in
-//    30 K triangles 232 -> 123 us, 60,000 in 1.4 M 851 -> 492; even at 27,000 in
-//    2 K, 58,000 in 30 K and 185,000 in 1.4 M (1,301, 1,213 at 160,000; 1,441,
-//    1,572 at 210,000). bvh2 q16: even at 19,000, 47,000 and 120,000; bvh8 f16:
-//    34,000 in 2 K and 75,000 in 30 K.
+//  - points: (log2 of the triangles - 4)^2 / 18 and at most 7, for own-box nodes / 25
+//    and 6, 8-wide nodes / 15 and 9: a point in a large tree is long work. Random
+//    points gain up to far more of them (bvh4 f32, 1.4 M triangles: 60,000 points
+//    851 -> 492 us, even at 185,000), but neighbours that take the same way share it
+//    lane by lane: 70,000 points of a frame's scan lines took 516 us a warp each
+//    against 279. The line is where points in image order take what whole batches of
+//    32 took. bvh2 f32, scan lines in 1.4 M triangles: 20,000 345 -> 239 us, 40,000
+//    378 -> 432; near the surface of 34 K 274 -> 192, 277 -> 342; of 2.7 K 10,000 75
+//    -> 64, 20,000 75 -> 112. bvh4 f32: even at 38,000, 43,000 and 18,000; bvh8 u8 at
+//    48,000, 50,000 and 21,000.
 // Only with the default launch shape, stack and step limit, which are parameters of
 // the per-lane kernels, and only for trees that cannot overflow those kernels'
 // stack, so that what they report as an error stays one.
@@ -543,7 +547,8 @@ void use_coop(const scion_bvh b, const scion_trace_params &p, int query, TraceLa
   if (query == kQueryPoint) {
     uint64_t l = 4;
     while (l < 31 && (1ull << l) < b->n_leaf_entries) ++l;
-    most = std::max<uint64_t>(warps, warps * (l - 4) * (l - 4) / (eight ? 8 : (b->own_box ? 12 : 10)));
+    const uint64_t div = eight ? 15 : (b->own_box ? 25 : 18), cap = eight ? 9 : (b->own_box ? 6 : 7);
+    most = warps * std::max<uint64_t>(div, std::min<uint64_t>((l - 4) * (l - 4), cap * div)) / div;
   }
   if (L->a.n > most) return;
   const TraceKernel k = pick_coop_kernel(b, query);
