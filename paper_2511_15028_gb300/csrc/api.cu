@@ -229,16 +229,10 @@ void set_raster(TraceArgs &a, uint32_t raster_w) {
 // against this rule: 1,000 rays 43.6 -> 31.1 us, 4,000 53.9 -> 43.4, 16,000
 // 68.2 -> 55.8, 40,000 68.2 -> 59.9; at 80,000 blocks of 16 are slower (70 ->
 // 79 us), and there the rule leaves 32.
-// Closest points refill, and with one to two blocks a warp some take one block and
-// some two of work that varies from point to point: they get blocks of 16. Around
-// 1.4 M triangles, 32 against 16: 220,000 points 1,426 -> 1,315 us (bvh4 f32),
-// 300,000 1,534 -> 1,507 (bvh2 q16 2,070 -> 1,964); no gain at 600,000 (2,278,
-// 2,302), nor for rays (bounce rays at 200,000 189 -> 197).
-void small_launch(TraceArgs &a, uint64_t resident_warps, bool points) {
+void small_launch(TraceArgs &a, uint64_t resident_warps) {
   a.chunk = 32;
   while (a.chunk > 1 && a.n_work / a.chunk < resident_warps / 2) a.chunk >>= 1;
   if (a.chunk < 32) a.refill_min = 32;
-  else if (points && a.n_work / 32 >= resident_warps && a.n_work / 32 < 2 * resident_warps) a.chunk = 16;
 }
 
 // Shared-memory stack bytes per entry, as StackFor (trace.cuh) chooses them:
@@ -512,7 +506,6 @@ struct TraceLaunch {
   uint32_t ctas_param = 0;  // scion_trace_params.ctas_per_sm (0: from occupancy)
   uint32_t reg_stack = 0;   // register entries at the top of the stack
   bool coop = false;        // one query per warp
-  bool points = false;      // closest points
 };
 
 // One query per warp (coop.cuh) instead of one per lane, for launches too small to
@@ -647,7 +640,6 @@ scion_status prepare_trace(scion_bvh b, const scion_ray *rays, uint64_t n, void 
   a.stack_need = b->stack_need;
   L->ctas_param = p.ctas_per_sm;
   L->reg_stack = p.reg_stack;
-  L->points = query == kQueryPoint;
   use_coop(b, p, query, L);
   return SCION_OK;
 }
@@ -665,7 +657,7 @@ scion_status issue_trace(TraceLaunch &L, cudaStream_t stream, TraceKernel k) {
   }
   const uint64_t resident = (uint64_t)ctas * device_sms(dev), warps = L.tpb / 32;
   if (L.coop) L.a.chunk = 1;
-  else small_launch(L.a, resident * warps, L.points);
+  else small_launch(L.a, resident * warps);
   const uint64_t blocks = (L.a.n_work + L.a.chunk - 1) / L.a.chunk;
   L.grid = std::min<uint64_t>(resident, (blocks + warps - 1) / warps);
   void *args[] = {&L.a};
@@ -1331,7 +1323,7 @@ scion_status scion_batch_create(const scion_bvh *bvhs, const scion_ray *const *d
     if (one_family) {
       TraceArgs whole{};
       whole.n_work = part.slots;
-      small_launch(whole, resident * warps, false);
+      small_launch(whole, resident * warps);
       part.chunk = whole.chunk;
     }
     const uint64_t units = part.slots / part.chunk;

@@ -413,7 +413,7 @@ __device__ __forceinline__ void cpq_kernel_body(const TraceArgs &a) {
   st.columns(smem_stack, a.smem_stack);
   st.reset();
   PointQuery<OWN, W, PREC, SOA, CREF, STATS, decltype(st)> q(st);
-  trace_loop(a, q);
+  trace_loop<true>(a, q);
   q.report(a);
 }
 

@@ -76,7 +76,7 @@ def test_config1_every_layout_per_lane(sc_mod, config1_points, kw):
 
 @pytest.mark.parametrize("n", [155_648, 200_001, 311_295])
 def test_one_to_two_blocks_per_warp(sc_mod, config1_points, n):
-    """Between one and two blocks of 32 points for each of 4,864 warps the blocks are halved: every point once."""
+    """Between one and two blocks of 32 points for each of 4,864 warps: every point once."""
     sc, pts, exp = config1_points
     many, exp = np.tile(pts, (39, 1))[:n], np.tile(exp, 39)[:n]
     for kw in (dict(box_prec="q16"), dict(width=4, box_layout="soa"), dict(width=8, box_prec="u8")):
@@ -134,6 +134,28 @@ def test_soup_gpu_built_refit_and_counting(sc_mod, oracle_mod):
     with pytest.raises(sc_mod.ScionError) as e:
         query(sc_mod, slab, pts)
     assert e.value.status == 2  # unsupported layout
+
+
+@pytest.mark.parametrize("n", [311_296, 400_003])
+def test_blocks_that_go_together_and_blocks_that_part(sc_mod, config1_points, n):
+    """Warps wait for whole blocks while their points take the same way and refill their lanes one by one while they
+    do not: blocks of one point (32 times and 31 times), of all kinds of points, and both in turn, with points that
+    find nothing among them; every point once."""
+    sc, pts, exp = config1_points
+    rng = np.random.default_rng(7)
+    far = np.concatenate([pts[:1], pts[:1]])
+    far[0, 3], far[1, 0] = -1.0, np.nan
+    pts, exp = np.concatenate([pts, far]), np.concatenate([exp, np.repeat(exp[:1], 2)])
+    exp[-2:] = (np.inf, 0.0, 0.0, 0xFFFFFFFF)
+    m = len(pts)
+    same_way, apart = np.repeat(rng.integers(0, m, n // 32 + 1), 32)[:n], rng.integers(0, m, n)
+    turns = np.where((np.arange(n) // 32) % 7 < 4, same_way, apart)
+    for kw in (dict(), dict(box_prec="q16", child_ref="indirect"), dict(width=4, box_layout="soa"),
+               dict(width=8, box_prec="u8")):
+        bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
+        for ix in (same_way, np.repeat(rng.integers(0, m, n // 31 + 1), 31)[:n], turns):
+            same(query(sc_mod, bvh, pts[ix]), exp[ix], f"{kw} {n}")
+        assert sc_mod.scion_get_status(bvh) == 0
 
 
 @pytest.mark.parametrize("kw", [dict(), dict(box_prec="q16"), dict(width=4, box_layout="soa"), dict(width=8, box_prec="u8")],
