@@ -500,11 +500,12 @@ __device__ __noinline__ bool leaf_is_cheaper(const TreeArgs &T, const Box3 &b, u
   return a * (double)cnt <= a + cl + cr;
 }
 
-// Box of node p from its children's, and where the subtree is small enough the
-// leaf choice (the children's costs only count for such a subtree).
+// Half the area, +inf where it overflows (also where an extent does and another is
+// 0): whoever compares it then takes the boxes.
 __device__ __forceinline__ float half_area(const Box3 &b) {
   const float ex = b.hi[0] - b.lo[0], ey = b.hi[1] - b.lo[1], ez = b.hi[2] - b.lo[2];
-  return ex * ey + ey * ez + ez * ex;
+  const float h = ex * ey + ey * ez + ez * ex;
+  return h >= 0.0f ? h : INFINITY;
 }
 // What a climb carries of a node and keeps of it in shared memory.
 struct Made {
@@ -512,6 +513,8 @@ struct Made {
   float cost;
   float open;  // half area, or -1: a logical leaf
 };
+// Box of node p from its children's, and where the subtree is small enough the
+// leaf choice (the children's costs only count for such a subtree).
 __device__ __forceinline__ Made make_node(const TreeArgs &T, uint32_t p, uint32_t l, uint32_t r, uint32_t cnt,
                                           const Made &ml, const Made &mr) {
   const Box3 &b0 = ml.b, &b1 = mr.b;

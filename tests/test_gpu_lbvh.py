@@ -200,6 +200,28 @@ def test_build_and_refit_of_tiny_and_huge_scenes(sc_mod, exp):
         assert scion.scion_get_status(moved) == 0
 
 
+def test_gpu_packer_where_extents_overflow(sc_mod):
+    """Flat triangles across the whole range of floats: extents overflow to infinity, and times a zero extent to NaN.
+    The GPU packer still opens the nodes that the host packer opens."""
+    scion = sc_mod
+    rng = np.random.default_rng(17)
+    v = rng.uniform(-1, 1, (1500, 3)).astype(np.float32)
+    v[:, 0] *= np.float32(3.3e38)
+    v[:, 2] = 0
+    d = torch.from_numpy(v).cuda()
+    for kw in (dict(width=4), dict(width=8), dict(width=8, box_prec="f16", order="bfs"), dict(width=8, box_prec="u16"),
+               dict(width=2, child_ref="indirect"), dict()):
+        desc = scion.layout(**kw)
+        try:
+            ref = scion.scion_build_gpu(d, desc, host_pack=True)
+        except scion.ScionError as e:  # codes that cannot enclose such boxes: both must refuse alike
+            with pytest.raises(scion.ScionError) as e2:
+                scion.scion_build_gpu(d, desc)
+            assert e2.value.status == e.status, kw
+            continue
+        _same_bytes(scion, scion.scion_build_gpu(d, desc), ref, str(kw))
+
+
 def test_gpu_packer_full_size(sc_mod, oracle_mod):
     """2^23 random triangles: the GPU packer's bytes equal the host packer's
     for the layouts the benchmark sweeps in both orders and one of each
