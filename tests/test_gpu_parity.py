@@ -229,6 +229,50 @@ def test_step_limit_counts_single_visits(sc_mod, kw, fetch):
         assert sc_mod.scion_get_status(bvh) == (6 if over.any() else 0)
 
 
+def caterpillars():
+    """Triangles whose radix tree over 30-bit Morton codes is 16 chains of 26 levels, each ending in 256 equal codes,
+    and rays through all the boxes: thin triangles along y = z whose boxes are all about [-1, 1]^3, a chain's next
+    node always nearer to a ray along +x than its leaf, so that a leaf per chain and level stays stacked. Taken 16
+    nodes at a time that is 518 entries of 512; one large triangle behind the boxes is hit."""
+    code, near = [], []
+    for chain in range(16):
+        code += [chain << 26 | 1 << b for b in range(26)] + [chain << 26] * 256
+        near += [-0.99 + 1e-4 * b for b in range(26)] + [-1.0] * 256
+    code, near = np.array(code), np.array(near)
+    cell = np.zeros((len(code), 3))
+    for i in range(30):  # bit 3m + 2 of a code is bit m of x, 3m + 1 of y, 3m of z
+        cell[:, 2 - i % 3] += (code >> i & 1) << i // 3
+    c = np.concatenate([cell + 0.5, [[0.0] * 3, [1024.0] * 3]]) * (0.1 / 1024)  # the last two span the grid
+    a = np.stack([np.append(near, [-1, -1]), np.full(len(c), -1), np.full(len(c), -1)], 1)
+    tri = np.stack([a, np.ones_like(a), 3 * c - a - 1], 1)  # centroids c
+    yz = np.array([[10, 0], [-5, 8], [-4.85, -7.85]])
+    back = np.concatenate([(0.05 + 1.08 * (yz[:, :1] - yz[:, 1:])), yz], 1)
+    verts = np.concatenate([tri.reshape(-1, 3), back]).astype(np.float32)
+    rng = np.random.default_rng(2)
+    o = np.stack([np.full(600, -20.0), rng.uniform(0.5, 0.95, 600), rng.uniform(-0.95, -0.5, 600)], 1)
+    rays = np.concatenate([o, np.zeros((600, 1)), np.tile([1.0, 0, 0], (600, 1)), np.full((600, 1), np.inf)], 1)
+    rays[200:400, 0], rays[200:400, 4] = 20.0, -1.0
+    rays[400:, 4:7] += rng.uniform(-0.01, 0.01, (200, 3))
+    rays[::3, 7] = 21.0  # ends between the boxes and the triangle behind them
+    return verts, rays.astype(np.float32)
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(box_prec="q16", child_ref="indirect"), dict(box_prec="eq10"),
+                                dict(width=2, box_prec="f16"), dict(width=2, box_prec="u8"),
+                                dict(width=4, box_layout="soa"), dict(width=8, box_prec="u8")], ids=str)
+def test_one_ray_per_warp_with_a_full_stack(sc_mod, oracle_mod, kw):
+    """A warp that has one ray takes many nodes at a time only while its stack has room for what the tree can need,
+    then one: trees that fill it give the oracle's hits."""
+    verts, rays = caterpillars()
+    bvh = sc_mod.scion_build_gpu(torch.from_numpy(verts).cuda(), sc_mod.layout(leaf_max=1, **kw))
+    tris = verts.reshape(-1, 9)
+    exp = oracle_mod.closest_brute(tris, rays)
+    assert 0.3 < np.mean(exp["prim"] == len(tris) - 1) < 0.9
+    assert_same_hits(gpu_closest(sc_mod, bvh, rays), exp, str(kw))
+    assert np.array_equal(gpu_any(sc_mod, bvh, rays), oracle_mod.any_brute(tris, rays))
+    assert sc_mod.scion_get_status(bvh) == 0
+
+
 def test_device_errors_are_reported_not_faulted(sc_mod):
     """A tiny step limit and a stack deeper than the traversal stack end the
     affected rays with prim = ERROR and a status code; nothing faults."""
