@@ -517,16 +517,15 @@ struct TraceLaunch {
 //    closest, 2 M triangles), 119 -> 92 (bvh2 q16, 30 K), 177 -> 57 (bvh8 u8, any
 //    hit, 2 M), 82 -> 66 (short any-hit rays, bvh2 q16); of these the last is the
 //    first to turn, at 28,000 (74, 92).
-//  - points: (log2 of the triangles - 4)^2 / 18 and at most 7, for own-box nodes / 25
-//    and 6, 8-wide nodes / 15 and 9: a point in a large tree is long work. Random
-//    points gain up to far more of them (bvh4 f32, 1.4 M triangles: 60,000 points
-//    851 -> 492 us, even at 185,000), but neighbours that take the same way share it
-//    lane by lane: 70,000 points of a frame's scan lines took 516 us a warp each
-//    against 279. The line is where points in image order take what whole batches of
-//    32 took. bvh2 f32, scan lines in 1.4 M triangles: 20,000 345 -> 239 us, 40,000
-//    378 -> 432; near the surface of 34 K 274 -> 192, 277 -> 342; of 2.7 K 10,000 75
-//    -> 64, 20,000 75 -> 112. bvh4 f32: even at 38,000, 43,000 and 18,000; bvh8 u8 at
-//    48,000, 50,000 and 21,000.
+//  - points: (log2 of the triangles - 4)^2 / 13 and at most 14, for own-box nodes / 15
+//    and 12, 8-wide nodes / 8 and 21: a point in a large tree is long work. What is
+//    best depends on the points' order, which a launch does not know: neighbours that
+//    take the same way share it lane by lane. At 70,000 points in 1.4 M triangles (bvh4
+//    f32, us, a warp each and a lane each): scan lines of a frame half way to the
+//    surface 516, 270, on the surface 555, 519; every fifth pixel 597, 349 and 636, 693;
+//    random 625, 899, sorted 567, 1,043. The line is where the geometric mean over
+//    these six is the same: for bvh4 f32 at 68,000 in 1.4 M, 52,000 in 34 K and 24,000
+//    in 2.7 K; bvh2 f32 62,000, 50,000, 18,000; bvh8 u8 102,000, 90,000, 42,000.
 // Only with the default launch shape, stack and step limit, which are parameters of
 // the per-lane kernels, and only for trees that cannot overflow those kernels'
 // stack, so that what they report as an error stays one.
@@ -540,7 +539,7 @@ void use_coop(const scion_bvh b, const scion_trace_params &p, int query, TraceLa
   if (query == kQueryPoint) {
     uint64_t l = 4;
     while (l < 31 && (1ull << l) < b->n_leaf_entries) ++l;
-    const uint64_t div = eight ? 15 : (b->own_box ? 25 : 18), cap = eight ? 9 : (b->own_box ? 6 : 7);
+    const uint64_t div = eight ? 8 : (b->own_box ? 15 : 13), cap = eight ? 21 : (b->own_box ? 12 : 14);
     most = warps * std::max<uint64_t>(div, std::min<uint64_t>((l - 4) * (l - 4), cap * div)) / div;
   }
   if (L->a.n > most) return;
