@@ -233,9 +233,11 @@ scion_status scion_build_many(const float *verts, uint64_t n_verts, const uint32
  *  d_indices : uint32 [n_tris][3] in DEVICE memory, or NULL for a soup.
  *  stream    : stream for the build kernels and copies; the call returns
  *              after they complete.
- * Device scratch of about 180 bytes per triangle is taken for the duration of
- * the call from a memory pool of the library, which keeps up to 512 MB of it
- * for the next call. Errors as scion_build; host pointers give INVALID_ARG. */
+ * Device scratch of up to 210 bytes per triangle, depending on the layout, is
+ * taken for the duration of the call from a memory pool of the library, which
+ * keeps up to 512 MB of it for the next call, until scion_release_scratch or
+ * until an allocation of the library finds the device full. Errors as
+ * scion_build; host pointers give INVALID_ARG. */
 scion_status scion_build_gpu(const float *d_verts, uint64_t n_verts, const uint32_t *d_indices,
                              uint64_t n_tris, const scion_layout_desc *desc, scion_stream stream,
                              scion_bvh *out);
@@ -430,6 +432,11 @@ scion_status scion_trace_batched(const scion_bvh *bvhs, const scion_ray *const *
 scion_status scion_get_status(scion_bvh bvh, scion_stream stream, scion_status *device_status);
 
 void scion_destroy(scion_bvh bvh);
+
+/* Gives the device scratch that the library keeps for the next scion_build_gpu
+ * on the current device back to the device (waits for the device's work).
+ * Errors: CUDA. */
+scion_status scion_release_scratch(void);
 
 const char *scion_status_string(scion_status s);
 

@@ -160,7 +160,7 @@ template <typename T>
 scion_status upload(void **dst, const std::vector<T> &src, cudaStream_t s, uint64_t *bytes) {
   *bytes = src.size() * sizeof(T);
   if (src.empty()) return SCION_OK;
-  SCION_CUDA(cudaMalloc(dst, *bytes));
+  SCION_CUDA(device_malloc(dst, *bytes));
   SCION_CUDA(cudaMemcpyAsync(*dst, src.data(), *bytes, cudaMemcpyHostToDevice, s));
   return SCION_OK;
 }
@@ -724,7 +724,7 @@ scion_status upload_bvh(HostBVH &hb, uint64_t n_tris, uint64_t n_verts, bool ind
   if (us == SCION_OK) us = upload(&b->d_verts, hb.verts4, s, &b->vert_bytes);
   if (us == SCION_OK) us = upload(&b->d_idx, hb.indices, s, &b->idx_bytes);
   if (us == SCION_OK) {
-    cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&b->d_scratch), kScratchBytes);
+    cudaError_t e = device_malloc(reinterpret_cast<void **>(&b->d_scratch), kScratchBytes);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_scratch, 0, kScratchBytes, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) us = e == cudaErrorMemoryAllocation ? SCION_ERR_OOM : cuda_fail(e);
@@ -977,10 +977,10 @@ scion_status scion_refit(scion_bvh bvh, const float *d_verts, uint64_t n_verts, 
   scion_bvh b = bvh;
   if (!b->d_refit_parent && b->n_nodes > 0) {
     const size_t n = b->n_nodes;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&b->d_refit_parent), n * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&b->d_refit_pending), n * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_refit_boxes, n * 6 * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&b->d_refit_frame), kRefitFrameFloats * sizeof(float));
+    cudaError_t e = device_malloc(reinterpret_cast<void **>(&b->d_refit_parent), n * sizeof(uint32_t));
+    if (e == cudaSuccess) e = device_malloc(reinterpret_cast<void **>(&b->d_refit_pending), n * sizeof(uint32_t));
+    if (e == cudaSuccess) e = device_malloc(&b->d_refit_boxes, n * 6 * sizeof(float));
+    if (e == cudaSuccess) e = device_malloc(reinterpret_cast<void **>(&b->d_refit_frame), kRefitFrameFloats * sizeof(float));
     if (e != cudaSuccess) {
       cudaFree(b->d_refit_parent);
       cudaFree(b->d_refit_pending);
@@ -1294,10 +1294,10 @@ scion_status scion_batch_create(const scion_bvh *bvhs, const scion_ray *const *d
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const size_t counter_bytes = 16 * std::max<size_t>(1, bt->parts.size());
-  cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&bt->d_counters), counter_bytes);
+  cudaError_t e = device_malloc(reinterpret_cast<void **>(&bt->d_counters), counter_bytes);
   if (e == cudaSuccess) e = cudaMemsetAsync(bt->d_counters, 0, counter_bytes, s);
   if (e == cudaSuccess && !table.empty()) {
-    e = cudaMalloc(reinterpret_cast<void **>(&bt->d_scenes), table.size() * sizeof(BatchScene));
+    e = device_malloc(reinterpret_cast<void **>(&bt->d_scenes), table.size() * sizeof(BatchScene));
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(bt->d_scenes, table.data(), table.size() * sizeof(BatchScene), cudaMemcpyHostToDevice, s);
   }
@@ -1403,6 +1403,12 @@ scion_status scion_get_status(scion_bvh b, scion_stream stream, scion_status *de
 }
 
 void scion_destroy(scion_bvh b) { free_bvh(b); }
+
+scion_status scion_release_scratch(void) {
+  SCION_CUDA(cudaDeviceSynchronize());  // scratch still in use is not given back
+  release_scratch();
+  return SCION_OK;
+}
 
 // ---------------------------------------------------------------- debug ABI
 struct scion_host_bvh_s {

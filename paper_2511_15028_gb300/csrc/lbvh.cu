@@ -664,6 +664,20 @@ cudaMemPool_t scratch_pool() {
 
 }  // namespace
 
+void release_scratch() {
+  if (const cudaMemPool_t pool = scratch_pool()) cudaMemPoolTrimTo(pool, 0);
+}
+
+cudaError_t device_malloc(void **p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    release_scratch();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
 Arena::~Arena() {
   if (!base_) return;
   if (pooled_) cudaFreeAsync(base_, stream_);
@@ -672,7 +686,7 @@ Arena::~Arena() {
 
 cudaError_t Arena::commit() {
   void *q = nullptr;
-  const cudaError_t e = cudaMalloc(&q, used_ ? used_ : 256);
+  const cudaError_t e = device_malloc(&q, used_ ? used_ : 256);
   base_ = static_cast<char *>(e == cudaSuccess ? q : nullptr);
   used_ = 0;
   return e;
@@ -685,7 +699,7 @@ cudaError_t Arena::commit(cudaStream_t stream) {
   const cudaError_t e = cudaMallocFromPoolAsync(&q, used_ ? used_ : 256, pool, stream);
   if (e != cudaSuccess) {  // e.g. the device is full but for what the pool keeps
     cudaGetLastError();
-    cudaMemPoolTrimTo(pool, 0);
+    release_scratch();
     return commit();
   }
   base_ = static_cast<char *>(q);

@@ -57,6 +57,11 @@ class Arena {
   cudaStream_t stream_ = nullptr;
 };
 
+// Gives back what the current device's pool keeps and no call uses.
+void release_scratch();
+// cudaMalloc, once more without what the pool keeps where the device is full.
+cudaError_t device_malloc(void **p, size_t bytes);
+
 // The logical BVH2 as the GPU builds it, left in device memory: the binary
 // radix tree over the nv valid triangles in Morton order. Interior node i in
 // [0, nv-2] has children left[i], right[i]; node ids >= nv-1 are radix

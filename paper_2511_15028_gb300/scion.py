@@ -181,7 +181,7 @@ def lib():
                      "scion_trace_stats", "scion_trace_backward", "scion_trace_backward_split",
                      "scion_split_hits", "scion_batch_create",
                      "scion_batch_launch", "scion_batch_info", "scion_trace_batched",
-                     "scion_get_status", "scion_debug_build_host", "scion_debug_host_stats",
+                     "scion_get_status", "scion_release_scratch", "scion_debug_build_host", "scion_debug_host_stats",
                      "scion_debug_host_decode", "scion_debug_host_raw"):
             getattr(L, name).restype = I
         _lib = L
@@ -694,6 +694,12 @@ def scion_get_status(bvh: BVH, stream=None) -> int:
     st = ctypes.c_int()
     _check(lib().scion_get_status(bvh.handle, _stream_ptr(stream), ctypes.byref(st)), "scion_get_status")
     return st.value
+
+
+def scion_release_scratch() -> None:
+    """Give the device scratch that the library keeps between scion_build_gpu
+    calls (512 MB at most) back to the current device."""
+    _check(lib().scion_release_scratch(), "scion_release_scratch")
 
 
 def scion_destroy(bvh: BVH):

@@ -126,6 +126,27 @@ def test_degenerate_inputs(sc_mod, oracle_mod):
     assert np.all(occluded(sc_mod, none, rays[:64]) == 0)
 
 
+def test_scratch_is_given_back(sc_mod):
+    """A build's scratch stays in the library's pool, 512 MB of it at most, until it is asked for; the next build
+    gives the same tree."""
+    scion = sc_mod
+    n = 1 << 21
+    d = torch.from_numpy(scenes.random_soup(scenes.rng_for(71), n, mu=math.log(0.004))).cuda()
+    desc = scion.layout(width=8, box_prec="u8")
+    scion.scion_release_scratch()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    before = scion.scion_build_gpu(d, desc)
+    torch.cuda.synchronize()
+    size = sum(x.size for x in scion.scion_debug_bvh_bytes(before)) + n * 3 * 16
+    kept = free - torch.cuda.mem_get_info()[0] - size
+    assert (100 << 20) < kept < (560 << 20)
+    scion.scion_release_scratch()
+    assert free - torch.cuda.mem_get_info()[0] - size < (40 << 20)
+    scion.scion_release_scratch()  # nothing left
+    _same_bytes(scion, scion.scion_build_gpu(d, desc), before, "after the scratch was given back")
+
+
 def test_invalid_arguments(sc_mod):
     base = np.array([[0, 0, 0], [1, 0, 0], [0, 1, 0]], np.float32)
     L = sc_mod.lib()
