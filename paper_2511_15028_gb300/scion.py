@@ -469,11 +469,16 @@ def _trace_fn():
             ctx.save_for_backward(rays, hits)
             ctx.bvh = bvh
             ctx.set_materialize_grads(False)  # a missing gradient is zero to the kernel
-            n = hits.shape[0]
-            t, u, v = (torch.empty(n, dtype=torch.float32, device=hits.device) for _ in range(3))
-            prim = torch.empty(n, dtype=torch.int32, device=hits.device)
-            _check(lib().scion_split_hits(hits.data_ptr(), n, t.data_ptr(), u.data_ptr(), v.data_ptr(),
-                                          prim.data_ptr(), _stream_ptr(None)), "scion_split_hits")
+            if hits.is_cuda:
+                n = hits.shape[0]
+                t, u, v = (torch.empty(n, dtype=torch.float32, device=hits.device) for _ in range(3))
+                prim = torch.empty(n, dtype=torch.int32, device=hits.device)
+                _check(lib().scion_split_hits(hits.data_ptr(), n, t.data_ptr(), u.data_ptr(), v.data_ptr(),
+                                              prim.data_ptr(), _stream_ptr(None)), "scion_split_hits")
+            else:  # rays in pinned host memory: the trace writes the hits there
+                torch.cuda.current_stream().synchronize()
+                f = hits.view(torch.float32)
+                t, u, v, prim = f[:, 0].clone(), f[:, 1].clone(), f[:, 2].clone(), hits[:, 3].clone()
             ctx.mark_non_differentiable(prim)
             return t, u, v, prim
 

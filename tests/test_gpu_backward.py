@@ -162,6 +162,19 @@ def test_autograd_missing_and_strided_gradients(setup):
     assert torch.equal(two, 2 * one)
 
 
+def test_autograd_forward_on_pinned_rays(setup):
+    """Rays in pinned host memory give the outputs of rays on the device, there; gradients want device memory."""
+    scion, sc, rays, tris, g, hits, gv64, gr64 = setup
+    bvh = scion.scion_build(sc.verts, scion.layout(width=4, box_layout="soa"), sc.indices)
+    verts = torch.from_numpy(sc.verts).cuda().requires_grad_(True)
+    want = scion.trace_fn().apply(verts, torch.from_numpy(rays).cuda(), bvh)
+    got = scion.trace_fn().apply(verts, torch.from_numpy(rays).pin_memory(), bvh)
+    for x, y in zip(got, want):
+        assert not x.is_cuda and torch.equal(x.detach(), y.detach().cpu())
+    with pytest.raises(scion.ScionError):
+        got[0].sum().backward()
+
+
 def test_backward_and_counters_take_device_buffers_only(setup):
     """Gradients and visit counters are added with device atomics: host
     buffers are rejected before any launch."""
