@@ -94,15 +94,33 @@ def test_config1_every_layout_bit_exact(sc_mod, config1, kw):
 @pytest.mark.parametrize("n", [1, 2, 31, 33, 1000, 2431, 2433, 4865, 9729, 16383])
 def test_small_launches(sc_mod, config1, n):
     """Launches below and around the sizes at which a warp takes fewer than 32
-    rays at a time: every ray is traced once, in every fetch mode and for tiles
-    cut short by the block size."""
+    rays at a time: every ray is traced once, by a warp each (the default
+    shape) and by lanes (a block size given), in every fetch mode and for tiles
+    cut short by the block size or the image."""
     sc, rays, exp, occ = config1
     for kw in (dict(), dict(width=4, box_layout="soa"), dict(width=8, box_prec="u8")):
         bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
-        for p in (None, dict(rays_per_fetch=4), dict(raster_width=37), dict(threads_per_block=32, ctas_per_sm=1)):
+        lanes = dict(threads_per_block=128)
+        for p in (None, dict(rays_per_fetch=4), dict(raster_width=37), dict(threads_per_block=32, ctas_per_sm=1), lanes,
+                  dict(lanes, rays_per_fetch=4), dict(lanes, raster_width=37), dict(lanes, raster_width=1001)):
             for _ in range(2):  # the counters are ready for the next launch
                 assert_same_hits(gpu_closest(sc_mod, bvh, rays[:n], params=p), exp[:n], f"{kw} {p}")
             assert np.array_equal(gpu_any(sc_mod, bvh, rays[:n], params=p), occ[:n]), f"{kw} {p}"
+        assert sc_mod.scion_get_status(bvh) == 0
+
+
+@pytest.mark.parametrize("n", [19_457, 29_185, 38_911, 38_913, 77_823, 77_825])
+def test_launches_of_small_blocks(sc_mod, config1, n):
+    """Launches above those of a ray per warp and below 77,824 rays (152 SMs): lanes take blocks of 8 or 16 rays, which
+    cut tiles short; above, blocks of 32."""
+    sc, rays, exp, occ = config1
+    many, exp, occ = np.tile(rays, (5, 1))[:n], np.tile(exp, 5)[:n], np.tile(occ, 5)[:n]
+    for kw in (dict(), dict(width=4, box_layout="soa"), dict(width=8, box_prec="u8")):
+        bvh = sc_mod.scion_build(sc.verts, sc_mod.layout(**kw), sc.indices)
+        for p in (None, dict(rays_per_fetch=4), dict(raster_width=37), dict(raster_width=301)):
+            for _ in range(2):  # the counters are ready for the next launch
+                assert_same_hits(gpu_closest(sc_mod, bvh, many, params=p), exp, f"{kw} {p}")
+            assert np.array_equal(gpu_any(sc_mod, bvh, many, params=p), occ), f"{kw} {p}"
         assert sc_mod.scion_get_status(bvh) == 0
 
 
