@@ -1269,7 +1269,6 @@ scion_status scion_batch_create(const scion_bvh *bvhs, const scion_ray *const *d
     a.smem_stack = bt->smem_stack;
     a.refill_min = p.rays_per_fetch ? p.rays_per_fetch : 32u;
     a.status = b->d_scratch + 3;
-    sc.begin = total;
     sc.family = (uint32_t)fam;
     of.resize(std::max<size_t>(of.size(), (size_t)fam + 1), nullptr);
     if (!of[fam]) of[fam] = b;

@@ -28,7 +28,6 @@
 #include "gpack.h"
 
 #include <algorithm>
-#include <chrono>
 #include <vector>
 
 #include "codec_fast.h"
@@ -696,7 +695,6 @@ scion_status gpu_pack(const LbvhTree &t, const float *d_verts, uint64_t n_verts,
                       uint64_t n_tris, const scion_layout_desc &d, bool own_box, cudaStream_t s,
                       DevicePacked *out, std::string *err) {
   *out = DevicePacked{};
-  const auto t0 = std::chrono::steady_clock::now();
   const uint32_t nv = t.nv, W = d.width;
   const bool dfs = d.order != ORDER_BFS, group = dfs && d.child_ref == REF_INDIRECT, pre = dfs && !group;
   const bool direct = d.prim_ref == REF_DIRECT;
@@ -952,7 +950,6 @@ scion_status gpu_pack(const LbvhTree &t, const float *d_verts, uint64_t n_verts,
   out->verts4 = verts4;
   out->idx = idx;
   out->block = block.release();  // the caller's now
-  out->pack_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
   return SCION_OK;
 }
 

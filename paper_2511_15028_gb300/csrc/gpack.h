@@ -32,7 +32,6 @@ struct DevicePacked {
            idx_bytes = 0;
   uint32_t n_nodes = 0, node_stride = 0, n_leaf_entries = 0, root_ref = kEmptyRef, depth = 0, stack_need = 0;
   float frame[9] = {};
-  double pack_ms = 0.0;  // wall time of the packing
 };
 
 // Enqueues the check that every index of the device array d_indices

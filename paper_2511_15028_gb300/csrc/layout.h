@@ -133,7 +133,6 @@ constexpr uint32_t kQ16Max = 65535u, kEq10Max = 1023u;
 SCION_HD uint32_t qbin_leaf(uint32_t first, uint32_t count) { return (first << 4) | count; }
 SCION_HD uint32_t qbin_interior(uint32_t field, uint32_t axis) { return (field << 6) | (axis << 4); }
 SCION_HD uint32_t qbin_count(uint32_t w) { return w & 15u; }
-SCION_HD uint32_t qbin_axis(uint32_t w) { return (w >> 4) & 3u; }
 SCION_HD uint32_t qbin_field(uint32_t w) { return w >> 6; }
 SCION_HD uint32_t qbin_first(uint32_t w) { return w >> 4; }
 SCION_HD uint32_t eq10_pack(uint32_t x, uint32_t y, uint32_t z) { return (x << 20) | (y << 10) | z; }
@@ -151,8 +150,5 @@ SCION_HD bool prec_has_frame(uint32_t prec) { return prec_is_world_grid(prec) ||
 constexpr uint32_t kSlabNodeBytes = 16;
 
 constexpr uint32_t kPrimDirectBytes = 48;
-
-// scratch words per BVH (device): work counter, exit counter, status, spare
-constexpr uint32_t kScratchWords = 4;
 
 }  // namespace scion

@@ -338,7 +338,6 @@ struct StackT {
   float *locf;
   static constexpr int kRegs = R;
   static constexpr bool kTF = TF, kKeyed = KEYED;
-  static constexpr uint32_t kEntryBytes = KEYED ? 8 : 4;  // without the exit distance
 
   __device__ __forceinline__ void attach(StackTail<TF, KEYED> &t) {
     loc = t.loc;
@@ -872,8 +871,6 @@ __device__ __forceinline__ float u16lo_b(uint32_t w) {  // 2^23 + low half
 __device__ __forceinline__ float u16hi_b(uint32_t w) {  // 2^23 + high half
   return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7432u));
 }
-__device__ __forceinline__ float u16lo_f(uint32_t w) { return u16lo_b(w) - 8388608.0f; }
-__device__ __forceinline__ float u16hi_f(uint32_t w) { return u16hi_b(w) - 8388608.0f; }
 __device__ __forceinline__ float eq10_f(uint32_t w, int axis) {
   return __uint_as_float(0x4B000000u | eq10_code(w, axis)) - 8388608.0f;
 }
