@@ -309,8 +309,8 @@ scion_status scion_trace_any(scion_bvh bvh, const scion_ray *d_rays, uint64_t n,
  * Missed rays (prim = SCION_PRIM_MISS) and errored rays contribute nothing.
  * The per-ray 3x3 solve is done in single precision and refined once with a
  * residual of about twice that; where that is singular or out of range, in
- * double precision. Every buffer must be device memory (the gradients are scattered with device atomics), else
- * SCION_ERR_INVALID_ARG. */
+ * double precision. Every buffer must be device memory (the gradients are
+ * scattered with device atomics), else SCION_ERR_INVALID_ARG. */
 scion_status scion_trace_backward(scion_bvh bvh, const scion_ray *d_rays, const scion_hit *d_hits,
                                   const float *d_grad_tuv, uint64_t n, float *d_grad_verts,
                                   scion_ray *d_grad_rays, scion_stream stream);

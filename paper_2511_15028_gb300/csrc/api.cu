@@ -184,9 +184,10 @@ void bvh_args(const scion_bvh b, TraceArgs &a) {
 // default limit of 48 KB also covers the kernels' static shared memory).
 constexpr size_t kSmemOptIn = 32 * 1024;
 
-// Closest point queries are refilled once this many lanes of a warp are idle
-// (1 M random points around 1.4 M triangles, bvh4 f32: 3.33 ms at 4 lanes, 3.37
-// at 1, 3.34 at 8; whole batches of 32 took 5.90 when a step was one visit).
+// Closest point queries are refilled once this many lanes of a warp are idle, unless
+// the warp waits for its block (refill_loop). 1 M random points around 1.4 M
+// triangles, bvh4 f32: 3.73 ms at 4 lanes, 3.77 at 8, 3.85 at 12, 4.47 at 24, and
+// 5.40 in whole batches of 32.
 constexpr uint32_t kCpRefill = 4;
 
 // Query kinds of launch_trace.

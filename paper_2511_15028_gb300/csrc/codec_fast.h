@@ -8,8 +8,8 @@
 // unevaluated sum of two floats (error-free transformations: TwoSum by Knuth,
 // products by one fma), about 2^-46 accurate. The direction of the rounding
 // is then certain unless the value lies within that error of a float or an
-// integer; those few cases (and ranges where the pairs could underflow) are
-// computed as codec.h does. Compiled for host and device.
+// integer; those few cases, and ranges where the pairs could underflow or
+// overflow, are computed as codec.h does. Compiled for host and device.
 #pragma once
 
 #include "codec.h"

@@ -338,10 +338,10 @@ __device__ __forceinline__ void cp_node_bin(const TraceArgs &a, CpLane &L, S &st
   L.field = right ? rf : lf;
 }
 
-// Closest point queries as a query of refill_loop. Neighbouring points share
-// little of their paths unless they are sorted: in batches of 32 a warp had 4
-// of its lanes active on random points. Idle lanes are refilled and a leaf runs
-// triangle by triangle; 1 M random points around 1.4 M triangles, before and
+// Closest point queries as a query of refill_loop. Random neighbours share little of
+// their paths: in batches of 32 a warp had 4 of its lanes active. Idle lanes are
+// refilled, except while a warp's points go together, and a leaf runs triangle by
+// triangle; 1 M random points around 1.4 M triangles, before and
 // after: bvh4 f32 5.90 -> 3.65 ms, bvh8 f16 7.47 -> 5.48, bvh2 q16 6.89 -> 4.47; with
 // nodes and triangles in one step (node_then_leaf) 3.33, 4.53 and 3.90.
 template <bool OWN, int W, int PREC, int SOA, int CREF, bool STATS, class S>

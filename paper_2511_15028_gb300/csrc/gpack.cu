@@ -698,7 +698,7 @@ scion_status gpu_pack(const LbvhTree &t, const float *d_verts, uint64_t n_verts,
   const uint32_t nv = t.nv, W = d.width;
   const bool dfs = d.order != ORDER_BFS, group = dfs && d.child_ref == REF_INDIRECT, pre = dfs && !group;
   const bool direct = d.prim_ref == REF_DIRECT;
-  // most nodes the tree can have, and the levels issued before the first look
+  // most nodes the tree can have
   const uint64_t cap = nv == 0 ? 0 : (own_box ? 2ull * nv - 1 : std::max<uint64_t>(1, nv - 1));
   cudaError_t e;
 #define SCION_GP(call)                                \

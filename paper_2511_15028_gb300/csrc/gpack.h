@@ -3,7 +3,8 @@
 // GPU builder leaves in device memory, so a GPU build never moves the tree
 // through host memory. The packed bytes are those of the host packer
 // (builder.cpp) for the same logical tree: the same greedy collapse to width
-// W, the same node orders and the same host/device codecs (codec.h).
+// W, the same node orders, and encoders that give the bytes of the host codecs
+// (codec_fast.h).
 #pragma once
 
 #include <cuda_runtime.h>

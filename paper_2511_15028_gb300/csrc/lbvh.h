@@ -29,7 +29,8 @@ namespace scion {
 // library's own that keeps up to kScratchKept bytes per device between calls
 // (the driver gives the rest back, and hands the pool's memory to any thread
 // or stream in order); commit() allocates a result with cudaMalloc. Freed with
-// the object unless released.
+// the object unless released. Every array starts at a multiple of 256 bytes: the
+// kernels' 32-byte node loads rely on it.
 constexpr uint64_t kScratchKept = 512ull << 20;
 class Arena {
  public:

@@ -1,6 +1,6 @@
 // Refit of a packed BVH to new vertex positions (same triangles, same tree):
 // boxes are recomputed bottom-up on the GPU and re-encoded in place in the
-// BVH's own layout with the codecs the host packer uses (codec.h).
+// BVH's own layout, to the bytes of the host packer's codecs (codec_fast.h).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -271,8 +271,8 @@ __device__ __forceinline__ void ldg8(const uint4 *p, uint4 &lo, uint4 &hi) {
       : "l"(p));
 }
 // A node of NQ 16-byte words at a 32-byte aligned address (node strides are
-// multiples of 32 bytes and node buffers are separately allocated): 256-bit
-// loads, and a 128-bit load for an odd last word.
+// multiples of 32 bytes, and node buffers start at a multiple of 256: cudaMalloc's,
+// or Arena's in lbvh.h): 256-bit loads, and a 128-bit load for an odd last word.
 template <int NQ>
 __device__ __forceinline__ void load_node(const uint4 *np, uint4 (&q)[NQ]) {
 #pragma unroll
@@ -1200,8 +1200,9 @@ __device__ __forceinline__ void batch_loop(const TraceArgs &a, Q &q) {
 // are mid-ray. Every lane steps kFreeSteps times between two checks: the vote
 // brings the whole warp together, and measured (750,000 shadow rays in 1.4 M
 // triangles, bvh4 f32, 4 idle lanes) 1, 2 and 4 steps take 470, 465 and 448 us;
-// 8.4 M random rays in 8.4 M triangles (bvh4 u8) 7.36, 7.43 and 7.34 ms. A finished lane keeps its result until the refill, so results leave
-// and rays enter with many lanes at a time.
+// 8.4 M random rays in 8.4 M triangles (bvh4 u8) 7.36, 7.43 and 7.34 ms. A finished
+// lane keeps its result until the refill, so results leave and rays enter with many
+// lanes at a time.
 constexpr int kFreeSteps = 4;
 // WAIT (closest points): neighbours that take the same way share its nodes while
 // they stay together, and lanes refilled one by one part them, so the warp waits for
