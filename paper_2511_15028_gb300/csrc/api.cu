@@ -193,16 +193,18 @@ constexpr uint32_t kCpRefill = 4;
 // Query kinds of launch_trace.
 constexpr int kQueryClosest = 0, kQueryAny = 1, kQueryPoint = 2;
 
-// Shared-memory stack entries per thread. The traversal kernels of the
-// own-box bvh2 nodes (all but the shared-slab one) and of 2/4-wide nodes keep
-// the shared part of the stack as a ring indexed with a mask (StackFor in
-// trace.cuh), so for them the count is rounded down to a power of two.
-uint32_t stack_entries(scion_bvh b, uint32_t requested) {
+// Shared-memory stack entries per thread. The kernels of the own-box bvh2 nodes (all
+// but the shared-slab one) and of 2/4-wide nodes keep the shared part of the stack as
+// a ring indexed with a mask (StackFor in trace.cuh), so for them the count is
+// rounded down to a power of two, or up where trees that need up to `need` entries
+// would otherwise have less room than requested (closest points and batches; plain
+// traces, need = 0, are always rounded down).
+uint32_t stack_entries(scion_bvh b, uint32_t requested, uint32_t need) {
   const bool ring = b->own_box ? b->desc.box_prec != PREC_SLAB : b->desc.width <= 4;
   if (!ring) return requested;
   uint32_t p = 1;
   while (p * 2 <= requested) p *= 2;
-  return p;
+  return p < requested && p + kLocalStack < need ? 2 * p : p;
 }
 
 // Warp-batch work of a launch over a.n rays: consecutive 32-ray batches, or
@@ -603,7 +605,7 @@ scion_status prepare_trace(scion_bvh b, const scion_ray *rays, uint64_t n, void 
     g_last_error = "smem_stack exceeds 64 entries";
     return SCION_ERR_INVALID_ARG;
   }
-  smem_entries = stack_entries(b, smem_entries);
+  smem_entries = stack_entries(b, smem_entries, query == kQueryPoint ? b->stack_need : 0u);
   if (p.ordered_children > 3) {
     g_last_error = "ordered_children must be 0..3";
     return SCION_ERR_INVALID_ARG;
@@ -676,7 +678,8 @@ scion_status launch_trace(scion_bvh b, const scion_ray *rays, uint64_t n, void *
   TraceKernel k = L.k;
   if (stats) {
     L.coop = false;
-    L.a.smem_stack = stack_entries(b, params && params->smem_stack ? params->smem_stack : 16);
+    L.a.smem_stack = stack_entries(b, params && params->smem_stack ? params->smem_stack : 16,
+                                   query == kQueryPoint ? b->stack_need : 0u);
     L.smem = (size_t)L.tpb * L.a.smem_stack * stack_entry_bytes(b, query);
     k = pick_kernel(b, query, 1, 0);
     if (!k) return SCION_ERR_UNSUPPORTED_LAYOUT;
@@ -1268,6 +1271,7 @@ scion_status scion_batch_create(const scion_bvh *bvhs, const scion_ray *const *d
     a.max_steps = p.max_steps ? p.max_steps : 2u * (b->n_nodes + b->n_leaf_entries) + 64u;
     a.ordered = order_mode(p.ordered_children);
     a.smem_stack = bt->smem_stack;
+    a.stack_need = b->stack_need;
     a.refill_min = p.rays_per_fetch ? p.rays_per_fetch : 32u;
     a.status = b->d_scratch + 3;
     sc.family = (uint32_t)fam;
@@ -1305,8 +1309,11 @@ scion_status scion_batch_create(const scion_bvh *bvhs, const scion_ray *const *d
   for (size_t i = 0; i < bt->parts.size() && e == cudaSuccess; ++i) {
     scion_batch_s::Part &part = bt->parts[i];
     const bool one_family = split || families == 1;
-    // a ring as in the plain kernels
-    if (one_family) part.smem_stack = stack_entries(of[table[part.first].family], part.smem_stack);
+    if (one_family) {  // a ring as in the plain kernels
+      uint32_t need = 0;
+      for (uint32_t k = part.first; k < part.first + part.n; ++k) need = std::max(need, table[k].a.stack_need);
+      part.smem_stack = stack_entries(of[table[part.first].family], part.smem_stack, need);
+    }
     const size_t smem = (size_t)bt->threads * part.smem_stack * sizeof(uint2);
     int nb = 0;
     const scion_status so = ensure_smem_optin((const void *)part.kernel, smem, dev);

@@ -291,6 +291,42 @@ def test_one_ray_per_warp_with_a_full_stack(sc_mod, oracle_mod, kw):
     assert sc_mod.scion_get_status(bvh) == 0
 
 
+def chain_scene(n):
+    """Triangles at x = 4^k (k = -n/2 .. n/2 - 1) whose two-bin SAH tree peels one triangle per level (depth n); a
+    ray along +x through all of them pushes one far child per level, and so does the point where it starts."""
+    c = 4.0 ** (np.arange(n) - n // 2)
+    s = c / 2
+    v = np.zeros((n, 3, 3))
+    v[:, 0] = np.stack([c, -s, -s], -1)
+    v[:, 1] = np.stack([c, s, -s], -1)
+    v[:, 2] = np.stack([c, 0 * s, 2 * s], -1)
+    return v.astype(np.float32).reshape(-1, 3)
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(box_prec="f32", child_ref="indirect"), dict(width=2, box_prec="f16")], ids=str)
+def test_stack_entries_that_are_no_power_of_two(sc_mod, oracle_mod, kw):
+    """20 entries in shared memory and 48 behind them hold the 66 that a tree of depth 67 needs, for closest points
+    and in batches, where the kernels round to a power of two."""
+    v = chain_scene(67)
+    desc = sc_mod.layout(leaf_max=1, sah_bins=2, **kw)
+    assert sc_mod.scion_debug_build_host(v, desc).info["depth"] >= 66
+    b = sc_mod.scion_build(v, desc)
+    tris = v.reshape(-1, 9)
+    ray = np.array([[-1.0, 0.0, 0.0, 0.0, 1, 0, 0, np.inf]] * 40, np.float32)
+    pts = np.array([[-1.0, 0.0, 0.0, np.inf], [1e-9, 0, 0, np.inf]] * 20, np.float32)
+    for p in (dict(smem_stack=20), dict(smem_stack=40, threads_per_block=128)):
+        got = sc_mod.split_hits(sc_mod.scion_query_closest_point(b, torch.from_numpy(pts).cuda(), params=p))
+        assert got.tobytes() == oracle_mod.cpq_brute(tris, pts).tobytes(), p
+        out = sc_mod.scion_trace_stats(b, torch.from_numpy(pts).cuda(), 2, params=p)[0]
+        assert sc_mod.split_hits(out).tobytes() == got.tobytes(), p
+        if kw:
+            continue  # no batched node family: a plain launch, whose rounding down is as documented
+        batch = sc_mod.Batch([b] * 2, [torch.from_numpy(ray).cuda()] * 2, params=[p] * 2)
+        for h in batch.launch():
+            assert_same_hits(sc_mod.split_hits(h), oracle_mod.closest_brute(tris, ray), str(p))
+    assert sc_mod.scion_get_status(b) == 0
+
+
 def test_device_errors_are_reported_not_faulted(sc_mod):
     """A tiny step limit and a stack deeper than the traversal stack end the
     affected rays with prim = ERROR and a status code; nothing faults."""
@@ -307,17 +343,9 @@ def test_device_errors_are_reported_not_faulted(sc_mod):
         gpu_closest(sc_mod, bvh, rays, params=dict(rays_per_fetch=33))
     with pytest.raises(sc_mod.ScionError):  # tiles need warp batches
         gpu_closest(sc_mod, bvh, rays, params=dict(raster_width=128, rays_per_fetch=8))
-    # a chain: triangles at x = 4^k (k = -50..49) whose two-bin SAH tree peels
-    # one triangle per level (depth 100); a ray along +x through all of them
-    # pushes one far child per level, more than the 64-entry stack holds
+    # a chain whose depth is more than the 64-entry stack holds
     n = 100
-    c = 4.0 ** (np.arange(n) - n // 2)
-    s = c / 2
-    v = np.zeros((n, 3, 3))
-    v[:, 0] = np.stack([c, -s, -s], -1)
-    v[:, 1] = np.stack([c, s, -s], -1)
-    v[:, 2] = np.stack([c, 0 * s, 2 * s], -1)
-    v = v.astype(np.float32).reshape(-1, 3)
+    v = chain_scene(n)
     desc = sc_mod.layout(leaf_max=1, sah_bins=2)
     assert sc_mod.scion_debug_build_host(v, desc).info["depth"] == n
     b = sc_mod.scion_build(v, desc)
